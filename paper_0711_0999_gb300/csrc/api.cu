@@ -13,8 +13,6 @@ namespace nedmft {
 
 namespace {
 
-constexpr int kNbSimt = 32;  // Gauss-Jordan block of the CUDA-core path
-
 int padded(int n) { return ((n + 127) / 128) * 128; }
 
 bool valid_contour(const nedmft_contour* c) {
@@ -53,7 +51,7 @@ int default_batch(const nedmft_contour& c, int nq, Path path, int width) {
   int cap = 152;
   switch (path) {
     case Path::Small64: per = sizeof(double2) * c.n_c * c.n_c; cap = 2048; break;
-    case Path::Blocked64: per = sizeof(double2) * np * np; cap = 152; break;
+    case Path::Blocked64: per = sizeof(double2) * np * np + gj64_scratch_bytes((int)np, 1); cap = 152; break;
     case Path::MixedUmma: per = umma_batch_bytes_per_matrix((int)np, width); cap = umma_default_batch((int)np); break;
   }
   int b = (int)(budget / (per ? per : 1));
@@ -64,7 +62,7 @@ int default_batch(const nedmft_contour& c, int nq, Path path, int width) {
 }
 
 struct LatticeLayout {
-  size_t S, gscratch, jacc, batch, pbuf, rbuf, cbuf, extra, total;
+  size_t S, gscratch, jacc, batch, extra, total;
   int np, mb, width;
   Path path;
 };
@@ -90,16 +88,14 @@ LatticeLayout lattice_layout(const nedmft_contour& c, int nq, nedmft_precision p
       break;
     case Path::Blocked64:
       L.batch = align256(sizeof(double2) * np * np * mb);
-      L.pbuf = align256(sizeof(double2) * kNbSimt * kNbSimt * mb);
-      L.rbuf = align256(sizeof(double2) * kNbSimt * np * mb);
-      L.cbuf = align256(sizeof(double2) * np * kNbSimt * mb);
+      L.extra = align256(gj64_scratch_bytes((int)np, (int)mb));
       break;
     case Path::MixedUmma:
       L.batch = align256(umma_batch_bytes((int)np, (int)mb, width));
       L.extra = align256(umma_shared_bytes((int)np, nq));
       break;
   }
-  L.total = L.S + L.gscratch + L.jacc + L.batch + L.pbuf + L.rbuf + L.cbuf + L.extra + 256;
+  L.total = L.S + L.gscratch + L.jacc + L.batch + L.extra + 256;
   return L;
 }
 
@@ -132,9 +128,6 @@ int lattice_run_batch(const nedmft_contour& c, const nedmft_model& m, const doub
   double2* gs = reinterpret_cast<double2*>(p); p += L.gscratch;
   double2* jacc = reinterpret_cast<double2*>(p); p += L.jacc;
   char* batch = p; p += L.batch;
-  char* pbuf = p; p += L.pbuf;
-  char* rbuf = p; p += L.rbuf;
-  char* cbuf = p; p += L.cbuf;
   char* extra = p;
   if (!gloc) gloc = gs;
   double2* ja = (j || ji) ? jacc : nullptr;
@@ -158,9 +151,7 @@ int lattice_run_batch(const nedmft_contour& c, const nedmft_model& m, const doub
       case Path::Blocked64: {
         double2* A = reinterpret_cast<double2*>(batch);
         if ((rc = launch_gen_a<double>(cd, md, eps, ebar, q0, nb, S, A, np, st))) return rc;
-        if ((rc = gj_blocked_simt<double>(A, cd.n, np, nb, reinterpret_cast<double2*>(pbuf), reinterpret_cast<double2*>(rbuf),
-                                          reinterpret_cast<double2*>(cbuf), status, st)))
-          return rc;
+        if ((rc = gj64_invert(A, cd.n, np, nb, extra, status, st))) return rc;
         if ((rc = launch_reduce<double>(cd, md, eps, ebar, wq, q0, nb, A, nullptr, np, true, first, gloc, ja, st)))
           return rc;
         break;

@@ -18,9 +18,11 @@ int small_path_max_n();
 int launch_gj_small_fp64(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, int q0,
                          int nb, const double2* S, double2* out, int* status, cudaStream_t st);
 
-template <class T>
-int gj_blocked_simt(cplx_t<T>* A, int n, int np, int nb_batch, cplx_t<T>* Pbuf, cplx_t<T>* Rbuf, cplx_t<T>* Cbuf,
-                    int* status, cudaStream_t st);
+// Batched FP64 inverses on the tensor cores (gj64_umma.cu): nb matrices of np x np (np a multiple of 128, the
+// identity outside n x n), in place, scratch of gj64_scratch_bytes.
+size_t gj64_scratch_bytes(int np, int nb);
+int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, cudaStream_t st);
+int gj64_set_wait_ns(uint64_t ns, cudaStream_t st);  // its bounded waits' limit on the current device
 
 template <class T>
 int launch_reduce(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, const double* wq,

@@ -2316,6 +2316,7 @@ int umma_wait_selftest(int* status, cudaStream_t st) {
 int umma_set_wait_ns(uint64_t ns, cudaStream_t st) {
   NED_CUDA(cudaMemcpyToSymbolAsync(umma::g_wait_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, st));
   NED_CUDA(cudaStreamSynchronize(st));
+  if (int rc = gj64_set_wait_ns(ns, st)) return rc;
   return oz64_set_wait_ns(ns, st);
 }
 
