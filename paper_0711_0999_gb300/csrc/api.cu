@@ -144,15 +144,15 @@ int lattice_run_batch(const nedmft_contour& c, const nedmft_model& m, const doub
       case Path::Small64: {
         double2* out = reinterpret_cast<double2*>(batch);
         if ((rc = launch_gj_small_fp64(cd, md, eps, ebar, q0, nb, S, out, status, st))) return rc;
-        if ((rc = launch_reduce<double>(cd, md, eps, ebar, wq, q0, nb, out, nullptr, cd.n, false, first, gloc, ja, st)))
+        if ((rc = launch_reduce(cd, md, eps, ebar, wq, q0, nb, out, cd.n, false, first, gloc, ja, st)))
           return rc;
         break;
       }
       case Path::Blocked64: {
         double2* A = reinterpret_cast<double2*>(batch);
-        if ((rc = launch_gen_a<double>(cd, md, eps, ebar, q0, nb, S, A, np, st))) return rc;
+        if ((rc = launch_gen_a(cd, md, eps, ebar, q0, nb, S, A, np, st))) return rc;
         if ((rc = gj64_invert(A, cd.n, np, nb, extra, status, st))) return rc;
-        if ((rc = launch_reduce<double>(cd, md, eps, ebar, wq, q0, nb, A, nullptr, np, true, first, gloc, ja, st)))
+        if ((rc = launch_reduce(cd, md, eps, ebar, wq, q0, nb, A, np, true, first, gloc, ja, st)))
           return rc;
         break;
       }

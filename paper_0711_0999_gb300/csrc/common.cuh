@@ -192,14 +192,6 @@ __device__ __forceinline__ bool shifted_point(const ModelDev& m, double eps) { r
 // Column of X' = (P A)^-1 holding column j of A^-1.
 __device__ __forceinline__ int unshift_col(int j, int n, bool sh) { return sh ? (j == 0 ? n - 1 : j - 1) : j; }
 
-// ebar_{k + theta(t) E t} at upper-branch time t (Eq. current_def with v -> -ebar).
-__device__ __forceinline__ double ebar_at(double t, double eps, double ebar, double E) {
-  if (t <= 0.0) return ebar;
-  double sn, cs;
-  sincos(E * t, &sn, &cs);
-  return ebar * cs + eps * sn;
-}
-
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 

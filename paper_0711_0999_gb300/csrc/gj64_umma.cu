@@ -38,6 +38,20 @@ constexpr int kARow = kTileElems;            // bf16 elements of one digit of a 
 constexpr int kATile = kS * kTileElems;      // ... of all digits
 constexpr int kBDig = 2 * kTn * kK;          // bf16 elements of one digit of a 16-column tile of R
 constexpr int kBTile = kS * kBDig;
+constexpr int kPTile = kS * 64 * kK;         // ... of the 64 real rows of P
+
+__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
+  const uint64_t t0 = global_ns();
+  while (!mbar_test(bar, parity) && global_ns() - t0 < kDrainNs) {
+  }
+}
+// eight TMEM columns of this warp's 32 lanes (wait with tmem_wait_ld)
+__device__ __forceinline__ void tmem_ld8(uint32_t addr, float (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "r"(addr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ------------------------------------------------------------------ digits
 
@@ -84,6 +98,20 @@ __device__ __forceinline__ void put_digits(const long long (&y)[8], Put&& put) {
                     digit_pair<S>(y[6], y[7])));
   if constexpr (S + 1 < kS) put_digits<S + 1>(y, put);
 }
+template <int S = 0, class Put>
+__device__ __forceinline__ void put_digits2(const long long (&y)[16], Put&& put) {
+  put(S, make_uint4(digit_pair<S>(y[0], y[1]), digit_pair<S>(y[2], y[3]), digit_pair<S>(y[4], y[5]),
+                    digit_pair<S>(y[6], y[7])),
+      make_uint4(digit_pair<S>(y[8], y[9]), digit_pair<S>(y[10], y[11]), digit_pair<S>(y[12], y[13]),
+                 digit_pair<S>(y[14], y[15])));
+  if constexpr (S + 1 < kS) put_digits2<S + 1>(y, put);
+}
+// 32 bytes (one sector) in one store; p 32-byte aligned
+__device__ __forceinline__ void st32(void* p, uint4 a, uint4 b) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+               "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+               : "memory");
+}
 __device__ __forceinline__ uint4 neg_bf16(uint4 v) {
   return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
 }
@@ -94,87 +122,163 @@ __device__ __forceinline__ int core_off(int row, int k) { return ((row >> 3) * 8
 
 // 2^(e-53) sum_o c_o 2^(8(5-o)) / 2 as a double, rounded once; c_o, o = 0 .. 6,
 // are integers with |c_o| <= (o + 1) 2^20.  ebase = 1023 + e - 53.
-// Float to int by the 1.5 2^23 trick (below 2^22; conversion instructions run
-// at an eighth of the rate), orders 4 .. 6 with the half of order 4 split off
-// first; the sum as a 64-bit integer in units of 2; its leading bit found by
-// the one int-to-float conversion, then shifted, rounded and assembled on the
-// integer units.
+// Float to int by adding 1.5 2^23 (below 2^22; conversion instructions run at
+// an eighth of the rate), orders 4 .. 6 with the half of order 4 split off
+// first.  Pairs of orders share a word, offset so that it stays positive, and
+// three wide multiply-adds make the sum T, 64 bits, in units of 2.  Its leading
+// bit comes from a float rounded towards zero; then it is shifted, rounded and
+// assembled on the integer units: about 40 instructions, none in FP64.  Written
+// as single instructions, without a branch: the same in C++ with 64-bit shifts
+// and conditionals took twice as many.
 __device__ __forceinline__ double orders_to_double(float c0, float c1, float c2, float c3, float c4, float c5,
                                                    float c6, int ebase) {
   constexpr float kM = 12582912.f;
-  constexpr uint32_t kOff = 0x4B400000u * 257u;
+  constexpr unsigned long long kOff = 0x8B400000ull;  // 0x4B400000 * 257 mod 2^32: the offset of a pair's word
+  constexpr unsigned long long kLess = 0ull - kOff * ((1ull << 31) + (1ull << 15) + 1ull);
   const uint32_t b0 = __float_as_uint(c0 + kM), b1 = __float_as_uint(c1 + kM);
   const uint32_t b2 = __float_as_uint(c2 + kM), b3 = __float_as_uint(c3 + kM);
   const float t4 = fmaf(c4, 0.5f, kM);
   const float rem = fmaf(c4, 0.5f, kM - t4);
   const float g = fmaf(rem, 512.f, fmaf(c6, 0.00390625f, c5));
   const uint32_t b4 = __float_as_uint(t4), b5 = __float_as_uint(fmaf(g, 0.5f, kM));
-  const int u0 = (int)(b0 * 256u + b1 - kOff);
-  const int u1 = (int)(b2 * 256u + b3 - kOff);
-  const int u2 = (int)(b4 * 256u + b5 - kOff);
-  const long long T = ((long long)u0 << 31) + (long long)u1 * 32768ll + (long long)u2;
-  const unsigned long long a = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
-  uint32_t hi = (uint32_t)(a >> 32), lo = (uint32_t)a;
-  const bool low = hi == 0;
-  if (low) { hi = lo; lo = 0; }
-  const uint32_t f = __float_as_uint(__uint2float_rz(hi));  // exponent 127 + index of the leading bit
-  const int n = 158 - (int)(f >> 23);                       // shift that brings it to bit 31
-  const uint32_t mh = __funnelshift_l(lo, hi, n), ml = lo << (n & 31);
-  uint32_t ql = __funnelshift_r(ml, mh, 11), qh = mh >> 11;
-  const uint32_t rnd = (ml >> 10) & 1u;
-  ql += rnd;
-  qh += (rnd && ql == 0) ? 1u : 0u;
-  int ex = (int)(f >> 23) - 127 + (low ? 0 : 32) + ebase;  // biased exponent of the result
-  ex = min(ex, 2047);                                      // beyond FP64: infinite or NaN, caught at the next digit cut
-  const uint32_t rh = (qh + ((uint32_t)(ex - 1) << 20)) | (T < 0 ? 0x80000000u : 0u);
-  return hi == 0 ? 0.0 : __hiloint2double((int)rh, (int)ql);
+  const uint32_t u0 = b0 * 256u + b1, u1 = b2 * 256u + b3, u2 = b4 * 256u + b5;  // the pairs + kOff
+  uint32_t rh, ql;
+  asm("{\n\t"
+      ".reg .u64 t;\n\t.reg .u32 lo, hi, s, n, ld, e, qh;\n\t.reg .f32 fh, fl;\n\t.reg .pred z;\n\t"
+      "mad.wide.u32 t, %4, 1, %5;\n\t"
+      "mad.wide.u32 t, %3, 32768, t;\n\t"
+      "mad.wide.u32 t, %2, 0x80000000, t;\n\t"
+      "mov.b64 {lo, hi}, t;\n\t"
+      "shr.s32 s, hi, 31;\n\t"  // |T|
+      "xor.b32 lo, lo, s;\n\txor.b32 hi, hi, s;\n\t"
+      "sub.cc.u32 lo, lo, s;\n\tsubc.u32 hi, hi, s;\n\t"
+      "cvt.rz.f32.u32 fh, hi;\n\tcvt.rz.f32.u32 fl, lo;\n\t"
+      "fma.rz.f32 fh, fh, 0f4F800000, fl;\n\t"
+      "mov.b32 ld, fh;\n\tshr.u32 ld, ld, 23;\n\t"  // 127 + index of the leading bit, 0 for T = 0
+      "sub.u32 n, 189, ld;\n\t"
+      "mov.b64 t, {lo, hi};\n\tshl.b64 t, t, n;\n\tmov.b64 {lo, hi}, t;\n\t"  // leading bit to bit 62
+      "add.cc.u32 lo, lo, 0x200;\n\taddc.u32 hi, hi, 0;\n\t"                    // 53 bits, rounded to nearest
+      "shf.r.wrap.b32 %1, lo, hi, 10;\n\tshr.u32 qh, hi, 10;\n\t"
+      "add.s32 e, ld, %6;\n\tmin.s32 e, e, 2046;\n\t"  // beyond FP64: infinite or NaN, caught at the next digit cut
+      "mad.lo.u32 qh, e, 0x100000, qh;\n\t"
+      "and.b32 s, s, 0x80000000;\n\tor.b32 qh, qh, s;\n\t"
+      "setp.eq.u32 z, ld, 0;\n\tselp.u32 %0, 0, qh, z;\n\t"
+      "}"
+      : "=&r"(rh), "=&r"(ql)
+      : "r"(u0), "r"(u1), "r"(u2), "l"(kLess), "r"(ebase - 128));
+  return __hiloint2double((int)rh, (int)ql);
 }
 
 // ------------------------------------------------------------------ pivot block and C digits
 
+// 1 / z as cinv_guard, the real reciprocal by two Newton steps on the
+// hardware's approximation (20 bits, then 40, then all): a third of the FP64
+// instructions of a division on the pivot row's serial path.
+__device__ __forceinline__ bool recip(double2 z, double2& out) {
+  const double m = z.x * z.x + z.y * z.y;
+  if (!(m > 1e-24)) {  // |z| <= 1e-12 or NaN
+    out = make_double2(1e12, 0.0);
+    return false;
+  }
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(m));
+  r = fma(r, fma(-m, r, 1.0), r);
+  r = fma(r, fma(-m, r, 1.0), r);
+  out = make_double2(z.x * r, -z.y * r);
+  return true;
+}
+
 // CTAs 0 .. nb-1: P = inv(A_KK) of matrix b, 32 x 32 FP64, a warp per four
 // rows, lane = column.  Step k: the pivot row, divided by its pivot (its own
-// entry replaced by the pivot's inverse), goes to shared memory (two buffers,
-// one barrier per step); every other row subtracts its entry of column k times
-// it, that entry counted as zero before.  FP64 bound: 32 rows x 4 FMAs x 16
-// cycles per step.
+// entry replaced by the pivot's inverse), is in shared memory (two buffers, one
+// barrier per step); every other row subtracts its entry of column k times it,
+// that entry counted as zero before.  The warp of the next pivot row takes that
+// row first and publishes it, so the reciprocal is off the other warps' path.
+// FP64 bound: 32 rows x 4 FMAs x 16 cycles per step, 33 us.
 // CTAs nb ..: digits of 128 rows of C, two threads per row; this work hides
 // behind the pivot blocks' latency.
 __global__ void __launch_bounds__(256) gj64_pivot_kernel(const double2* __restrict__ A, int np, int mtiles, int k0,
                                                          int nb, double2* __restrict__ Pbuf,
+                                                         __nv_bfloat16* __restrict__ pimg, int* __restrict__ pexp,
                                                          __nv_bfloat16* __restrict__ cimg, int* __restrict__ cexp,
                                                          int* status) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   if ((int)blockIdx.x < nb) {
     __shared__ double2 rowb[2][32];
+    __shared__ double2 prow[kNB][kNB + 1];
     const int b = blockIdx.x;
     const double2* a = A + (size_t)b * np * np + (size_t)k0 * np + k0;
     double2 v[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = a[(size_t)(4 * warp + q) * np + lane];
+    // row (warp, kq) as step k's pivot row: divided by its pivot and published
+    auto publish = [&](double2& z, int k) {
+      const double2 d = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+      double2 pinv;
+      if (!recip(d, pinv) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
+      z = lane == k ? pinv : cmul(z, pinv);
+      rowb[k & 1][lane] = z;
+    };
+    if (warp == 0) publish(v[0], 0);
+    __syncthreads();
     for (int kw = 0; kw < 8; ++kw)
 #pragma unroll
       for (int kq = 0; kq < 4; ++kq) {
-        const int k = 4 * kw + kq, buf = k & 1;
-        if (warp == kw) {
-          const double2 d = make_double2(__shfl_sync(0xffffffffu, v[kq].x, k), __shfl_sync(0xffffffffu, v[kq].y, k));
-          double2 pinv;
-          if (!cinv_guard<double>(d, pinv, 1e-12) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
-          v[kq] = lane == k ? pinv : cmul(v[kq], pinv);
-          rowb[buf][lane] = v[kq];
+        const int k = 4 * kw + kq;
+        const double2 rb = rowb[k & 1][lane];
+        auto eliminate = [&](double2& z) {
+          const double2 c = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+          const double2 o = lane == k ? make_double2(0.0, 0.0) : z;
+          z = make_double2(fma(-c.x, rb.x, fma(c.y, rb.y, o.x)), fma(-c.x, rb.y, fma(-c.y, rb.x, o.y)));
+        };
+        constexpr int kNext[4] = {1, 2, 3, 0};  // the next pivot row's place in its warp
+        const int nq = kNext[kq];
+        const bool mine = k + 1 < 32 && warp == (kq == 3 ? kw + 1 : kw);
+        if (mine) {  // the next pivot row first: its reciprocal runs beside the other warps' rows
+          eliminate(v[nq]);
+          publish(v[nq], k + 1);
         }
-        __syncthreads();
-        const double2 rb = rowb[buf][lane];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (warp == kw && q == kq) continue;
-          const double2 c = make_double2(__shfl_sync(0xffffffffu, v[q].x, k), __shfl_sync(0xffffffffu, v[q].y, k));
-          const double2 o = lane == k ? make_double2(0.0, 0.0) : v[q];
-          v[q] = make_double2(fma(-c.x, rb.x, fma(c.y, rb.y, o.x)), fma(-c.x, rb.y, fma(-c.y, rb.x, o.y)));
-        }
+        for (int q = 0; q < 4; ++q)
+          if (!(warp == kw && q == kq) && !(mine && q == nq)) eliminate(v[q]);
+        __syncthreads();
       }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) Pbuf[(size_t)b * kNB * kNB + (4 * warp + q) * kNB + lane] = v[q];
+    for (int q = 0; q < 4; ++q) {
+      const int r = 4 * warp + q;
+      Pbuf[(size_t)b * kNB * kNB + r * kNB + lane] = v[q];
+      prow[r][lane] = v[q];
+    }
+    __syncthreads();
+    // digits of the 64 real rows of P, eight threads per row r, four entries
+    // each: row 2r = [Re P_r | -Im P_r], row 2r + 1 = [Im P_r | Re P_r]
+    const int r = t >> 3, c4 = 4 * (t & 7);
+    double2 p[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) p[c] = prow[r][c4 + c];
+    unsigned m = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) m = max(m, max(mag_hi(p[c].x), mag_hi(p[c].y)));
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int be = row_biased(m);
+    if ((t & 7) == 0) pexp[b * kNB + r] = be - 1022;
+    if (m >= 0x7ff00000u && status) atomicCAS(status, 0, DS_SINGULAR);
+    long long y[8];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      y[c] = digit_word(p[c].x, be);
+      y[4 + c] = digit_word(p[c].y, be);
+    }
+    const int o_re = core_off(2 * r, c4), o_im = core_off(2 * r, 32 + c4);  // row 2r + 1: 8 elements on
+    put_digits(y, [&](int s, uint4 w) {
+      __nv_bfloat16* d = pimg + (size_t)b * kPTile + s * 64 * kK;
+      const uint4 n = neg_bf16(w);
+      *reinterpret_cast<uint2*>(d + o_re) = make_uint2(w.x, w.y);
+      *reinterpret_cast<uint2*>(d + o_im) = make_uint2(n.z, n.w);
+      *reinterpret_cast<uint2*>(d + o_re + 8) = make_uint2(w.z, w.w);
+      *reinterpret_cast<uint2*>(d + o_im + 8) = make_uint2(w.x, w.y);
+    });
     return;
   }
   const int u = blockIdx.x - nb, b = u / mtiles, mt = u % mtiles;
@@ -211,84 +315,56 @@ __global__ void __launch_bounds__(256) gj64_pivot_kernel(const double2* __restri
 // ------------------------------------------------------------------ R panel
 
 struct RSmem {
-  static constexpr int kA = kATile * 2;          // digits of 128 columns of A_K
-  static constexpr int kB = kS * 64 * kK * 2;    // digits of the 64 real rows of P
+  static constexpr int kA = kATile * 2;  // digits of 128 columns of A_K
+  static constexpr int kB = kPTile * 2;  // digits of the 64 real rows of P
   static constexpr int kBytes = kA + kB + 1024;
 };
 
 // Digits of R = P A_{K,:} for 128 columns j of one matrix: thread (j = t & 127,
-// h = t >> 7) cuts half of column j of A_K into digits (the MMA's A operand:
-// rows j, k = [re | im]), all threads the rows of P (the B operand: row 2r =
-// [Re P_r | -Im P_r], row 2r + 1 = [Im P_r | Re P_r]); 28 digit products give
-// Re, Im of R[r][j] at lane j, columns 2r, 2r + 1 of seven orders; each thread
-// turns 32 of its column's 64 sums into FP64 and those into the digits of the
-// update's B operand: row 2j = [Re R_j | -Im R_j], row 2j + 1 = [Im R_j | Re R_j],
-// one exponent per column.  A column costs the same whatever np is; at one CTA
-// per SM the phases follow one another (latency bound), 4 % of the update's work.
-__global__ void __launch_bounds__(256, 1)
+// h = t >> 7) cuts a quarter of column j of A_K into digits (the MMA's A
+// operand: rows j, k = [re | im]) while the digits of P come in (the B
+// operand); 28 digit products give Re, Im of R[r][j] at lane j, columns 2r,
+// 2r + 1 of seven orders; each thread turns 16 of its column's 64 sums into
+// FP64 and those into the digits of the update's B operand: row 2j =
+// [Re R_j | -Im R_j], row 2j + 1 = [Im R_j | Re R_j], one exponent per column.
+// One CTA per SM, its phases one after the other: latency bound, hence 16 warps.
+__global__ void __launch_bounds__(512, 1)
     gj64_rpanel_kernel(const double2* __restrict__ A, int np, int k0, const double2* __restrict__ Pbuf,
+                       const __nv_bfloat16* __restrict__ pimg, const int* __restrict__ pexp,
                        __nv_bfloat16* __restrict__ rimg, int* __restrict__ rexp, int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __nv_bfloat16* sa = reinterpret_cast<__nv_bfloat16*>(smem);
   __nv_bfloat16* sp = reinterpret_cast<__nv_bfloat16*>(smem + RSmem::kA);
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bars[2];  // the digits of P, the products
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   __shared__ unsigned colmax[2][128];
-  __shared__ int pexp[kNB];
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, warp = t >> 5;
   const int b = blockIdx.y, j0 = blockIdx.x * 128, jl = t & 127, h = t >> 7, j = j0 + jl;
   constexpr uint32_t kCols = 512;  // 7 x 64
   if (t == 0) {
-    mbar_init(&bar, 1);
+    mbar_init(&bars[0], 1);
+    mbar_init(&bars[1], 1);
     abort_flag = 0;
     fence_barrier_init();
+    mbar_arrive_expect_tx(&bars[0], RSmem::kB);
+    bulk_g2s(sp, pimg + (size_t)b * kPTile, RSmem::kB, &bars[0]);
   }
   if (t < 128) colmax[0][t] = colmax[1][t] = 0;
   if (warp == 0) tmem_alloc(&tmem_slot, kCols);
-  const double2* P = Pbuf + (size_t)b * kNB * kNB;
-  double2 z[16];
-  const double2* src = A + (size_t)b * np * np + (size_t)(k0 + 16 * h) * np + j;
+  double2 z[8];
+  const double2* src = A + (size_t)b * np * np + (size_t)(k0 + 8 * h) * np + j;
 #pragma unroll
-  for (int c = 0; c < 16; ++c) z[c] = src[(size_t)c * np];
-  {  // rows of P: eight threads per row, four entries each
-    const int r = t >> 3, c4 = 4 * (t & 7);
-    double2 p[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) p[c] = P[r * kNB + c4 + c];
-    unsigned m = 0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) m = max(m, max(mag_hi(p[c].x), mag_hi(p[c].y)));
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const int be = row_biased(m);
-    if ((t & 7) == 0) pexp[r] = be - 1022;
-    if (m >= 0x7ff00000u && status) atomicCAS(status, 0, DS_SINGULAR);
-    long long y[8];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      y[c] = digit_word(p[c].x, be);
-      y[4 + c] = digit_word(p[c].y, be);
-    }
-    const int o_re = core_off(2 * r, c4), o_im = core_off(2 * r, 32 + c4);  // row 2r + 1: 8 elements on
-    put_digits(y, [&](int s, uint4 v) {
-      __nv_bfloat16* d = sp + s * 64 * kK;
-      const uint4 w = neg_bf16(v);
-      *reinterpret_cast<uint2*>(d + o_re) = make_uint2(v.x, v.y);
-      *reinterpret_cast<uint2*>(d + o_im) = make_uint2(w.z, w.w);
-      *reinterpret_cast<uint2*>(d + o_re + 8) = make_uint2(v.z, v.w);
-      *reinterpret_cast<uint2*>(d + o_im + 8) = make_uint2(v.x, v.y);
-    });
-  }
+  for (int c = 0; c < 8; ++c) z[c] = src[(size_t)c * np];
   tc_fence_before();
-  __syncthreads();  // colmax cleared, TMEM allocated
+  __syncthreads();  // barriers, colmax, TMEM address
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   {
     unsigned m = 0;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) m = max(m, max(mag_hi(z[c].x), mag_hi(z[c].y)));
+    for (int c = 0; c < 8; ++c) m = max(m, max(mag_hi(z[c].x), mag_hi(z[c].y)));
     atomicMax(&colmax[0][jl], m);
   }
   __syncthreads();
@@ -296,68 +372,66 @@ __global__ void __launch_bounds__(256, 1)
   if (cm >= 0x7ff00000u && h == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
   const int be_a = row_biased(cm);
 #pragma unroll
-  for (int part = 0; part < 2; ++part)
+  for (int part = 0; part < 2; ++part) {
+    long long y[8];
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      long long y[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) y[c] = digit_word(part ? z[8 * g + c].y : z[8 * g + c].x, be_a);
-      const int off = core_off(jl, 32 * part + 16 * h + 8 * g);
-      put_digits(y, [&](int s, uint4 v) { *reinterpret_cast<uint4*>(sa + s * kARow + off) = v; });
-    }
+    for (int c = 0; c < 8; ++c) y[c] = digit_word(part ? z[c].y : z[c].x, be_a);
+    const int off = core_off(jl, 32 * part + 8 * h);
+    put_digits(y, [&](int s, uint4 v) { *reinterpret_cast<uint4*>(sa + s * kARow + off) = v; });
+  }
   fence_proxy_async();
-  __syncthreads();
+  bool ok = mbar_wait(&bars[0], 0, &abort_flag);
+  if (!ok) drain_wait(&bars[0], 0);
+  ok = __syncthreads_and(ok);
   if (t == 0) {
-    for (int a = 0; a < kS; ++a)
-      for (int n0 = 0; n0 < (kS - a) * 64; n0 += 256) {  // an MMA's N is at most 256
-        const int n = (kS - a) * 64 - n0 < 256 ? (kS - a) * 64 - n0 : 256;
+    tc_fence_after();
+    if (ok)
+      for (int a = 0; a < kS; ++a)
+        for (int n0 = 0; n0 < (kS - a) * 64; n0 += 256) {  // an MMA's N is at most 256
+          const int n = (kS - a) * 64 - n0 < 256 ? (kS - a) * 64 - n0 : 256;
 #pragma unroll
-        for (int kk = 0; kk < kK / 16; ++kk)
-          mma_bf16(tmem + (uint32_t)(a * 64 + n0), smem_desc(smem_u32(sa + a * kARow) + kk * 256, 128, 1024),
-                   smem_desc(smem_u32(sp + n0 * kK) + kk * 256, 128, 1024), idesc_bf16(128, n),
-                   (a > 0 || kk > 0) ? 1u : 0u);
-      }
-    mma_commit(&bar);
+          for (int kk = 0; kk < kK / 16; ++kk)
+            mma_bf16(tmem + (uint32_t)(a * 64 + n0), smem_desc(smem_u32(sa + a * kARow) + kk * 256, 128, 1024),
+                     smem_desc(smem_u32(sp + n0 * kK) + kk * 256, 128, 1024), idesc_bf16(128, n),
+                     (a > 0 || kk > 0) ? 1u : 0u);
+        }
+    mma_commit(&bars[1]);
   }
   // the products read this CTA's shared memory: nobody leaves before they are done
-  bool ok = mbar_wait(&bar, 0, &abort_flag);
-  if (!ok) {
-    const uint64_t t0 = global_ns();
-    while (!mbar_test(&bar, 0) && global_ns() - t0 < kDrainNs) {
-    }
-  }
+  if (ok) ok = mbar_wait(&bars[1], 0, &abort_flag);
+  if (!ok) drain_wait(&bars[1], 0);
   ok = __syncthreads_and(ok);
   tc_fence_after();
   if (ok) {
     const int ebase = 1023 + (be_a - 1022) - 53;
-    const bool in_k = j >= k0 && j < k0 + kNB;
-    double2 rv[16];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {  // eight sums (four rows r) at a time
+    const double2* P = Pbuf + (size_t)b * kNB * kNB;
+    double2 rv[8];
+#pragma unroll 1
+    for (int g = 0; g < 2; ++g) {  // eight sums (four rows r) at a time
       float c[kS][8];
 #pragma unroll
       for (int o = 0; o < kS; ++o)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=f"(c[o][0]), "=f"(c[o][1]), "=f"(c[o][2]), "=f"(c[o][3]), "=f"(c[o][4]), "=f"(c[o][5]),
-                       "=f"(c[o][6]), "=f"(c[o][7])
-                     : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(o * 64 + 32 * h + 8 * g)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tmem_ld8(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(o * 64 + 16 * h + 8 * g), c[o]);
+      tmem_wait_ld();
+      double2 x[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int eb = ebase + pexp[16 * h + 4 * g + q];
-        rv[4 * g + q].x = orders_to_double(c[0][2 * q], c[1][2 * q], c[2][2 * q], c[3][2 * q], c[4][2 * q],
-                                           c[5][2 * q], c[6][2 * q], eb);
-        rv[4 * g + q].y = orders_to_double(c[0][2 * q + 1], c[1][2 * q + 1], c[2][2 * q + 1], c[3][2 * q + 1],
-                                           c[4][2 * q + 1], c[5][2 * q + 1], c[6][2 * q + 1], eb);
+        const int eb = ebase + pexp[b * kNB + 8 * h + 4 * g + q];
+        x[q].x = orders_to_double(c[0][2 * q], c[1][2 * q], c[2][2 * q], c[3][2 * q], c[4][2 * q], c[5][2 * q],
+                                  c[6][2 * q], eb);
+        x[q].y = orders_to_double(c[0][2 * q + 1], c[1][2 * q + 1], c[2][2 * q + 1], c[3][2 * q + 1],
+                                  c[4][2 * q + 1], c[5][2 * q + 1], c[6][2 * q + 1], eb);
       }
-    }
-    if (in_k) {
 #pragma unroll
-      for (int r = 0; r < 16; ++r) rv[r] = P[(16 * h + r) * kNB + j - k0];
+      for (int q = 0; q < 4; ++q) (g ? rv[4 + q] : rv[q]) = x[q];
+    }
+    if (j >= k0 && j < k0 + kNB) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) rv[r] = P[(8 * h + r) * kNB + j - k0];
     }
     unsigned m = 0;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) m = max(m, max(mag_hi(rv[r].x), mag_hi(rv[r].y)));
+    for (int r = 0; r < 8; ++r) m = max(m, max(mag_hi(rv[r].x), mag_hi(rv[r].y)));
     atomicMax(&colmax[1][jl], m);
     __syncthreads();
     m = colmax[1][jl];
@@ -366,23 +440,17 @@ __global__ void __launch_bounds__(256, 1)
     if (h == 0) rexp[(size_t)b * np + j] = be - 1022;
     __nv_bfloat16* img = rimg + ((size_t)b * (np / kTn) + (j / kTn)) * kBTile;
     const int row = 2 * (j % kTn);
+    const int o_re = core_off(row, 8 * h), o_im = core_off(row, 32 + 8 * h);  // row 2j + 1: 8 elements on
+    long long y[16];  // Re and Im: rows 2j and 2j + 1 lie side by side, 32 bytes to a store
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      long long y[8];
-      const int o_re = core_off(row, 16 * h + 8 * g), o_im = core_off(row, 32 + 16 * h + 8 * g);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) y[c] = digit_word(rv[8 * g + c].x, be);
-      put_digits(y, [&](int s, uint4 v) {
-        *reinterpret_cast<uint4*>(img + s * kBDig + o_re) = v;
-        *reinterpret_cast<uint4*>(img + s * kBDig + o_im + 8) = v;  // row 2j + 1
-      });
-#pragma unroll
-      for (int c = 0; c < 8; ++c) y[c] = digit_word(rv[8 * g + c].y, be);
-      put_digits(y, [&](int s, uint4 v) {
-        *reinterpret_cast<uint4*>(img + s * kBDig + o_im) = neg_bf16(v);
-        *reinterpret_cast<uint4*>(img + s * kBDig + o_re + 8) = v;
-      });
+    for (int c = 0; c < 8; ++c) {
+      y[c] = digit_word(rv[c].x, be);
+      y[8 + c] = digit_word(rv[c].y, be);
     }
+    put_digits2(y, [&](int s, uint4 re, uint4 im) {
+      st32(img + s * kBDig + o_re, re, im);
+      st32(img + s * kBDig + o_im, neg_bf16(im), re);
+    });
   }
   tc_fence_before();
   __syncthreads();
@@ -396,29 +464,21 @@ __global__ void __launch_bounds__(256, 1)
 // ------------------------------------------------------------------ update
 
 constexpr int kEpiW = 8;     // epilogue warps, two per TMEM lane quarter
-constexpr int kBoxCols = 4;  // complex columns of a box (64 bytes per row), 32 rows
+constexpr int kBoxCols = 8;  // complex columns of a box (128 bytes per row), 32 rows
 constexpr int kBoxBytes = 32 * kBoxCols * 16;
-constexpr int kRing = 3;     // boxes of a warp: one worked on, two coming in or going out
 struct USmem {
   static constexpr int kA = kATile * 2;
   static constexpr int kB = kBTile * 2;
-  static constexpr int kBoxes = kEpiW * kRing * kBoxBytes;
+  static constexpr int kBoxes = kEpiW * kBoxBytes;
   static constexpr int kBars = 512;
   static constexpr int kBytes = kA + 2 * kB + kBoxes + kBars + 1024;
 };
 struct UBars {
   uint64_t a_full, a_empty, b_full[2], b_empty[2], d_full[2], d_empty[2], drain;
-  uint64_t box[kEpiW * kRing];
   uint32_t tmem_slot;
   int abort;
 };
 static_assert(sizeof(UBars) <= USmem::kBars, "barrier block");
-
-__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = global_ns();
-  while (!mbar_test(bar, parity) && global_ns() - t0 < kDrainNs) {
-  }
-}
 
 // Persistent over tiles of 128 rows x 16 complex columns, column tiles fastest,
 // a contiguous run per CTA: the 112 KB of C digits stay in shared memory for a
@@ -426,16 +486,16 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
 // products (two buffers), two accumulator sets of 7 x 32 TMEM columns let the
 // products of one tile run beside the epilogue of the other.  Warp 0 loads,
 // warp 1 issues 28 MMAs per tile (7 digits x 4 k steps, N = 224 .. 32), warps
-// 2-9 drain: a thread has one row and 8 complex columns, in two boxes of four.
-// The old values come in by TMA two boxes ahead (64-byte swizzle: conflict-free
-// 16-byte accesses with one row per lane), the result leaves by TMA from the
-// same box.  Column tiles at or past `jskip` move up by `nskip` (a window that
-// another kernel updates).
-// What bounds it: the FP64 matrix is read and written once per 32 columns, 64 KB
-// per tile, 3050 cycles at 6.5 TB/s over 152 SMs; the products take 1792, the
-// epilogue about 1800 issue cycles, its FP64 subtraction 2048.
-// With TMA FP64 reductions at L2 in place of load and subtract the payload rate
-// measured 2.6 TB/s against 3.3 TB/s for read-modify-write: not used.
+// 2-9 drain: a thread has one row and 8 complex columns, a warp one box of 32
+// rows x 128 bytes, which is added to A at L2 by a TMA FP64 reduction (rows and
+// columns of block K: stored).  Column tiles at or past `jskip` move up by
+// `nskip` (a window that another kernel updates).
+// What bounds it: the L2's FP64 reductions, 2.6 TB/s of payload measured alone;
+// here 604 MB (64 matrices of 768 x 768) in 243 us, 2.5 TB/s.  Products 1792
+// cycles per tile of 4400, epilogue about 1700 issue cycles.  Measured before
+// it: old values loaded by TMA in 64-byte rows two boxes ahead, subtracted and
+// stored, 292 us (the shared memory left for boxes does not cover the latency);
+// half of the boxes each way, 274 us.
 __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
     gj64_update_kernel(const __grid_constant__ CUtensorMap amap, int np, int mtiles, int ntn, int total, int k0,
                        int jskip, int nskip, const __nv_bfloat16* __restrict__ cimg, const int* __restrict__ cexp,
@@ -462,7 +522,6 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
       mbar_init(&bars.d_empty[s], kEpiW);
     }
     mbar_init(&bars.drain, 1);
-    for (int k = 0; k < kEpiW * kRing; ++k) mbar_init(&bars.box[k], 1);
     bars.abort = 0;
     fence_barrier_init();
   }
@@ -529,88 +588,72 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
     }
   } else {
     const int w = warp - 2, quarter = warp & 3, c0 = 8 * (w >> 2);
-    unsigned char* box0 = sbox + w * kRing * kBoxBytes;
-    uint64_t* box_bar = bars.box + w * kRing;
-    const int nbox = 2 * (hi - lo);
-    // row and column of box k's corner in the batch's matrix of 2 np doubles per row
-    auto corner = [&](int k, int& x, int& y) {
-      const int tile = lo + (k >> 1), u = tile / ntn, jt = col_tile(tile % ntn);
-      x = 2 * (jt * kTn + c0 + kBoxCols * (k & 1));
-      y = (u / mtiles) * np + (u % mtiles) * 128 + quarter * 32;
+    unsigned char* box = sbox + w * kBoxBytes;
+    // tile coordinates: column tile, matrix, row tile; stepped, not divided
+    struct Pos {
+      int jn, b, mt;
     };
-    auto fetch = [&](int k) {  // lane 0
-      int x, y;
-      corner(k, x, y);
-      mbar_arrive_expect_tx(&box_bar[k % kRing], kBoxBytes);
-      tma_load_2d(&amap, box0 + (k % kRing) * kBoxBytes, x, y, &box_bar[k % kRing]);
+    auto step = [&](Pos& p) {
+      if (++p.jn == ntn) {
+        p.jn = 0;
+        if (++p.mt == mtiles) {
+          p.mt = 0;
+          ++p.b;
+        }
+      }
     };
-    int issued = 0;
-    if (lane == 0)
-      for (; issued < 2 && issued < nbox; ++issued) fetch(issued);
+    Pos cur{lo % ntn, lo / ntn / mtiles, lo / ntn % mtiles};
     bool ok = true;
     for (int tile = lo, it = 0; tile < hi && ok; ++tile, ++it) {
-      const int u = tile / ntn, jt = col_tile(tile % ntn), s = it & 1;
-      const int b = u / mtiles, i = (u % mtiles) * 128 + quarter * 32 + lane;
+      const int jt = col_tile(cur.jn), s = it & 1;
+      const int b = cur.b, i = cur.mt * 128 + quarter * 32 + lane;
       const bool ik = i >= k0 && i < k0 + kNB;  // the same for the whole warp
       const int ei = cexp[(size_t)b * np + i] + 1023 - 53;
       ok = __all_sync(0xffffffffu, mbar_wait(&bars.d_full[s], (it >> 1) & 1, abort_flag));
       if (!ok) break;
       tc_fence_after();
-#pragma unroll 1
-      for (int hb = 0; hb < 2 && ok; ++hb) {
-        const int k = 2 * it + hb, slot = k % kRing, col = c0 + kBoxCols * hb, j = jt * kTn + col;
-        const int4 ej = *reinterpret_cast<const int4*>(rexp + (size_t)b * np + j);
-        float c[kS][8];
+      // the warp's sums at once: the accumulators are free for the next tile's products before the arithmetic
+      float acc[2][kS][8];
+#pragma unroll
+      for (int hb = 0; hb < 2; ++hb)
 #pragma unroll
         for (int o = 0; o < kS; ++o)
-          asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                       : "=f"(c[o][0]), "=f"(c[o][1]), "=f"(c[o][2]), "=f"(c[o][3]), "=f"(c[o][4]), "=f"(c[o][5]),
-                         "=f"(c[o][6]), "=f"(c[o][7])
-                       : "r"(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)s * kDCols +
-                             (uint32_t)(o * 2 * kTn + 2 * col)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (hb == 1) {  // this warp is done with the accumulators
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&bars.d_empty[s]);
-        }
-        ok = __all_sync(0xffffffffu, mbar_wait(&box_bar[slot], (k / kRing) & 1, abort_flag));
-        if (!ok) break;
-        const bool zero = ik || (j >= k0 && j < k0 + kNB);
-        unsigned char* box = box0 + slot * kBoxBytes + lane * 64;
-        const int sw = (lane >> 1) & 3;
-        const int eq[4] = {ej.x, ej.y, ej.z, ej.w};
+          tmem_ld8(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)s * kDCols +
+                       (uint32_t)(o * 2 * kTn + 2 * c0 + 8 * hb),
+                   acc[hb][o]);
+      tmem_wait_ld();
+      tc_fence_before();
+      if (lane == 0) bulk_wait_read_n<0>();  // the last tile's box has been read
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars.d_empty[s]);
+      const int j = jt * kTn + c0;
 #pragma unroll
-        for (int q = 0; q < kBoxCols; ++q) {
-          double2* p = reinterpret_cast<double2*>(box + ((q ^ sw) << 4));
-          const double2 old = zero ? make_double2(0.0, 0.0) : *p;
+      for (int hb = 0; hb < 2; ++hb) {
+        const int4 ej = *reinterpret_cast<const int4*>(rexp + (size_t)b * np + j + 4 * hb);
+        const int eq[4] = {ej.x, ej.y, ej.z, ej.w};
+        const float(&c)[kS][8] = acc[hb];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
           const int eb = ei + eq[q];
           const double dx = orders_to_double(c[0][2 * q], c[1][2 * q], c[2][2 * q], c[3][2 * q], c[4][2 * q],
                                              c[5][2 * q], c[6][2 * q], eb);
           const double dy = orders_to_double(c[0][2 * q + 1], c[1][2 * q + 1], c[2][2 * q + 1], c[3][2 * q + 1],
                                              c[4][2 * q + 1], c[5][2 * q + 1], c[6][2 * q + 1], eb);
-          *p = make_double2(old.x - dx, old.y - dy);
+          *reinterpret_cast<double2*>(box + lane * 128 + (((4 * hb + q) ^ (lane & 7)) << 4)) = make_double2(-dx, -dy);
         }
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) {
-          int x, y;
-          corner(k, x, y);
-          tma_store_2d(&amap, box0 + slot * kBoxBytes, x, y);
-          bulk_commit();
-          if (issued < nbox) {
-            bulk_wait_read_n<1>();  // the store from the slot that is filled next has read it
-            fetch(issued++);
-          }
-        }
-        __syncwarp();
       }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) {
+        const int x = 2 * j, y = b * np + cur.mt * 128 + quarter * 32;
+        if (ik || (j >= k0 && j < k0 + kNB)) tma_store_2d(&amap, box, x, y);  // block K: nothing to add to
+        else tma_reduce_add_2d(&amap, box, x, y);
+        bulk_commit();
+      }
+      __syncwarp();
+      step(cur);
     }
-    if (lane == 0) {
-      // every box load issued has landed (on the normal path they all were waited for)
-      for (int k = issued > kRing ? issued - kRing : 0; k < issued; ++k) drain_wait(&box_bar[k % kRing], (k / kRing) & 1);
-      bulk_wait_all();
-    }
+    if (lane == 0) bulk_wait_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -640,24 +683,26 @@ int encode_f64_boxes(CUtensorMap* map, double2* base, uint64_t np, uint64_t rows
   const cuuint32_t box[2] = {2 * kBoxCols, 32};
   const cuuint32_t elem_strides[2] = {1, 1};
   const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, base, dims, strides, box, elem_strides,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return set_error(NEDMFT_ECUDA, "cuTensorMapEncodeTiled (FP64) failed (CUresult %d)", (int)r);
   return NEDMFT_OK;
 }
 
 struct Gj64Layout {
-  size_t p, c, r, ce, re, total;
+  size_t p, pi, pe, c, r, ce, re, total;
 };
 Gj64Layout gj64_layout(int np, int nb) {
   Gj64Layout L;
   const size_t n = np, b = nb;
   L.p = align256(sizeof(double2) * kNB * kNB * b);
+  L.pi = align256(2 * (size_t)kPTile * b);
+  L.pe = align256(sizeof(int) * kNB * b);
   L.c = align256(2 * (size_t)kATile * (n / 128) * b);
   L.r = align256(2 * (size_t)kBTile * (n / kTn) * b);
   L.ce = align256(sizeof(int) * n * b);
   L.re = align256(sizeof(int) * n * b);
-  L.total = L.p + L.c + L.r + L.ce + L.re;
+  L.total = L.p + L.pi + L.pe + L.c + L.r + L.ce + L.re;
   return L;
 }
 
@@ -680,6 +725,8 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
   const Gj64Layout L = gj64_layout(np, nb);
   char* p = static_cast<char*>(scratch);
   double2* pbuf = reinterpret_cast<double2*>(p); p += L.p;
+  __nv_bfloat16* pimg = reinterpret_cast<__nv_bfloat16*>(p); p += L.pi;
+  int* pexp = reinterpret_cast<int*>(p); p += L.pe;
   __nv_bfloat16* cimg = reinterpret_cast<__nv_bfloat16*>(p); p += L.c;
   __nv_bfloat16* rimg = reinterpret_cast<__nv_bfloat16*>(p); p += L.r;
   int* cexp = reinterpret_cast<int*>(p); p += L.ce;
@@ -693,9 +740,11 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
   if (rc) return rc;
   const int mtiles = np / 128, ntn = ceil_div(n, kTn), total = nb * mtiles * ntn;
   for (int k0 = 0; k0 < n; k0 += kNB) {
-    gj64_pivot_kernel<<<nb + nb * mtiles, 256, 0, st>>>(A, np, mtiles, k0, nb, pbuf, cimg, cexp, status);
+    gj64_pivot_kernel<<<nb + nb * mtiles, 256, 0, st>>>(A, np, mtiles, k0, nb, pbuf, pimg, pexp, cimg,
+                                                          cexp, status);
     NED_LAUNCH_CHECK("gj64_pivot_kernel");
-    gj64_rpanel_kernel<<<dim3(mtiles, nb), 256, RSmem::kBytes, st>>>(A, np, k0, pbuf, rimg, rexp, status);
+    gj64_rpanel_kernel<<<dim3(mtiles, nb), 512, RSmem::kBytes, st>>>(A, np, k0, pbuf, pimg, pexp, rimg, rexp,
+                                                                        status);
     NED_LAUNCH_CHECK("gj64_rpanel_kernel");
     const int slot = instr_begin(st);
     gj64_update_kernel<<<total < sms ? total : sms, 64 + 32 * kEpiW, USmem::kBytes, st>>>(

@@ -8,9 +8,8 @@ namespace nedmft {
 int launch_build_s(const ContourDev& c, const double2* sigma, double2* S, cudaStream_t st);
 int launch_g0_build(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, int nq,
                     double2* g0, cudaStream_t st);
-template <class T>
 int launch_gen_a(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, int q0, int nb,
-                 const double2* S, cplx_t<T>* A, int np, cudaStream_t st);
+                 const double2* S, double2* A, int np, cudaStream_t st);
 
 // Largest n_c of the single-CTA FP64 Gauss-Jordan path (whole matrix in shared memory).
 constexpr int kSmallPathMaxN = 112;
@@ -24,10 +23,9 @@ size_t gj64_scratch_bytes(int np, int nb);
 int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, cudaStream_t st);
 int gj64_set_wait_ns(uint64_t ns, cudaStream_t st);  // its bounded waits' limit on the current device
 
-template <class T>
 int launch_reduce(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, const double* wq,
-                  int q0, int nb, const cplx_t<T>* X, const cplx_t<T>* dX, int ldx, bool cycled, bool first,
-                  double2* gloc, double2* jacc, cudaStream_t st);
+                  int q0, int nb, const double2* X, int ldx, bool cycled, bool first, double2* gloc, double2* jacc,
+                  cudaStream_t st);
 int launch_finish_current(int nt, const double2* jacc, double* j, double* ji, cudaStream_t st);
 
 // Dense FP64 inversion with partial pivoting (impurity step).

@@ -67,41 +67,58 @@ int launch_g0_build(const ContourDev& c, const ModelDev& m, const double* eps, c
 
 // ------------------------------------------------------------------ A'_q = P (B_q - S), padded
 
-template <class T>
-__global__ void gen_a_kernel(ContourDev c, ModelDev m, const double* __restrict__ eps_d,
-                             const double* __restrict__ ebar_d, int q0, const double2* __restrict__ S,
-                             cplx_t<T>* __restrict__ A, int np) {
-  const int b = blockIdx.y;
-  const double eps = eps_d[q0 + b], ebar = ebar_d[q0 + b];
-  const bool sh = shifted_point(m, eps);
-  const size_t total = (size_t)np * np;
-  cplx_t<T>* out = A + (size_t)b * total;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    int r = (int)(e / np), col = (int)(e % np);
-    double2 v;
-    if (r < c.n && col < c.n) {
-      int i = sh ? (r + 1 == c.n ? 0 : r + 1) : r;
-      v = a_entry(c, m, eps, ebar, S, i, col);
-    } else {
-      v = make_double2(r == col ? 1.0 : 0.0, 0.0);
+// 32 rows of one matrix per CTA: the first warp forms the rows' entries of B_q
+// (one lane per row, so a sincos and an exponential per row run side by side),
+// then a warp per row copies -S and adds them.  One pass over the output: HBM
+// bound.  (With the entry of B_q formed where the copying thread met it, one
+// lane of a warp ran that chain while 31 waited: 450 us for 100 matrices of
+// 256 x 256, 105 MB.)
+constexpr int kGenRows = 32;
+__global__ void __launch_bounds__(256) gen_a_kernel(ContourDev c, ModelDev m, const double* __restrict__ eps_d,
+                                                    const double* __restrict__ ebar_d, int q0,
+                                                    const double2* __restrict__ S, double2* __restrict__ A, int np) {
+  const int r0 = blockIdx.x * kGenRows, b = blockIdx.y;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ double2 sub[kGenRows];  // the entry of B_q left of the diagonal, or in the corner for row 0
+  __shared__ int src_row[kGenRows];
+  if (warp == 0) {
+    const double eps = eps_d[q0 + b], ebar = ebar_d[q0 + b];
+    const int r = r0 + lane;
+    int i = r;
+    if (r < c.n && shifted_point(m, eps)) i = r + 1 == c.n ? 0 : r + 1;
+    src_row[lane] = i;
+    if (i < c.n) sub[lane] = i >= 1 ? b_sub(c, m, eps, ebar, i) : b_corner(c, m, eps);
+  }
+  __syncthreads();
+  for (int rr = warp; rr < kGenRows; rr += 8) {
+    const int i = src_row[rr];
+    double2* dst = A + (size_t)b * np * np + (size_t)(r0 + rr) * np;
+    if (i >= c.n) {  // padding
+      for (int j = lane; j < np; j += 32) dst[j] = make_double2(j == i ? 1.0 : 0.0, 0.0);
+      continue;
     }
-    out[e] = cvt<T>(v);
+    const double2* src = S + (size_t)i * c.n;
+    const int js = i >= 1 ? i - 1 : c.n - 1;
+    for (int j = lane; j < np; j += 32) {
+      double2 v = make_double2(0.0, 0.0);
+      if (j < c.n) {
+        v = src[j];
+        v.x = -v.x;
+        v.y = -v.y;
+        if (j == i) v.y += 1.0;
+        if (j == js) v = cadd(v, sub[rr]);
+      }
+      dst[j] = v;
+    }
   }
 }
 
-template <class T>
 int launch_gen_a(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, int q0, int nb,
-                 const double2* S, cplx_t<T>* A, int np, cudaStream_t st) {
-  size_t total = (size_t)np * np;
-  int bx = (int)((total + 255) / 256);
-  if (bx > 4096) bx = 4096;
-  dim3 grid(bx, nb);
-  gen_a_kernel<T><<<grid, 256, 0, st>>>(c, m, eps, ebar, q0, S, A, np);
+                 const double2* S, double2* A, int np, cudaStream_t st) {
+  gen_a_kernel<<<dim3(np / kGenRows, nb), 256, 0, st>>>(c, m, eps, ebar, q0, S, A, np);
   NED_LAUNCH_CHECK("gen_a_kernel");
   return NEDMFT_OK;
 }
-template int launch_gen_a<double>(const ContourDev&, const ModelDev&, const double*, const double*, int, int,
-                                  const double2*, double2*, int, cudaStream_t);
 
 // ------------------------------------------------------------------ record a device failure
 
@@ -709,55 +726,88 @@ int pivot_inverse(double2* a, int n, void* ws, cudaStream_t st, int* status) {
 
 // ------------------------------------------------------------------ FP64 reductions over the points
 
-// gloc[i][j] (= or +=) sum_b wq[q0+b] (X[b] + dX[b])[i][col(j)], b ascending,
-// col = unshift_col if `cycled` (the batch holds X' = (P A)^-1).
-template <class T>
-__global__ void reduce_gloc_kernel(ContourDev c, ModelDev m, const double* __restrict__ eps_d,
-                                   const double* __restrict__ wq_d, int q0, int nb, const cplx_t<T>* __restrict__ X,
-                                   const cplx_t<T>* __restrict__ dX, int ldx, bool cycled, bool first,
-                                   double2* __restrict__ gloc) {
-  const size_t total = (size_t)c.n * c.n;
-  const size_t bstride = (size_t)ldx * ldx;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    int i = (int)(e / c.n), j = (int)(e % c.n);
-    double2 acc = first ? make_double2(0.0, 0.0) : gloc[e];
-    for (int b = 0; b < nb; ++b) {
-      const int q = q0 + b;
-      const bool sh = cycled && shifted_point(m, eps_d[q]);
-      const size_t off = (size_t)b * bstride + (size_t)i * ldx + unshift_col(j, c.n, sh);
-      double2 v = to_d(X[off]);
-      if (dX) v = cadd(v, to_d(dX[off]));
-      const double w = wq_d[q];
-      acc.x = fma(w, v.x, acc.x);
-      acc.y = fma(w, v.y, acc.y);
+// gloc[i][j] (= or +=) sum_b wq[q0+b] X[b][i][col(j)], b ascending, col =
+// unshift_col if `cycled` (the batch holds X' = (P A)^-1).  A thread per entry
+// with eight matrices' loads in flight, the weights of 256 points at a time in
+// shared memory; small blocks, so that an 80 x 80 result covers the SMs (100 us
+// with one load in flight and 25 blocks, 256 points of 80 x 80).
+constexpr int kRedPts = 256;
+__global__ void __launch_bounds__(128) reduce_gloc_kernel(ContourDev c, ModelDev m, const double* __restrict__ eps_d,
+                                                          const double* __restrict__ wq_d, int q0, int nb,
+                                                          const double2* __restrict__ X, int ldx, bool cycled,
+                                                          bool first, double2* __restrict__ gloc) {
+  __shared__ double w[kRedPts];
+  __shared__ bool sh[kRedPts];
+  const size_t total = (size_t)c.n * c.n, bstride = (size_t)ldx * ldx;
+  const size_t span = (size_t)gridDim.x * blockDim.x;
+  for (size_t e0 = (size_t)blockIdx.x * blockDim.x; e0 < total; e0 += span) {  // the same trips for a whole block
+    const size_t e = e0 + threadIdx.x;
+    const bool live = e < total;
+    const int i = (int)((live ? e : 0) / c.n), j = (int)((live ? e : 0) % c.n);
+    const size_t off0 = (size_t)i * ldx + j, off1 = (size_t)i * ldx + unshift_col(j, c.n, true);
+    double2 acc = first || !live ? make_double2(0.0, 0.0) : gloc[e];
+    for (int p0 = 0; p0 < nb; p0 += kRedPts) {
+      const int np = nb - p0 < kRedPts ? nb - p0 : kRedPts;
+      __syncthreads();
+      for (int b = threadIdx.x; b < np; b += blockDim.x) {
+        w[b] = wq_d[q0 + p0 + b];
+        sh[b] = cycled && shifted_point(m, eps_d[q0 + p0 + b]);
+      }
+      __syncthreads();
+      constexpr int U = 8;
+      for (int b0 = 0; b0 < np && live; b0 += U) {
+        double2 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          v[u] = b0 + u < np ? X[(size_t)(p0 + b0 + u) * bstride + (sh[b0 + u] ? off1 : off0)] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (b0 + u < np) {
+            acc.x = fma(w[b0 + u], v[u].x, acc.x);
+            acc.y = fma(w[b0 + u], v[u].y, acc.y);
+          }
+      }
     }
-    gloc[e] = acc;
+    if (live) gloc[e] = acc;
   }
 }
 
-// jacc[m] (= or +=) sum_b wq ebar_q(t_m) G_q[m][2 N_t - m].
-template <class T>
-__global__ void reduce_current_kernel(ContourDev c, ModelDev mo, const double* __restrict__ eps_d,
-                                      const double* __restrict__ ebar_d, const double* __restrict__ wq_d, int q0,
-                                      int nb, const cplx_t<T>* __restrict__ X, const cplx_t<T>* __restrict__ dX,
-                                      int ldx, bool cycled, bool first, double2* __restrict__ jacc) {
-  const int mm = blockIdx.x * blockDim.x + threadIdx.x;
-  if (mm >= c.nt) return;
+// jacc[m] (= or +=) sum_b wq ebar_q(t_m) G_q[m][2 N_t - m]: a warp per time,
+// lane l the points l, l + 32, ..., the lanes' sums added in a fixed tree.  The
+// field's sine and cosine are the time's, not the point's (287 us with a thread
+// per time and a sincos per point, 256 points).
+__global__ void __launch_bounds__(128) reduce_current_kernel(ContourDev c, ModelDev mo,
+                                                             const double* __restrict__ eps_d,
+                                                             const double* __restrict__ ebar_d,
+                                                             const double* __restrict__ wq_d, int q0, int nb,
+                                                             const double2* __restrict__ X, int ldx, bool cycled,
+                                                             bool first, double2* __restrict__ jacc) {
+  const int mm = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (mm >= c.nt) return;  // whole warps
   const double t = t_re(c, mm);
   const int jcol = 2 * c.nt - mm;
-  double2 acc = first ? make_double2(0.0, 0.0) : jacc[mm];
-  for (int b = 0; b < nb; ++b) {
+  double sn = 0.0, cs = 1.0;  // ebar_q(t) = ebar cos(Et) + eps sin(Et), ebar before the field
+  if (t > 0.0) sincos(mo.E * t, &sn, &cs);
+  double2 part = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int b = lane; b < nb; b += 32) {
     const int q = q0 + b;
     const double eps = eps_d[q];
-    const bool sh = cycled && shifted_point(mo, eps);
-    const size_t off = (size_t)b * ldx * ldx + (size_t)mm * ldx + unshift_col(jcol, c.n, sh);
-    double2 v = to_d(X[off]);
-    if (dX) v = cadd(v, to_d(dX[off]));
-    const double w = wq_d[q] * ebar_at(t, eps, ebar_d[q], mo.E);
-    acc.x = fma(w, v.x, acc.x);
-    acc.y = fma(w, v.y, acc.y);
+    const double2 v = X[(size_t)b * ldx * ldx + (size_t)mm * ldx +
+                        unshift_col(jcol, c.n, cycled && shifted_point(mo, eps))];
+    const double w = wq_d[q] * (ebar_d[q] * cs + eps * sn);
+    part.x = fma(w, v.x, part.x);
+    part.y = fma(w, v.y, part.y);
   }
-  jacc[mm] = acc;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    part.x += __shfl_xor_sync(0xffffffffu, part.x, o);
+    part.y += __shfl_xor_sync(0xffffffffu, part.y, o);
+  }
+  if (lane == 0) {
+    const double2 acc = first ? make_double2(0.0, 0.0) : jacc[mm];
+    jacc[mm] = cadd(acc, part);
+  }
 }
 
 // j = Re(i acc) = -acc.y, j_imag = Im(i acc) = acc.x.
@@ -769,25 +819,20 @@ __global__ void finish_current_kernel(int nt, const double2* __restrict__ jacc, 
   if (ji) ji[mm] = jacc[mm].x;
 }
 
-template <class T>
 int launch_reduce(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, const double* wq,
-                  int q0, int nb, const cplx_t<T>* X, const cplx_t<T>* dX, int ldx, bool cycled, bool first,
-                  double2* gloc, double2* jacc, cudaStream_t st) {
-  size_t total = (size_t)c.n * c.n;
-  int bx = (int)((total + 255) / 256);
-  if (bx > 152 * 8) bx = 152 * 8;
-  reduce_gloc_kernel<T><<<bx, 256, 0, st>>>(c, m, eps, wq, q0, nb, X, dX, ldx, cycled, first, gloc);
+                  int q0, int nb, const double2* X, int ldx, bool cycled, bool first, double2* gloc, double2* jacc,
+                  cudaStream_t st) {
+  const size_t total = (size_t)c.n * c.n;
+  const size_t blocks = (total + 127) / 128;
+  reduce_gloc_kernel<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 128, 0, st>>>(c, m, eps, wq, q0, nb, X, ldx,
+                                                                                   cycled, first, gloc);
   NED_LAUNCH_CHECK("reduce_gloc_kernel");
   if (jacc) {
-    reduce_current_kernel<T><<<ceil_div(c.nt, 128), 128, 0, st>>>(c, m, eps, ebar, wq, q0, nb, X, dX, ldx, cycled,
-                                                                  first, jacc);
+    reduce_current_kernel<<<ceil_div(c.nt, 4), 128, 0, st>>>(c, m, eps, ebar, wq, q0, nb, X, ldx, cycled, first, jacc);
     NED_LAUNCH_CHECK("reduce_current_kernel");
   }
   return NEDMFT_OK;
 }
-template int launch_reduce<double>(const ContourDev&, const ModelDev&, const double*, const double*, const double*,
-                                   int, int, const double2*, const double2*, int, bool, bool, double2*, double2*,
-                                   cudaStream_t);
 
 int launch_finish_current(int nt, const double2* jacc, double* j, double* ji, cudaStream_t st) {
   finish_current_kernel<<<ceil_div(nt, 128), 128, 0, st>>>(nt, jacc, j, ji);

@@ -78,7 +78,7 @@ extern "C" int nedmft_lattice_gloc_static(const nedmft_contour* c, const nedmft_
   for (int q0 = 0; q0 < nq; q0 += kStaticBatch) {
     const int nb = nq - q0 < kStaticBatch ? nq - q0 : kStaticBatch;
     if ((rc = launch_gj_small_fp64(cd, md, eps_d, ebar_d, q0, nb, S, out, status, st))) return rc;
-    if ((rc = launch_reduce<double>(cd, md, eps_d, ebar_d, wq_d, q0, nb, out, nullptr, cd.n, false, q0 == 0, gl, ja,
+    if ((rc = launch_reduce(cd, md, eps_d, ebar_d, wq_d, q0, nb, out, cd.n, false, q0 == 0, gl, ja,
                                     st)))
       return rc;
   }
