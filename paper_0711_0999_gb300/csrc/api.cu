@@ -24,8 +24,15 @@ ModelDev model_dev(const nedmft_model& m) { return ModelDev{m.U, m.E, m.w1, isna
 
 enum class Path { Small64, Blocked64, MixedUmma };
 
+// FP64: the whole matrix in shared memory up to 20 rows, the blocked tensor-core
+// elimination above.  Both measured, 4 x 4 / 8 x 8 / 32 x 32 points: 104 / 116 /
+// 808 us against 109 / 128 / 1305 us at 20 rows, 142 / 159 / 1030 against 110 /
+// 126 / 1273 at 24 (304 points a batch), 3374 / 3390 / 24048 against 358 / 410 /
+// 4117 at 112.
+constexpr int kSmall64MaxN = 20;
+
 Path choose_path(const nedmft_contour& c, nedmft_precision p) {
-  if (p == NEDMFT_FP64) return c.n_c <= small_path_max_n() ? Path::Small64 : Path::Blocked64;
+  if (p == NEDMFT_FP64) return c.n_c <= kSmall64MaxN ? Path::Small64 : Path::Blocked64;
   return Path::MixedUmma;
 }
 
@@ -51,13 +58,21 @@ int default_batch(const nedmft_contour& c, int nq, Path path, int width) {
   int cap = 152;
   switch (path) {
     case Path::Small64: per = sizeof(double2) * c.n_c * c.n_c; cap = 2048; break;
-    case Path::Blocked64: per = sizeof(double2) * np * np + gj64_scratch_bytes((int)np, 1); cap = 152; break;
+    case Path::Blocked64:
+      // every step of 32 columns is three launches for the whole batch, two of
+      // them latency bound: larger batches while a step is short (1024 points of
+      // 80 rows 4286 / 3100 / 2420 / 2315 us in batches of 76 / 152 / 304 / 1024;
+      // of 220 rows 11.9 / 10.6 / 8.9 / 8.0 ms)
+      per = sizeof(double2) * np * np + gj64_scratch_bytes((int)np, 1);
+      cap = np <= 256 ? 1024 : np <= 512 ? 608 : 304;
+      break;
     case Path::MixedUmma: per = umma_batch_bytes_per_matrix((int)np, width); cap = umma_default_batch((int)np); break;
   }
   int b = (int)(budget / (per ? per : 1));
   if (b > cap) b = cap;
   if (b > nq) b = nq;
   if (b < 1) b = 1;
+  if (path == Path::Blocked64) b = ceil_div(nq, ceil_div(nq, b));  // batches of even size
   return b;
 }
 
