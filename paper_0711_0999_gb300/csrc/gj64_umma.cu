@@ -21,6 +21,8 @@
 // One MMA per digit a of the left operand takes all its partners b = 0 .. 6-a
 // at once: the right operand's digits lie back to back in shared memory, and
 // orders a .. 6 back to back in TMEM.
+#include <type_traits>
+
 #include "lattice.cuh"
 #include "umma_core.cuh"
 
@@ -188,6 +190,42 @@ __device__ __forceinline__ bool recip(double2 z, double2& out) {
   return true;
 }
 
+// Digits of 128 rows of C = A_{:,K} (C_K = -I), TPR threads per row: image rows
+// [Re | Im].  Row i is read from row src[i - 128 mt] when `src` is given.
+template <int TPR>
+__device__ __forceinline__ void pack_c_rows(const double2* __restrict__ A, int np, int k0, int mt, const int* src,
+                                            __nv_bfloat16* __restrict__ img, int* __restrict__ cexp, int* status) {
+  constexpr int CNT = kNB / TPR;
+  const int row = threadIdx.x / TPR, part = threadIdx.x % TPR, i = mt * 128 + row;
+  double2 z[CNT];
+  if (i >= k0 && i < k0 + kNB) {
+#pragma unroll
+    for (int c = 0; c < CNT; ++c) z[c] = make_double2(CNT * part + c == i - k0 ? -1.0 : 0.0, 0.0);
+  } else {
+    const double2* a = A + (size_t)(src ? src[row] : i) * np + k0 + CNT * part;
+#pragma unroll
+    for (int c = 0; c < CNT; ++c) z[c] = a[c];
+  }
+  unsigned m = 0;
+#pragma unroll
+  for (int c = 0; c < CNT; ++c) m = max(m, max(mag_hi(z[c].x), mag_hi(z[c].y)));
+#pragma unroll
+  for (int o = 1; o < TPR; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (m >= 0x7ff00000u && status) atomicCAS(status, 0, DS_SINGULAR);  // not finite
+  const int be = row_biased(m);
+  if (part == 0) cexp[i] = be - 1022;
+#pragma unroll
+  for (int im = 0; im < 2; ++im)
+#pragma unroll
+    for (int g = 0; g < CNT / 8; ++g) {
+      long long y[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) y[c] = digit_word(im ? z[8 * g + c].y : z[8 * g + c].x, be);
+      const int off = core_off(row, 32 * im + CNT * part + 8 * g);
+      put_digits(y, [&](int s, uint4 v) { *reinterpret_cast<uint4*>(img + s * kARow + off) = v; });
+    }
+}
+
 // CTAs 0 .. nb-1: P = inv(A_KK) of matrix b, 32 x 32 FP64, a warp per four
 // rows, lane = column.  Step k: the pivot row, divided by its pivot (its own
 // entry replaced by the pivot's inverse), is in shared memory (two buffers, one
@@ -282,37 +320,18 @@ __global__ void __launch_bounds__(256) gj64_pivot_kernel(const double2* __restri
     return;
   }
   const int u = blockIdx.x - nb, b = u / mtiles, mt = u % mtiles;
-  const int row = t >> 1, half = t & 1, i = mt * 128 + row;
-  const double2* src = A + (size_t)b * np * np + (size_t)i * np + k0 + 16 * half;
-  double2 z[16];
-  if (i >= k0 && i < k0 + kNB) {
-#pragma unroll
-    for (int c = 0; c < 16; ++c) z[c] = make_double2(16 * half + c == i - k0 ? -1.0 : 0.0, 0.0);
-  } else {
-#pragma unroll
-    for (int c = 0; c < 16; ++c) z[c] = src[c];
-  }
-  unsigned m = 0;
-#pragma unroll
-  for (int c = 0; c < 16; ++c) m = max(m, max(mag_hi(z[c].x), mag_hi(z[c].y)));
-  m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-  if (m >= 0x7ff00000u && status) atomicCAS(status, 0, DS_SINGULAR);  // not finite
-  const int be = row_biased(m);
-  if (half == 0) cexp[(size_t)b * np + i] = be - 1022;
-  __nv_bfloat16* img = cimg + (size_t)u * kATile;
-#pragma unroll
-  for (int part = 0; part < 2; ++part)
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      long long y[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) y[c] = digit_word(part ? z[8 * g + c].y : z[8 * g + c].x, be);
-      const int off = core_off(row, 32 * part + 16 * half + 8 * g);
-      put_digits(y, [&](int s, uint4 v) { *reinterpret_cast<uint4*>(img + s * kARow + off) = v; });
-    }
+  pack_c_rows<2>(A + (size_t)b * np * np, np, k0, mt, nullptr, cimg + (size_t)u * kATile, cexp + (size_t)b * np,
+                 status);
 }
 
 // ------------------------------------------------------------------ R panel
+
+// The row exchanges of one pivoted step: the row chosen for each place of block
+// K, and the block's rows that move out to the chosen rows' places.
+struct RowSwaps {
+  int win[kNB];
+  int moved, to[kNB], from[kNB];
+};
 
 struct RSmem {
   static constexpr int kA = kATile * 2;  // digits of 128 columns of A_K
@@ -328,10 +347,26 @@ struct RSmem {
 // FP64 and those into the digits of the update's B operand: row 2j =
 // [Re R_j | -Im R_j], row 2j + 1 = [Im R_j | Re R_j], one exponent per column.
 // One CTA per SM, its phases one after the other: latency bound, hence 16 warps.
+// With `sw` (one matrix, pivoted): row k0 + r of A_K is row sw->win[r]; the rows
+// that leave block K for the winners' places are copied there, each CTA its own
+// columns; and CTAs mtiles .. 2 mtiles - 1 cut C into digits with the rows so
+// moved.  No CTA writes what another reads: the copies go to the winners' rows,
+// whose only readers are the CTA of the same columns, before its copies.
 __global__ void __launch_bounds__(512, 1)
-    gj64_rpanel_kernel(const double2* __restrict__ A, int np, int k0, const double2* __restrict__ Pbuf,
+    gj64_rpanel_kernel(double2* A, int np, int mtiles, int k0, const double2* __restrict__ Pbuf,
                        const __nv_bfloat16* __restrict__ pimg, const int* __restrict__ pexp,
-                       __nv_bfloat16* __restrict__ rimg, int* __restrict__ rexp, int* status) {
+                       __nv_bfloat16* __restrict__ rimg, int* __restrict__ rexp, const RowSwaps* __restrict__ sw,
+                       __nv_bfloat16* __restrict__ cimg, int* __restrict__ cexp, int* status) {
+  if ((int)blockIdx.x >= mtiles) {
+    __shared__ int src[128];
+    const int mt = blockIdx.x - mtiles, t = threadIdx.x;
+    if (t < 128) src[t] = mt * 128 + t;
+    __syncthreads();
+    if (t < sw->moved && sw->to[t] / 128 == mt) src[sw->to[t] % 128] = sw->from[t];
+    __syncthreads();
+    pack_c_rows<4>(A, np, k0, mt, src, cimg + (size_t)mt * kATile, cexp, status);
+    return;
+  }
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __nv_bfloat16* sa = reinterpret_cast<__nv_bfloat16*>(smem);
@@ -354,12 +389,14 @@ __global__ void __launch_bounds__(512, 1)
   if (t < 128) colmax[0][t] = colmax[1][t] = 0;
   if (warp == 0) tmem_alloc(&tmem_slot, kCols);
   double2 z[8];
-  const double2* src = A + (size_t)b * np * np + (size_t)(k0 + 8 * h) * np + j;
+  double2* col = A + (size_t)b * np * np + j;
 #pragma unroll
-  for (int c = 0; c < 8; ++c) z[c] = src[(size_t)c * np];
+  for (int c = 0; c < 8; ++c) z[c] = col[(size_t)(sw ? sw->win[8 * h + c] : k0 + 8 * h + c) * np];
   tc_fence_before();
-  __syncthreads();  // barriers, colmax, TMEM address
+  __syncthreads();  // barriers, colmax, TMEM address; every row of A_K is read
   tc_fence_after();
+  if (sw)
+    for (int e = h; e < sw->moved; e += 4) col[(size_t)sw->to[e] * np] = col[(size_t)sw->from[e] * np];
   const uint32_t tmem = tmem_slot;
   {
     unsigned m = 0;
@@ -743,8 +780,8 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
     gj64_pivot_kernel<<<nb + nb * mtiles, 256, 0, st>>>(A, np, mtiles, k0, nb, pbuf, pimg, pexp, cimg,
                                                           cexp, status);
     NED_LAUNCH_CHECK("gj64_pivot_kernel");
-    gj64_rpanel_kernel<<<dim3(mtiles, nb), 512, RSmem::kBytes, st>>>(A, np, k0, pbuf, pimg, pexp, rimg, rexp,
-                                                                        status);
+    gj64_rpanel_kernel<<<dim3(mtiles, nb), 512, RSmem::kBytes, st>>>(A, np, mtiles, k0, pbuf, pimg, pexp, rimg, rexp,
+                                                                     nullptr, nullptr, nullptr, status);
     NED_LAUNCH_CHECK("gj64_rpanel_kernel");
     const int slot = instr_begin(st);
     gj64_update_kernel<<<total < sms ? total : sms, 64 + 32 * kEpiW, USmem::kBytes, st>>>(
@@ -753,6 +790,417 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
     const int live = n - k0 < kNB ? n - k0 : kNB;
     instr_end(slot, st, 8.0 * (double)n * n * live * nb, 2.0 * sizeof(double2) * (double)n * n * nb);
   }
+  return NEDMFT_OK;
+}
+
+// ------------------------------------------------------------------ pivoted inversion of one matrix
+
+namespace {
+
+constexpr int kPanCtas = 8;   // CTAs of a panel cluster
+constexpr int kPanWarps = 32;
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, double2 v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, int2 v) {
+  asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "r"(v.x), "r"(v.y) : "memory");
+}
+
+// Pivot choice for the 32 columns from k0 on and, in the last round, the block's
+// inverse.  A cluster of eight CTAs runs partial pivoting in FP32 on up to 256 R
+// candidate rows (rows k0 + i, or in[i]), a warp per R rows, lane = column: per
+// column each warp's largest entry sits in one lane, a warp maximum over the 32
+// warps' gives the CTA's, whose row goes to all eight CTAs' shared memory, and
+// after one cluster barrier every warp picks the largest of the eight and
+// eliminates its own rows with it.  Rows do not move and the column loop is not
+// unrolled (the unrolled form with a row per thread, 200 KB of code used once,
+// spent its time fetching it: 55 us per round of 256 rows).
+// Last round: P = inv of the chosen rows' block in FP64, four rows per CTA, a
+// warp per row, the next pivot row first; its digits (the B operand of
+// gj64_rpanel_kernel); the row exchanges; the row permutation.  Both parts are
+// latency bound: 32 cluster barriers each.
+template <int R>
+__global__ void __cluster_dims__(kPanCtas, 1, 1) __launch_bounds__(32 * kPanWarps, 1)
+    gj64_panel_kernel(const double2* __restrict__ A, int np, int n, int k0, const int* __restrict__ in, int count,
+                      int* __restrict__ out, int last, double2* __restrict__ Pbuf, __nv_bfloat16* __restrict__ pimg,
+                      int* __restrict__ pexp, RowSwaps* __restrict__ sw, int* __restrict__ rowperm, int* status) {
+  __shared__ int cand[2][kPanWarps];                      // the warps' largest |entry|^2, as ordered bits
+  __shared__ __align__(16) float2 crow[2][kPanCtas][32];  // the CTAs' candidate rows
+  __shared__ __align__(8) int2 cmag[2][kPanCtas];         // their |entry|^2 and row
+  __shared__ __align__(16) double2 rowb[2][32];
+  __shared__ int win[kNB];
+  const int q = (int)cluster_ctarank(), c = blockIdx.x / kPanCtas;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int base = c * 256 * R, here = min(count - base, 256 * R);
+  const int ncol = min(kNB, n - k0), steps = min(ncol, here);
+  float2 v[R];
+  int row[R];
+  unsigned live = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int i = base + r * 256 + q * 32 + warp;
+    row[r] = i < base + here ? (in ? in[i] : k0 + i) : -1;
+    v[r] = make_float2(0.f, 0.f);
+    if (row[r] >= 0) {
+      live |= 1u << r;
+      if (lane < ncol) {
+        const double2 z = A[(size_t)row[r] * np + k0 + lane];
+        v[r] = make_float2((float)z.x, (float)z.y);
+      }
+    }
+  }
+  if (threadIdx.x < kNB) win[threadIdx.x] = -1;
+  cluster_barrier();  // every CTA runs before another writes its shared memory
+  for (int j = 0; j < steps; ++j) {
+    const int sb = j & 1;
+    float bm = -1.f;
+    float2 bv = make_float2(0.f, 0.f);
+    int br = 0, brow = -1;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {  // in lane j: this warp's rows' entries of column j
+      const float m = (live >> r) & 1 ? v[r].x * v[r].x + v[r].y * v[r].y : -1.f;
+      if (m > bm) {
+        bm = m;
+        br = r;
+      }
+    }
+    bm = __shfl_sync(0xffffffffu, bm, j);
+    br = __shfl_sync(0xffffffffu, br, j);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (r == br) {
+        bv = v[r];
+        brow = row[r];
+      }
+    if (lane == 0) cand[sb][warp] = __float_as_int(bm);  // -1 orders below every magnitude
+    __syncthreads();
+    const int x = cand[sb][lane];
+    const int top = __reduce_max_sync(0xffffffffu, x);
+    const int wtop = __ffs(__ballot_sync(0xffffffffu, x == top)) - 1;
+    if (warp == wtop) {
+#pragma unroll
+      for (int d = 0; d < kPanCtas; ++d) {
+        st_remote(&crow[sb][q][lane], d, bv);
+        if (lane == 0) st_remote(&cmag[sb][q], d, make_int2(top, brow));
+      }
+    }
+    cluster_barrier();
+    const int2 y = cmag[sb][lane & (kPanCtas - 1)];
+    const int best = __reduce_max_sync(0xffffffffu, y.x);
+    const int qtop = __ffs(__ballot_sync(0xffffffffu, y.x == best)) - 1;
+    if (q == qtop && warp == wtop) live &= ~(1u << br);
+    if (threadIdx.x == 0) win[j] = best >= 0 ? cmag[sb][qtop].y : -1;  // -1: no candidate left, or none finite
+    const float2 pr = crow[sb][qtop][lane];
+    const float2 pj = make_float2(__shfl_sync(0xffffffffu, pr.x, j), __shfl_sync(0xffffffffu, pr.y, j));
+    const float pm = pj.x * pj.x + pj.y * pj.y;
+    const float rm = pm > 0.f ? 1.f / pm : 0.f;
+    // the pivot row over its pivot
+    const float2 g = make_float2((pr.x * pj.x + pr.y * pj.y) * rm, (pr.y * pj.x - pr.x * pj.y) * rm);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float fx = __shfl_sync(0xffffffffu, v[r].x, j), fy = __shfl_sync(0xffffffffu, v[r].y, j);
+      if (lane > j) {
+        v[r].x = fmaf(-fx, g.x, fmaf(fy, g.y, v[r].x));
+        v[r].y = fmaf(-fx, g.y, fmaf(-fy, g.x, v[r].y));
+      }
+    }
+  }
+  __syncthreads();
+  if (!last) {
+    if (q == 0 && threadIdx.x < kNB) out[c * kNB + threadIdx.x] = win[threadIdx.x];
+    cluster_barrier();  // nobody leaves while another may still write to it
+    return;
+  }
+  // P = inv of the chosen block, row r of it in warp r & 3 of CTA r / 4
+  const int pr = 4 * q + warp;  // warps 0 .. 3
+  double2 z = make_double2(0.0, 0.0);
+  if (warp < 4) z = A[(size_t)(win[pr] >= 0 ? win[pr] : k0 + pr) * np + k0 + lane];
+  auto publish = [&](int k) {
+    const double2 d = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+    double2 pinv;
+    if (!recip(d, pinv) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
+    z = lane == k ? pinv : cmul(z, pinv);
+#pragma unroll
+    for (int d8 = 0; d8 < kPanCtas; ++d8) st_remote(&rowb[k & 1][lane], d8, z);
+  };
+  if (q == 0 && warp == 0) publish(0);
+  cluster_barrier();
+  for (int k = 0; k < kNB; ++k) {
+    if (warp < 4) {
+      if (pr != k) {
+        const double2 rb = rowb[k & 1][lane];
+        const double2 f = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+        const double2 o = lane == k ? make_double2(0.0, 0.0) : z;
+        z = make_double2(fma(-f.x, rb.x, fma(f.y, rb.y, o.x)), fma(-f.x, rb.y, fma(-f.y, rb.x, o.y)));
+      }
+      if (pr == k + 1) publish(k + 1);
+    }
+    cluster_barrier();
+  }
+  if (warp < 4) {
+    Pbuf[pr * kNB + lane] = z;
+    // digits of rows 2 pr = [Re | -Im] and 2 pr + 1 = [Im | Re], two columns per even lane
+    const unsigned m = __reduce_max_sync(0xffffffffu, max(mag_hi(z.x), mag_hi(z.y)));
+    const int be = row_biased(m);
+    if (m >= 0x7ff00000u && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
+    if (lane == 0) pexp[pr] = be - 1022;
+    const long long yr = digit_word(z.x, be), yi = digit_word(z.y, be);
+    const long long yr1 = __shfl_down_sync(0xffffffffu, yr, 1), yi1 = __shfl_down_sync(0xffffffffu, yi, 1);
+    if ((lane & 1) == 0) {
+      const long long y[8] = {yr, yr1, yi, yi1, 0, 0, 0, 0};
+      const int o_re = core_off(2 * pr, lane), o_im = core_off(2 * pr, 32 + lane);
+      put_digits(y, [&](int s, uint4 w) {
+        __nv_bfloat16* d = pimg + s * 64 * kK;
+        *reinterpret_cast<uint32_t*>(d + o_re) = w.x;
+        *reinterpret_cast<uint32_t*>(d + o_im) = w.y ^ 0x80008000u;
+        *reinterpret_cast<uint32_t*>(d + o_re + 8) = w.y;
+        *reinterpret_cast<uint32_t*>(d + o_im + 8) = w.x;
+      });
+    }
+  }
+  if (q == 0 && warp == 4) {
+    // place k0 + lane takes row w; a winner from outside the block leaves its
+    // place to a row of the block that was not chosen (the t-th such place gets
+    // the t-th such row)
+    const int w = win[lane] >= 0 ? win[lane] : k0 + lane;
+    const bool inside = w >= k0 && w < k0 + kNB;
+    if (win[lane] < 0 && k0 + lane < n && status) atomicCAS(status, 0, DS_SINGULAR);  // fewer candidates than columns
+    const unsigned chosen = __reduce_or_sync(0xffffffffu, inside ? 1u << (w - k0) : 0u);
+    const unsigned outs = __ballot_sync(0xffffffffu, !inside);
+    const int t = __popc(outs & ((1u << lane) - 1u));
+    unsigned left = ~chosen;
+    for (int u = 0; u < t; ++u) left &= left - 1;  // drop the t lowest
+    const int from = k0 + __ffs(left) - 1;
+    const int pw = rowperm[w], pf = inside ? 0 : rowperm[from];
+    __syncwarp();
+    rowperm[k0 + lane] = pw;
+    sw->win[lane] = w;
+    if (!inside) {
+      rowperm[w] = pf;
+      sw->to[t] = w;
+      sw->from[t] = from;
+    }
+    if (lane == 0) sw->moved = __popc(outs);
+  }
+  cluster_barrier();  // nobody leaves while another may still write to it
+}
+
+int launch_panel(const double2* A, int np, int n, int k0, const int* in, int count, int* out, bool last, double2* pbuf,
+                 __nv_bfloat16* pimg, int* pexp, RowSwaps* sw, int* rowperm, int* status, cudaStream_t s) {
+  // 256 R rows per cluster: as few as hold the candidates, at most 2048
+  auto go = [&](auto r) {
+    constexpr int R = decltype(r)::value;
+    const int clusters = ceil_div(count, 256 * R);
+    gj64_panel_kernel<R><<<clusters * kPanCtas, 32 * kPanWarps, 0, s>>>(A, np, n, k0, in, count, out, last, pbuf, pimg,
+                                                                        pexp, sw, rowperm, status);
+  };
+  if (count <= 256) go(std::integral_constant<int, 1>{});
+  else if (count <= 512) go(std::integral_constant<int, 2>{});
+  else if (count <= 1024) go(std::integral_constant<int, 4>{});
+  else if (count <= 1536) go(std::integral_constant<int, 6>{});
+  else go(std::integral_constant<int, 8>{});
+  NED_LAUNCH_CHECK("gj64_panel_kernel");
+  return NEDMFT_OK;
+}
+
+// The inversion works on A 2^-e, e the exponent of max |Re|, |Im| over A
+// (exact scaling): its pivot thresholds are then relative and the FP32 pivot
+// choice stays in range.  amax holds the bits of that maximum (non-negative
+// doubles order like their bit patterns), set by amax_kernel after a clear.
+__device__ __forceinline__ int amax_exponent(const unsigned long long* amax) {
+  const double m = __longlong_as_double((long long)*amax);
+  int e = 0;
+  if (m > 0.0 && m <= 1.7976931348623157e308) frexp(m, &e);
+  return e;
+}
+
+__global__ void amax_kernel(const double2* __restrict__ a, size_t total, unsigned long long* __restrict__ amax) {
+  double m = 0.0;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+    const double2 z = a[e];
+    m = fmax(m, fmax(fabs(z.x), fabs(z.y)));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(amax, (unsigned long long)__double_as_longlong(m));
+}
+
+// The scaled copy, padded with the identity, and the identity row permutation.
+__global__ void pad_identity_kernel(const double2* __restrict__ a, int n, double2* __restrict__ ap, int np,
+                                    const unsigned long long* __restrict__ amax, int* __restrict__ rowperm) {
+  const int sh = -amax_exponent(amax);
+  const int i = blockIdx.x;
+  for (int j = blockIdx.y * blockDim.x + threadIdx.x; j < np; j += gridDim.y * blockDim.x) {
+    double2 v = make_double2(i == j ? 1.0 : 0.0, 0.0);
+    if (i < n && j < n) {
+      const double2 z = a[(size_t)i * n + j];
+      v = make_double2(scalbn(z.x, sh), scalbn(z.y, sh));
+    }
+    ap[(size_t)i * np + j] = v;
+    if (i == 0) rowperm[j] = j;
+  }
+}
+
+// y = the inverse of A from x = (P A 2^-e)^-1: column c of x is column
+// rowperm[c] of A^-1, and inv(A 2^-e) = 2^e inv(A)
+__global__ void unpermute_kernel(const double2* __restrict__ x, int np, int n, const int* __restrict__ rowperm,
+                                 double2* __restrict__ y, const unsigned long long* __restrict__ amax) {
+  const int sh = -amax_exponent(amax);
+  const int i = blockIdx.x;
+  for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < n; c += gridDim.y * blockDim.x) {
+    const double2 z = x[(size_t)i * np + c];
+    y[(size_t)i * n + rowperm[c]] = make_double2(scalbn(z.x, sh), scalbn(z.y, sh));
+  }
+}
+
+// Second stream (highest priority) and two events per device and host
+// thread for the look-ahead below, created on first use and kept.
+struct LookAhead {
+  cudaStream_t side = nullptr;
+  cudaEvent_t panel = nullptr, chain = nullptr;
+};
+
+int look_ahead(LookAhead** out) {
+  constexpr int kMaxDev = 64;
+  thread_local LookAhead la[kMaxDev];
+  int dev = 0;
+  NED_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDev) return set_error(NEDMFT_ECUDA, "pivot_inverse: device %d out of range", dev);
+  LookAhead& l = la[dev];
+  if (!l.side) {
+    int lo = 0, hi = 0;
+    NED_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    NED_CUDA(cudaEventCreateWithFlags(&l.panel, cudaEventDisableTiming));
+    NED_CUDA(cudaEventCreateWithFlags(&l.chain, cudaEventDisableTiming));
+    NED_CUDA(cudaStreamCreateWithPriority(&l.side, cudaStreamNonBlocking, hi));
+  }
+  *out = &l;
+  return NEDMFT_OK;
+}
+
+struct PivLayout {
+  size_t a, gj, cand, sw, perm, amax, total;
+};
+PivLayout piv_layout(int n) {
+  PivLayout L;
+  const int np = ceil_div(n, 128) * 128;
+  L.a = align256(sizeof(double2) * (size_t)np * np);
+  L.gj = gj64_layout(np, 1).total;
+  L.cand = align256(sizeof(int) * (size_t)ceil_div(n, 2048) * kNB);
+  L.sw = align256(sizeof(RowSwaps));
+  L.perm = align256(sizeof(int) * (size_t)np);
+  L.amax = align256(8);
+  L.total = L.a + L.gj + 2 * L.cand + L.sw + L.perm + L.amax;
+  return L;
+}
+
+}  // namespace
+
+size_t pivot_inverse_workspace(int n) { return piv_layout(n).total; }
+
+// Creates this host thread's look-ahead stream and events on the current
+// device and sets the kernels' shared-memory limits: for callers that are
+// about to capture pivot_inverse into a CUDA graph.
+int pivot_inverse_prepare() {
+  LookAhead* la = nullptr;
+  int rc = look_ahead(&la), sms = 0;
+  if (!rc) rc = device_sm_count(&sms);
+  if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_rpanel_kernel), RSmem::kBytes);
+  if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_update_kernel), USmem::kBytes);
+  return rc;
+}
+
+// In-place inverse of one n x n matrix with partial pivoting (the impurity
+// step), blocked Gauss-Jordan in steps of 32 columns.  Every step's pivot choice
+// and pivot-block inverse depend only on its 32 panel columns, so they run one
+// step ahead on the second stream: there the update kernel brings the next
+// panel's two column tiles up to date, then the panel kernel of step k + 1 runs,
+// while step k updates the rest of the matrix on the caller's stream.  The R
+// panel of step k + 1 waits for both and moves the rows.  The serial path of a
+// step is R panel, window, pivot choice and block inverse.
+int pivot_inverse(double2* a, int n, void* ws, cudaStream_t st, int* status) {
+  const int np = ceil_div(n, 128) * 128;
+  const PivLayout L = piv_layout(n);
+  const Gj64Layout G = gj64_layout(np, 1);
+  char* p = static_cast<char*>(ws);
+  double2* ap = reinterpret_cast<double2*>(p); p += L.a;
+  double2* pbuf = reinterpret_cast<double2*>(p); p += G.p;
+  __nv_bfloat16* pimg = reinterpret_cast<__nv_bfloat16*>(p); p += G.pi;
+  int* pexp = reinterpret_cast<int*>(p); p += G.pe;
+  __nv_bfloat16* cimg = reinterpret_cast<__nv_bfloat16*>(p); p += G.c;
+  __nv_bfloat16* rimg = reinterpret_cast<__nv_bfloat16*>(p); p += G.r;
+  int* cexp = reinterpret_cast<int*>(p); p += G.ce;
+  int* rexp = reinterpret_cast<int*>(p); p += G.re;
+  int* cand[2];
+  cand[0] = reinterpret_cast<int*>(p); p += L.cand;
+  cand[1] = reinterpret_cast<int*>(p); p += L.cand;
+  RowSwaps* sw = reinterpret_cast<RowSwaps*>(p); p += L.sw;
+  int* rowperm = reinterpret_cast<int*>(p); p += L.perm;
+  unsigned long long* amax = reinterpret_cast<unsigned long long*>(p);
+  LookAhead* la = nullptr;
+  int rc = look_ahead(&la);
+  if (!rc) rc = pivot_inverse_prepare();
+  CUtensorMap map;
+  if (!rc) rc = encode_f64_boxes(&map, ap, np, np);
+  int sms = 0;
+  if (!rc) rc = device_sm_count(&sms);
+  if (rc) return rc;
+  NED_CUDA(cudaMemsetAsync(amax, 0, sizeof(unsigned long long), st));
+  const size_t nn = (size_t)n * n;
+  amax_kernel<<<(int)((nn + 255) / 256 < 152 * 4 ? (nn + 255) / 256 : 152 * 4), 256, 0, st>>>(a, nn, amax);
+  NED_LAUNCH_CHECK("amax_kernel");
+  pad_identity_kernel<<<dim3(np, ceil_div(np, 1024)), 256, 0, st>>>(a, n, ap, np, amax, rowperm);
+  NED_LAUNCH_CHECK("pad_identity_kernel");
+  const int mtiles = np / 128, ntn = ceil_div(n, kTn);
+  auto update = [&](int k0, int tiles, int jskip, int nskip, int ctas, cudaStream_t s) -> int {
+    const int total = mtiles * tiles;
+    if (total <= 0) return NEDMFT_OK;
+    gj64_update_kernel<<<total < ctas ? total : ctas, 64 + 32 * kEpiW, USmem::kBytes, s>>>(
+        map, np, mtiles, tiles, total, k0, jskip, nskip, cimg, cexp, rimg, rexp, status);
+    NED_LAUNCH_CHECK("gj64_update_kernel");
+    return NEDMFT_OK;
+  };
+  auto panel = [&](int k0, cudaStream_t s) -> int {
+    const int* in = nullptr;
+    int count = n - k0, buf = 0;
+    while (count > 2048) {  // rounds of 2048 rows until one cluster holds the candidates
+      if (int e = launch_panel(ap, np, n, k0, in, count, cand[buf], false, pbuf, pimg, pexp, sw, rowperm, status, s))
+        return e;
+      in = cand[buf];
+      count = ceil_div(count, 2048) * kNB;
+      buf ^= 1;
+    }
+    return launch_panel(ap, np, n, k0, in, count, nullptr, true, pbuf, pimg, pexp, sw, rowperm, status, s);
+  };
+  constexpr int kFreeSms = 16;  // left to the window's and the panel's CTAs while the update runs
+  if ((rc = panel(0, st))) return rc;
+  for (int k0 = 0; k0 < n; k0 += kNB) {
+    gj64_rpanel_kernel<<<dim3(2 * mtiles, 1), 512, RSmem::kBytes, st>>>(ap, np, mtiles, k0, pbuf, pimg, pexp, rimg,
+                                                                        rexp, sw, cimg, cexp, status);
+    NED_LAUNCH_CHECK("gj64_rpanel_kernel");
+    const int k1 = k0 + kNB;
+    if (k1 >= n) {
+      if ((rc = update(k0, ntn, ntn, 0, sms, st))) return rc;
+      break;
+    }
+    const int w0 = k1 / kTn, wn = ntn - w0 < 2 ? ntn - w0 : 2;  // the next panel's column tiles
+    NED_CUDA(cudaEventRecord(la->panel, st));
+    NED_CUDA(cudaStreamWaitEvent(la->side, la->panel, 0));
+    if ((rc = update(k0, wn, 0, w0, sms, la->side))) return rc;
+    if ((rc = panel(k1, la->side))) return rc;
+    NED_CUDA(cudaEventRecord(la->chain, la->side));
+    if ((rc = update(k0, ntn - wn, w0, wn, sms > 2 * kFreeSms ? sms - kFreeSms : sms, st))) return rc;
+    NED_CUDA(cudaStreamWaitEvent(st, la->chain, 0));
+  }
+  unpermute_kernel<<<dim3(n, ceil_div(n, 1024)), 256, 0, st>>>(ap, np, n, rowperm, a, amax);
+  NED_LAUNCH_CHECK("unpermute_kernel");
   return NEDMFT_OK;
 }
 

@@ -42,25 +42,47 @@ __global__ void imp_build_kernel(ContourDev c, ModelDev m, const double2* __rest
 }
 
 // sigma_new = W^-1 [-w1 D + w1 (1 - w1) D X_h D] W^-1 with X_h = inv(A_h); if
-// g is given, g = A0 - W sigma_new W (= inv(G_imp)).
-__global__ void imp_sigma_kernel(ContourDev c, ModelDev m, const double2* __restrict__ xh,
-                                 const double2* __restrict__ a0, double2* __restrict__ sigma_new,
-                                 double2* __restrict__ g) {
-  const int n = c.n;
-  const size_t total = (size_t)n * n;
+// g is given, g = A0 - W sigma_new W (= inv(G_imp)).  16 rows of 256 columns per
+// CTA: the factors d_i / W_i and d_{j+1} / W_j are formed once per row and
+// column, so an entry costs two complex products (240 us at N_c = 1500 when
+// every entry formed and divided by W_i W_j in FP64).
+__global__ void __launch_bounds__(256) imp_sigma_kernel(ContourDev c, ModelDev m, const double2* __restrict__ xh,
+                                                        const double2* __restrict__ a0,
+                                                        double2* __restrict__ sigma_new, double2* __restrict__ g) {
+  constexpr int kRowsPer = 16;
+  __shared__ double2 fi[kRowsPer];
+  const int n = c.n, i0 = blockIdx.y * kRowsPer;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int jc = j < n ? j : 0, jn = jc + 1 == n ? 0 : jc + 1;  // the row of D whose entry lies in column j
+  auto over = [](double2 a, double2 w) {
+    const double m2 = w.x * w.x + w.y * w.y;
+    return cmul(a, make_double2(w.x / m2, -w.y / m2));
+  };
   const double w1 = m.w1;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / n), j = (int)(e % n);
-    const int ip = i == 0 ? n - 1 : i - 1;  // the column of row i's entry of D
-    const int jn = j + 1 == n ? 0 : j + 1;  // the row of D whose entry lies in column j
-    const double2 di = d_entry(c, m.U, i), dj = d_entry(c, m.U, jn);
-    double2 v = cmul(cmul(di, xh[(size_t)ip * n + jn]), dj);
-    v = make_double2(w1 * (1.0 - w1) * v.x, w1 * (1.0 - w1) * v.y);
-    if (j == ip) v = make_double2(v.x - w1 * di.x, v.y - w1 * di.y);
-    if (g) g[e] = csub(a0[e], v);
-    const double2 ww = cmul(weight(c, i), weight(c, j));
-    const double m2 = ww.x * ww.x + ww.y * ww.y;
-    sigma_new[e] = cmul(v, make_double2(ww.x / m2, -ww.y / m2));
+  const double2 wj = weight(c, jc), dj = d_entry(c, m.U, jn);
+  double2 fj = over(dj, wj);
+  fj = make_double2(w1 * (1.0 - w1) * fj.x, w1 * (1.0 - w1) * fj.y);
+  if (threadIdx.x < kRowsPer && i0 + threadIdx.x < n)
+    fi[threadIdx.x] = over(d_entry(c, m.U, i0 + threadIdx.x), weight(c, i0 + threadIdx.x));
+  __syncthreads();
+  if (j >= n) return;
+  for (int r = 0; r < kRowsPer && i0 + r < n; ++r) {
+    const int i = i0 + r, ip = i == 0 ? n - 1 : i - 1;  // the column of row i's entry of D
+    const size_t e = (size_t)i * n + j;
+    const double2 x = xh[(size_t)ip * n + jn];
+    double2 s = cmul(cmul(fi[r], x), fj);
+    if (j == ip) {
+      const double2 d = over(fi[r], wj);
+      s = make_double2(s.x - w1 * d.x, s.y - w1 * d.y);
+    }
+    sigma_new[e] = s;
+    if (g) {
+      const double2 di = d_entry(c, m.U, i);
+      double2 v = cmul(cmul(di, x), dj);
+      v = make_double2(w1 * (1.0 - w1) * v.x, w1 * (1.0 - w1) * v.y);
+      if (j == ip) v = make_double2(v.x - w1 * di.x, v.y - w1 * di.y);
+      g[e] = csub(a0[e], v);
+    }
   }
 }
 
@@ -105,7 +127,8 @@ extern "C" int nedmft_impurity_update(const nedmft_contour* c, const nedmft_mode
   imp_build_kernel<<<bx, 256, 0, st>>>(cd, md, reinterpret_cast<const double2*>(sigma_d), a0, ah);
   NED_LAUNCH_CHECK("imp_build_kernel");
   if ((rc = pivot_inverse(ah, n, pws, st, status))) return rc;  // ah = X_h = inv(A_h)
-  imp_sigma_kernel<<<bx, 256, 0, st>>>(cd, md, ah, a0, reinterpret_cast<double2*>(sigma_new_d), gimp_d ? g : nullptr);
+  imp_sigma_kernel<<<dim3(ceil_div(n, 256), ceil_div(n, 16)), 256, 0, st>>>(
+      cd, md, ah, a0, reinterpret_cast<double2*>(sigma_new_d), gimp_d ? g : nullptr);
   NED_LAUNCH_CHECK("imp_sigma_kernel");
   if (gimp_d) {
     if ((rc = pivot_inverse(g, n, pws, st, status))) return rc;  // G_imp = inv(A0 - W sigma_new W)

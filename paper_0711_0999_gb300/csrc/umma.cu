@@ -2318,8 +2318,7 @@ int umma_set_wait_ns(uint64_t ns, cudaStream_t st) {
   NED_CUDA(cudaMemcpyToSymbolAsync(umma::g_wait_ns, &ns, sizeof(ns), 0, cudaMemcpyHostToDevice, st));
   NED_CUDA(cudaStreamSynchronize(st));
   if (int rc = gj64_set_wait_ns(ns, st)) return rc;
-  if (int rc = mlp_set_wait_ns(ns, st)) return rc;
-  return oz64_set_wait_ns(ns, st);
+  return mlp_set_wait_ns(ns, st);
 }
 
 }  // namespace nedmft
