@@ -21,8 +21,6 @@
 // One MMA per digit a of the left operand takes all its partners b = 0 .. 6-a
 // at once: the right operand's digits lie back to back in shared memory, and
 // orders a .. 6 back to back in TMEM.
-#include <type_traits>
-
 #include "lattice.cuh"
 #include "umma_core.cuh"
 
@@ -797,154 +795,165 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
 
 namespace {
 
-constexpr int kPanCtas = 8;   // CTAs of a panel cluster
-constexpr int kPanWarps = 32;
+constexpr int kPanCtas = 8;     // CTAs of a panel cluster
+constexpr int kPanRows = 2048;  // most rows of one: 256 threads, a row each
 
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, double2 v) {
-  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "d"(v.x), "d"(v.y) : "memory");
-}
-__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "f"(v.x), "f"(v.y) : "memory");
-}
-__device__ __forceinline__ void st_remote(const void* p, uint32_t rank, int2 v) {
-  asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(cluster_addr(p, rank)), "r"(v.x), "r"(v.y) : "memory");
+// 16 bytes into CTA `rank`'s copy of *p, counted on its copy of `bar`
+__device__ __forceinline__ void st_async(const void* p, const uint64_t* bar, uint32_t rank, uint4 v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(
+                   cluster_addr(p, rank)),
+               "r"(cluster_addr(bar, rank)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
 }
 
+struct PanSmem {
+  float4 row[kNB][kPanCtas][kNB / 2];  // per step: the CTAs' candidate rows, from the step's column on
+  uint4 cand[kNB][kPanCtas];           // their |entry|^2 as ordered bits, and row
+  double2 prow[kNB][kNB];              // the block inverse's pivot rows, divided by their pivots
+  uint64_t bar[kNB], pbar[kNB];
+  int wtop[2][8];
+  int win[kNB];
+  int abort;
+};
+
 // Pivot choice for the 32 columns from k0 on and, in the last round, the block's
-// inverse.  A cluster of eight CTAs runs partial pivoting in FP32 on up to 256 R
-// candidate rows (rows k0 + i, or in[i]), a warp per R rows, lane = column: per
-// column each warp's largest entry sits in one lane, a warp maximum over the 32
-// warps' gives the CTA's, whose row goes to all eight CTAs' shared memory, and
-// after one cluster barrier every warp picks the largest of the eight and
-// eliminates its own rows with it.  Rows do not move and the column loop is not
-// unrolled (the unrolled form with a row per thread, 200 KB of code used once,
-// spent its time fetching it: 55 us per round of 256 rows).
+// inverse, on a cluster of eight CTAs.
+// Choice: partial pivoting in FP32 on up to 2048 candidate rows (rows k0 + i, or
+// in[i]), a thread per row with its entries in registers.  Per column: a warp
+// maximum, one over the warps, then the CTA's row goes to all eight CTAs'
+// shared memory (st.async, counted on the receivers' barrier of that step), every
+// thread picks the largest of the eight and eliminates its row, writing the
+// result one register down, so that the column in hand is always register 0 and
+// the loop needs no unrolling (unrolled with a row per thread, 200 KB of code
+// used once, the fetching alone bound it: 55 us per round of 256 rows; a warp
+// per R rows with two shuffles per row and a cluster barrier per column, 63 us
+// for R = 1 with the inverse, 88 for R = 6).
 // Last round: P = inv of the chosen rows' block in FP64, four rows per CTA, a
-// warp per row, the next pivot row first; its digits (the B operand of
-// gj64_rpanel_kernel); the row exchanges; the row permutation.  Both parts are
-// latency bound: 32 cluster barriers each.
-template <int R>
-__global__ void __cluster_dims__(kPanCtas, 1, 1) __launch_bounds__(32 * kPanWarps, 1)
+// warp per row, the next pivot row first and sent the same way; its digits (the
+// B operand of gj64_rpanel_kernel); the row exchanges; the row permutation.
+// Every step has buffers and a barrier of its own, so nothing waits for a slot.
+// Both parts are latency bound, 32 exchanges each.
+__global__ void __cluster_dims__(kPanCtas, 1, 1) __launch_bounds__(256, 1)
     gj64_panel_kernel(const double2* __restrict__ A, int np, int n, int k0, const int* __restrict__ in, int count,
                       int* __restrict__ out, int last, double2* __restrict__ Pbuf, __nv_bfloat16* __restrict__ pimg,
                       int* __restrict__ pexp, RowSwaps* __restrict__ sw, int* __restrict__ rowperm, int* status) {
-  __shared__ int cand[2][kPanWarps];                      // the warps' largest |entry|^2, as ordered bits
-  __shared__ __align__(16) float2 crow[2][kPanCtas][32];  // the CTAs' candidate rows
-  __shared__ __align__(8) int2 cmag[2][kPanCtas];         // their |entry|^2 and row
-  __shared__ __align__(16) double2 rowb[2][32];
-  __shared__ int win[kNB];
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  PanSmem& sm = *reinterpret_cast<PanSmem*>(smem_raw);
+  volatile int* abort_flag = &sm.abort;
   const int q = (int)cluster_ctarank(), c = blockIdx.x / kPanCtas;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int base = c * 256 * R, here = min(count - base, 256 * R);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nwarp = blockDim.x >> 5;
+  const int per = kPanCtas * blockDim.x, base = c * per, here = min(count - base, per);
   const int ncol = min(kNB, n - k0), steps = min(ncol, here);
-  float2 v[R];
-  int row[R];
-  unsigned live = 0;
+  if (t < kNB) {
+    mbar_init(&sm.bar[t], 1);
+    mbar_init(&sm.pbar[t], 1);
+    fence_barrier_init();
+    mbar_arrive_expect_tx(&sm.bar[t], kPanCtas * (kNB * 8 + 16));
+    mbar_arrive_expect_tx(&sm.pbar[t], kNB * 16);
+    sm.win[t] = -1;
+  }
+  if (t == 0) sm.abort = 0;
+  const int i = base + q * (int)blockDim.x + t;
+  const int row = i < base + here ? (in ? in[i] : k0 + i) : -1;
+  float2 v[kNB];
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int i = base + r * 256 + q * 32 + warp;
-    row[r] = i < base + here ? (in ? in[i] : k0 + i) : -1;
-    v[r] = make_float2(0.f, 0.f);
-    if (row[r] >= 0) {
-      live |= 1u << r;
-      if (lane < ncol) {
-        const double2 z = A[(size_t)row[r] * np + k0 + lane];
-        v[r] = make_float2((float)z.x, (float)z.y);
-      }
+  for (int e = 0; e < kNB; ++e) {
+    v[e] = make_float2(0.f, 0.f);
+    if (row >= 0 && e < ncol) {
+      const double2 z = A[(size_t)row * np + k0 + e];
+      v[e] = make_float2((float)z.x, (float)z.y);
     }
   }
-  if (threadIdx.x < kNB) win[threadIdx.x] = -1;
-  cluster_barrier();  // every CTA runs before another writes its shared memory
+  bool live = row >= 0, ok = true;
+  __syncthreads();
+  cluster_barrier();  // every CTA's barriers are set before another counts on them
+#pragma unroll 1
   for (int j = 0; j < steps; ++j) {
-    const int sb = j & 1;
-    float bm = -1.f;
-    float2 bv = make_float2(0.f, 0.f);
-    int br = 0, brow = -1;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {  // in lane j: this warp's rows' entries of column j
-      const float m = (live >> r) & 1 ? v[r].x * v[r].x + v[r].y * v[r].y : -1.f;
-      if (m > bm) {
-        bm = m;
-        br = r;
-      }
-    }
-    bm = __shfl_sync(0xffffffffu, bm, j);
-    br = __shfl_sync(0xffffffffu, br, j);
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-      if (r == br) {
-        bv = v[r];
-        brow = row[r];
-      }
-    if (lane == 0) cand[sb][warp] = __float_as_int(bm);  // -1 orders below every magnitude
+    // largest |entry|^2, as ordered bits (-1 below every magnitude; a NaN is never chosen)
+    const float m = v[0].x * v[0].x + v[0].y * v[0].y;
+    const int key = live && m >= 0.f ? __float_as_int(m) : -1;
+    const int wk = __reduce_max_sync(0xffffffffu, key);
+    if (lane == 0) sm.wtop[j & 1][warp] = wk;
     __syncthreads();
-    const int x = cand[sb][lane];
+    const int x = lane < nwarp ? sm.wtop[j & 1][lane] : -1;
     const int top = __reduce_max_sync(0xffffffffu, x);
     const int wtop = __ffs(__ballot_sync(0xffffffffu, x == top)) - 1;
     if (warp == wtop) {
+      const int src = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
+      float4* mine = sm.row[j][q];
+      if (lane == src) {
 #pragma unroll
-      for (int d = 0; d < kPanCtas; ++d) {
-        st_remote(&crow[sb][q][lane], d, bv);
-        if (lane == 0) st_remote(&cmag[sb][q], d, make_int2(top, brow));
+        for (int e = 0; e < kNB / 2; ++e) mine[e] = make_float4(v[2 * e].x, v[2 * e].y, v[2 * e + 1].x, v[2 * e + 1].y);
       }
+      const int srow = __shfl_sync(0xffffffffu, row, src);
+      __syncwarp();
+      // lane: CTA lane / 4, a quarter of the row (its own CTA's copy is rewritten with the same values)
+      const uint32_t d = lane >> 2;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float4 z = mine[4 * (lane & 3) + e];
+        st_async(&mine[4 * (lane & 3) + e], &sm.bar[j], d,
+                 make_uint4(__float_as_uint(z.x), __float_as_uint(z.y), __float_as_uint(z.z), __float_as_uint(z.w)));
+      }
+      if (lane < kPanCtas)
+        st_async(&sm.cand[j][q], &sm.bar[j], lane, make_uint4((uint32_t)top, (uint32_t)srow, 0u, 0u));
     }
-    cluster_barrier();
-    const int2 y = cmag[sb][lane & (kPanCtas - 1)];
-    const int best = __reduce_max_sync(0xffffffffu, y.x);
-    const int qtop = __ffs(__ballot_sync(0xffffffffu, y.x == best)) - 1;
-    if (q == qtop && warp == wtop) live &= ~(1u << br);
-    if (threadIdx.x == 0) win[j] = best >= 0 ? cmag[sb][qtop].y : -1;  // -1: no candidate left, or none finite
-    const float2 pr = crow[sb][qtop][lane];
-    const float2 pj = make_float2(__shfl_sync(0xffffffffu, pr.x, j), __shfl_sync(0xffffffffu, pr.y, j));
-    const float pm = pj.x * pj.x + pj.y * pj.y;
+    ok = mbar_wait(&sm.bar[j], 0, abort_flag);
+    if (!__syncthreads_and(ok)) {
+      ok = false;
+      break;
+    }
+    const uint4 y = sm.cand[j][lane & (kPanCtas - 1)];
+    const int best = __reduce_max_sync(0xffffffffu, (int)y.x);
+    const int qtop = __ffs(__ballot_sync(0xffffffffu, (int)y.x == best)) - 1;
+    const int wrow = (int)sm.cand[j][qtop].y;
+    if (t == 0) sm.win[j] = best >= 0 ? wrow : -1;  // -1: no candidate left, or none finite
+    if (best >= 0 && row == wrow) live = false;
+    const float4* pr = sm.row[j][qtop];
+    const float4 p0 = pr[0];
+    const float pm = p0.x * p0.x + p0.y * p0.y;
     const float rm = pm > 0.f ? 1.f / pm : 0.f;
-    // the pivot row over its pivot
-    const float2 g = make_float2((pr.x * pj.x + pr.y * pj.y) * rm, (pr.y * pj.x - pr.x * pj.y) * rm);
+    const float2 f = make_float2((v[0].x * p0.x + v[0].y * p0.y) * rm, (v[0].y * p0.x - v[0].x * p0.y) * rm);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const float fx = __shfl_sync(0xffffffffu, v[r].x, j), fy = __shfl_sync(0xffffffffu, v[r].y, j);
-      if (lane > j) {
-        v[r].x = fmaf(-fx, g.x, fmaf(fy, g.y, v[r].x));
-        v[r].y = fmaf(-fx, g.y, fmaf(-fy, g.x, v[r].y));
-      }
+    for (int e = 0; e < kNB / 2; ++e) {
+      const float4 z = e == 0 ? p0 : pr[e];
+      if (e > 0) v[2 * e - 1] = make_float2(fmaf(-f.x, z.x, fmaf(f.y, z.y, v[2 * e].x)),
+                                            fmaf(-f.x, z.y, fmaf(-f.y, z.x, v[2 * e].y)));
+      v[2 * e] = make_float2(fmaf(-f.x, z.z, fmaf(f.y, z.w, v[2 * e + 1].x)),
+                             fmaf(-f.x, z.w, fmaf(-f.y, z.z, v[2 * e + 1].y)));
     }
+    v[kNB - 1] = make_float2(0.f, 0.f);
   }
   __syncthreads();
   if (!last) {
-    if (q == 0 && threadIdx.x < kNB) out[c * kNB + threadIdx.x] = win[threadIdx.x];
-    cluster_barrier();  // nobody leaves while another may still write to it
-    return;
-  }
-  // P = inv of the chosen block, row r of it in warp r & 3 of CTA r / 4
-  const int pr = 4 * q + warp;  // warps 0 .. 3
-  double2 z = make_double2(0.0, 0.0);
-  if (warp < 4) z = A[(size_t)(win[pr] >= 0 ? win[pr] : k0 + pr) * np + k0 + lane];
-  auto publish = [&](int k) {
-    const double2 d = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
-    double2 pinv;
-    if (!recip(d, pinv) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
-    z = lane == k ? pinv : cmul(z, pinv);
+    if (q == 0 && t < kNB) out[c * kNB + t] = sm.win[t];
+  } else if (warp < 4) {
+    // P = inv of the chosen block, row r of it in warp r & 3 of CTA r / 4
+    const int pr = 4 * q + warp;
+    double2 z = A[(size_t)(sm.win[pr] >= 0 ? sm.win[pr] : k0 + pr) * np + k0 + lane];
+    auto publish = [&](int k) {
+      const double2 d = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+      double2 pinv;
+      if (!recip(d, pinv) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
+      z = lane == k ? pinv : cmul(z, pinv);
+      const uint4 w = make_uint4((uint32_t)__double2loint(z.x), (uint32_t)__double2hiint(z.x),
+                                 (uint32_t)__double2loint(z.y), (uint32_t)__double2hiint(z.y));
 #pragma unroll
-    for (int d8 = 0; d8 < kPanCtas; ++d8) st_remote(&rowb[k & 1][lane], d8, z);
-  };
-  if (q == 0 && warp == 0) publish(0);
-  cluster_barrier();
-  for (int k = 0; k < kNB; ++k) {
-    if (warp < 4) {
-      if (pr != k) {
-        const double2 rb = rowb[k & 1][lane];
-        const double2 f = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
-        const double2 o = lane == k ? make_double2(0.0, 0.0) : z;
-        z = make_double2(fma(-f.x, rb.x, fma(f.y, rb.y, o.x)), fma(-f.x, rb.y, fma(-f.y, rb.x, o.y)));
-      }
+      for (uint32_t d8 = 0; d8 < (uint32_t)kPanCtas; ++d8) st_async(&sm.prow[k][lane], &sm.pbar[k], d8, w);
+    };
+    if (pr == 0) publish(0);
+    for (int k = 0; k < kNB; ++k) {
+      if (pr == k) continue;
+      if (!__all_sync(0xffffffffu, mbar_wait(&sm.pbar[k], 0, abort_flag))) break;
+      const double2 rb = sm.prow[k][lane];
+      const double2 f = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+      const double2 o = lane == k ? make_double2(0.0, 0.0) : z;
+      z = make_double2(fma(-f.x, rb.x, fma(f.y, rb.y, o.x)), fma(-f.x, rb.y, fma(-f.y, rb.x, o.y)));
       if (pr == k + 1) publish(k + 1);
     }
-    cluster_barrier();
-  }
-  if (warp < 4) {
     Pbuf[pr * kNB + lane] = z;
     // digits of rows 2 pr = [Re | -Im] and 2 pr + 1 = [Im | Re], two columns per even lane
     const unsigned m = __reduce_max_sync(0xffffffffu, max(mag_hi(z.x), mag_hi(z.y)));
@@ -964,48 +973,43 @@ __global__ void __cluster_dims__(kPanCtas, 1, 1) __launch_bounds__(32 * kPanWarp
         *reinterpret_cast<uint32_t*>(d + o_im + 8) = w.x;
       });
     }
-  }
-  if (q == 0 && warp == 4) {
-    // place k0 + lane takes row w; a winner from outside the block leaves its
-    // place to a row of the block that was not chosen (the t-th such place gets
-    // the t-th such row)
-    const int w = win[lane] >= 0 ? win[lane] : k0 + lane;
-    const bool inside = w >= k0 && w < k0 + kNB;
-    if (win[lane] < 0 && k0 + lane < n && status) atomicCAS(status, 0, DS_SINGULAR);  // fewer candidates than columns
-    const unsigned chosen = __reduce_or_sync(0xffffffffu, inside ? 1u << (w - k0) : 0u);
-    const unsigned outs = __ballot_sync(0xffffffffu, !inside);
-    const int t = __popc(outs & ((1u << lane) - 1u));
-    unsigned left = ~chosen;
-    for (int u = 0; u < t; ++u) left &= left - 1;  // drop the t lowest
-    const int from = k0 + __ffs(left) - 1;
-    const int pw = rowperm[w], pf = inside ? 0 : rowperm[from];
-    __syncwarp();
-    rowperm[k0 + lane] = pw;
-    sw->win[lane] = w;
-    if (!inside) {
-      rowperm[w] = pf;
-      sw->to[t] = w;
-      sw->from[t] = from;
+    if (pr == 0) {
+      // place k0 + lane takes row w; a winner from outside the block leaves its
+      // place to a row of the block that was not chosen (the t-th such place gets
+      // the t-th such row)
+      const int w = sm.win[lane] >= 0 ? sm.win[lane] : k0 + lane;
+      const bool inside = w >= k0 && w < k0 + kNB;
+      if (sm.win[lane] < 0 && k0 + lane < n && status) atomicCAS(status, 0, DS_SINGULAR);  // too few candidates
+      const unsigned chosen = __reduce_or_sync(0xffffffffu, inside ? 1u << (w - k0) : 0u);
+      const unsigned outs = __ballot_sync(0xffffffffu, !inside);
+      const int at = __popc(outs & ((1u << lane) - 1u));
+      unsigned left = ~chosen;
+      for (int u = 0; u < at; ++u) left &= left - 1;  // drop the lowest
+      const int from = k0 + __ffs(left) - 1;
+      const int pw = rowperm[w], pf = inside ? 0 : rowperm[from];
+      __syncwarp();
+      rowperm[k0 + lane] = pw;
+      sw->win[lane] = w;
+      if (!inside) {
+        rowperm[w] = pf;
+        sw->to[at] = w;
+        sw->from[at] = from;
+      }
+      if (lane == 0) sw->moved = __popc(outs);
     }
-    if (lane == 0) sw->moved = __popc(outs);
   }
+  __syncthreads();
+  if (t == 0 && sm.abort && status) atomicCAS(status, 0, DS_TIMEOUT);
   cluster_barrier();  // nobody leaves while another may still write to it
 }
 
 int launch_panel(const double2* A, int np, int n, int k0, const int* in, int count, int* out, bool last, double2* pbuf,
                  __nv_bfloat16* pimg, int* pexp, RowSwaps* sw, int* rowperm, int* status, cudaStream_t s) {
-  // 256 R rows per cluster: as few as hold the candidates, at most 2048
-  auto go = [&](auto r) {
-    constexpr int R = decltype(r)::value;
-    const int clusters = ceil_div(count, 256 * R);
-    gj64_panel_kernel<R><<<clusters * kPanCtas, 32 * kPanWarps, 0, s>>>(A, np, n, k0, in, count, out, last, pbuf, pimg,
-                                                                        pexp, sw, rowperm, status);
-  };
-  if (count <= 256) go(std::integral_constant<int, 1>{});
-  else if (count <= 512) go(std::integral_constant<int, 2>{});
-  else if (count <= 1024) go(std::integral_constant<int, 4>{});
-  else if (count <= 1536) go(std::integral_constant<int, 6>{});
-  else go(std::integral_constant<int, 8>{});
+  // a thread per candidate row over the cluster's eight CTAs, 128 to 256 threads each
+  int threads = ceil_div(count < kPanRows ? count : kPanRows, kPanCtas * 32) * 32;
+  if (threads < 128) threads = 128;
+  gj64_panel_kernel<<<ceil_div(count, kPanCtas * threads) * kPanCtas, threads, sizeof(PanSmem), s>>>(
+      A, np, n, k0, in, count, out, last, pbuf, pimg, pexp, sw, rowperm, status);
   NED_LAUNCH_CHECK("gj64_panel_kernel");
   return NEDMFT_OK;
 }
@@ -1093,7 +1097,7 @@ PivLayout piv_layout(int n) {
   const int np = ceil_div(n, 128) * 128;
   L.a = align256(sizeof(double2) * (size_t)np * np);
   L.gj = gj64_layout(np, 1).total;
-  L.cand = align256(sizeof(int) * (size_t)ceil_div(n, 2048) * kNB);
+  L.cand = align256(sizeof(int) * (size_t)ceil_div(n, kPanRows) * kNB);
   L.sw = align256(sizeof(RowSwaps));
   L.perm = align256(sizeof(int) * (size_t)np);
   L.amax = align256(8);
@@ -1112,6 +1116,7 @@ int pivot_inverse_prepare() {
   LookAhead* la = nullptr;
   int rc = look_ahead(&la), sms = 0;
   if (!rc) rc = device_sm_count(&sms);
+  if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_panel_kernel), (int)sizeof(PanSmem));
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_rpanel_kernel), RSmem::kBytes);
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_update_kernel), USmem::kBytes);
   return rc;
@@ -1170,11 +1175,11 @@ int pivot_inverse(double2* a, int n, void* ws, cudaStream_t st, int* status) {
   auto panel = [&](int k0, cudaStream_t s) -> int {
     const int* in = nullptr;
     int count = n - k0, buf = 0;
-    while (count > 2048) {  // rounds of 2048 rows until one cluster holds the candidates
+    while (count > kPanRows) {  // rounds of 2048 rows until one cluster holds the candidates
       if (int e = launch_panel(ap, np, n, k0, in, count, cand[buf], false, pbuf, pimg, pexp, sw, rowperm, status, s))
         return e;
       in = cand[buf];
-      count = ceil_div(count, 2048) * kNB;
+      count = ceil_div(count, kPanRows) * kNB;
       buf ^= 1;
     }
     return launch_panel(ap, np, n, k0, in, count, nullptr, true, pbuf, pimg, pexp, sw, rowperm, status, s);
