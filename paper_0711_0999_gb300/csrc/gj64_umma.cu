@@ -21,6 +21,8 @@
 // One MMA per digit a of the left operand takes all its partners b = 0 .. 6-a
 // at once: the right operand's digits lie back to back in shared memory, and
 // orders a .. 6 back to back in TMEM.
+#include <stddef.h>
+
 #include "lattice.cuh"
 #include "umma_core.cuh"
 
@@ -189,21 +191,27 @@ __device__ __forceinline__ bool recip(double2 z, double2& out) {
 }
 
 // Digits of 128 rows of C = A_{:,K} (C_K = -I), TPR threads per row: image rows
-// [Re | Im].  Row i is read from row src[i - 128 mt] when `src` is given.
+// [Re | Im].  Row i is read from row src[i - 128 mt] when `src` is given.  The
+// rows pass through `stage` (128 x kStageRow), brought in by whole 512-byte rows
+// (34 us for 384 tiles when every thread read its own row).
+constexpr int kStageRow = kNB + 1;
 template <int TPR>
 __device__ __forceinline__ void pack_c_rows(const double2* __restrict__ A, int np, int k0, int mt, const int* src,
-                                            __nv_bfloat16* __restrict__ img, int* __restrict__ cexp, int* status) {
-  constexpr int CNT = kNB / TPR;
+                                            double2* stage, __nv_bfloat16* __restrict__ img, int* __restrict__ cexp,
+                                            int* status) {
+  constexpr int CNT = kNB / TPR, kWarps = 128 * TPR / 32;
   const int row = threadIdx.x / TPR, part = threadIdx.x % TPR, i = mt * 128 + row;
-  double2 z[CNT];
-  if (i >= k0 && i < k0 + kNB) {
-#pragma unroll
-    for (int c = 0; c < CNT; ++c) z[c] = make_double2(CNT * part + c == i - k0 ? -1.0 : 0.0, 0.0);
-  } else {
-    const double2* a = A + (size_t)(src ? src[row] : i) * np + k0 + CNT * part;
-#pragma unroll
-    for (int c = 0; c < CNT; ++c) z[c] = a[c];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 8
+  for (int r = warp; r < 128; r += kWarps) {
+    const int g = mt * 128 + r;
+    stage[r * kStageRow + lane] = g >= k0 && g < k0 + kNB ? make_double2(lane == g - k0 ? -1.0 : 0.0, 0.0)
+                                                          : A[(size_t)(src ? src[r] : g) * np + k0 + lane];
   }
+  __syncthreads();
+  double2 z[CNT];
+#pragma unroll
+  for (int c = 0; c < CNT; ++c) z[c] = stage[row * kStageRow + CNT * part + c];
   unsigned m = 0;
 #pragma unroll
   for (int c = 0; c < CNT; ++c) m = max(m, max(mag_hi(z[c].x), mag_hi(z[c].y)));
@@ -224,101 +232,374 @@ __device__ __forceinline__ void pack_c_rows(const double2* __restrict__ A, int n
     }
 }
 
-// CTAs 0 .. nb-1: P = inv(A_KK) of matrix b, 32 x 32 FP64, a warp per four
-// rows, lane = column.  Step k: the pivot row, divided by its pivot (its own
-// entry replaced by the pivot's inverse), is in shared memory (two buffers, one
-// barrier per step); every other row subtracts its entry of column k times it,
-// that entry counted as zero before.  The warp of the next pivot row takes that
-// row first and publishes it, so the reciprocal is off the other warps' path.
-// FP64 bound: 32 rows x 4 FMAs x 16 cycles per step, 33 us.
-// CTAs nb ..: digits of 128 rows of C, two threads per row; this work hides
-// behind the pivot blocks' latency.
-__global__ void __launch_bounds__(256) gj64_pivot_kernel(const double2* __restrict__ A, int np, int mtiles, int k0,
-                                                         int nb, double2* __restrict__ Pbuf,
-                                                         __nv_bfloat16* __restrict__ pimg, int* __restrict__ pexp,
-                                                         __nv_bfloat16* __restrict__ cimg, int* __restrict__ cexp,
-                                                         int* status) {
+struct BlockSmem {
+  __nv_bfloat16 a[kS * 64 * kK];   // digits of the block: row 2r = [Re | -Im], 2r + 1 = [Im | Re]
+  __nv_bfloat16 x[kS * kNB * kK];  // digits of X: row j = [Re X_j | Im X_j], column j over k
+  float2 xt[kNB][kNB], e[kNB][kNB + 1];  // X by columns, the residual by rows
+  float4 prow[kNB / 2];
+  uint64_t bar;
+  uint32_t tmem_slot;
+  int aexp[kNB], xexp[kNB];
+  unsigned amax, emax;
+  int abort, bad;
+};
+// The products read 128 rows of a digit; rows past 64 are the next digit's (the
+// last one's: those of X), and their sums are not read.
+static_assert(128 * kStageRow * sizeof(double2) <= sizeof(BlockSmem), "C rows are staged in the same space");
+static_assert(offsetof(BlockSmem, x) == kS * 64 * kK * 2 && kNB * kK * 2 * 2 <= (int)sizeof(BlockSmem::x), "row overrun");
+
+// x as a double, exactly, on the integer units (conversions run on the FP64
+// units); zero and subnormals become zero, infinities and NaN large values (the
+// caller has checked for them).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+  return a < 0x00800000u ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(u << 29));
+}
+__device__ __forceinline__ void cfmaf(float2& acc, float2 a, float2 b) {
+  acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
+  acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
+}
+
+// The inverse of a 32 x 32 FP64 block by 256 threads.  Thread t brings entries
+// in[0 .. 3] = (row t / 8, columns 4 (t % 8) ..) and gets out[0 .. 3] = (rows
+// 4 (t % 8) .., column t / 8) of the inverse.  False: not found to FP64 accuracy
+// this way (a pivot vanished in FP32, or the first residual is not small).
+// An FP32 Gauss-Jordan elimination by one warp, a lane per row (rows rotate one
+// register down per step, so the loop is rolled), then X <- X + X E with the
+// residual E = I - A X from the digit products on the tensor cores, exact to
+// 2^-54 of the row and column maxima as in the update, and the small product X E
+// in FP32: E squares from round to round (1e-5, 1e-10 as a rule), and below
+// 2^-30 FP32 is enough for the last correction.  Why: the same block by FP64 elimination is 32768 complex
+// multiply-adds on two FP64 units, 33 us at best and 55 us measured.
+__device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&in)[4], double2 (&out)[4],
+                                                uint32_t tmem, uint32_t& phase) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  if ((int)blockIdx.x < nb) {
-    __shared__ double2 rowb[2][32];
-    __shared__ double2 prow[kNB][kNB + 1];
-    const int b = blockIdx.x;
-    const double2* a = A + (size_t)b * np * np + (size_t)k0 * np + k0;
-    double2 v[4];
+  const int r = t >> 3, c4 = 4 * (t & 7);
+  unsigned m = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = a[(size_t)(4 * warp + q) * np + lane];
-    // row (warp, kq) as step k's pivot row: divided by its pivot and published
-    auto publish = [&](double2& z, int k) {
-      const double2 d = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
-      double2 pinv;
-      if (!recip(d, pinv) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
-      z = lane == k ? pinv : cmul(z, pinv);
-      rowb[k & 1][lane] = z;
-    };
-    if (warp == 0) publish(v[0], 0);
-    __syncthreads();
-    for (int kw = 0; kw < 8; ++kw)
+  for (int c = 0; c < 4; ++c) m = max(m, max(mag_hi(in[c].x), mag_hi(in[c].y)));
 #pragma unroll
-      for (int kq = 0; kq < 4; ++kq) {
-        const int k = 4 * kw + kq;
-        const double2 rb = rowb[k & 1][lane];
-        auto eliminate = [&](double2& z) {
-          const double2 c = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
-          const double2 o = lane == k ? make_double2(0.0, 0.0) : z;
-          z = make_double2(fma(-c.x, rb.x, fma(c.y, rb.y, o.x)), fma(-c.x, rb.y, fma(-c.y, rb.x, o.y)));
-        };
-        constexpr int kNext[4] = {1, 2, 3, 0};  // the next pivot row's place in its warp
-        const int nq = kNext[kq];
-        const bool mine = k + 1 < 32 && warp == (kq == 3 ? kw + 1 : kw);
-        if (mine) {  // the next pivot row first: its reciprocal runs beside the other warps' rows
-          eliminate(v[nq]);
-          publish(v[nq], k + 1);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (!(warp == kw && q == kq) && !(mine && q == nq)) eliminate(v[q]);
-        __syncthreads();
-      }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = 4 * warp + q;
-      Pbuf[(size_t)b * kNB * kNB + r * kNB + lane] = v[q];
-      prow[r][lane] = v[q];
-    }
-    __syncthreads();
-    // digits of the 64 real rows of P, eight threads per row r, four entries
-    // each: row 2r = [Re P_r | -Im P_r], row 2r + 1 = [Im P_r | Re P_r]
-    const int r = t >> 3, c4 = 4 * (t & 7);
-    double2 p[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) p[c] = prow[r][c4 + c];
-    unsigned m = 0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) m = max(m, max(mag_hi(p[c].x), mag_hi(p[c].y)));
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const int be = row_biased(m);
-    if ((t & 7) == 0) pexp[b * kNB + r] = be - 1022;
-    if (m >= 0x7ff00000u && status) atomicCAS(status, 0, DS_SINGULAR);
+  for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (t == 0) {
+    sm.amax = 0;
+    sm.bad = 0;
+  }
+  __syncthreads();
+  if ((t & 7) == 0) atomicMax(&sm.amax, m);
+  __syncthreads();
+  const unsigned am = sm.amax;
+  // FP32 needs the block near one: scaled by 2^-e when its largest entry is not within 2^20
+  const int ea = (int)(am >> 20) - 1022, e = ea > 20 || ea < -20 ? ea : 0;
+  if (am >= 0x7ff00000u || am < (24u << 20) || ea > 900) return false;
+  const double sc = __hiloint2double((1023 - e) << 20, 0);
+  const int be = row_biased(m);
+  {
     long long y[8];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      y[c] = digit_word(p[c].x, be);
-      y[4 + c] = digit_word(p[c].y, be);
+      y[c] = digit_word(in[c].x, be);
+      y[4 + c] = digit_word(in[c].y, be);
+      sm.xt[c4 + c][r] = e == 0 ? make_float2((float)in[c].x, (float)in[c].y)
+                                : make_float2((float)(in[c].x * sc), (float)(in[c].y * sc));
     }
-    const int o_re = core_off(2 * r, c4), o_im = core_off(2 * r, 32 + c4);  // row 2r + 1: 8 elements on
+    if ((t & 7) == 0) sm.aexp[r] = be - 1022 - e;
+    const int o_re = core_off(2 * r, c4), o_im = core_off(2 * r, 32 + c4);
     put_digits(y, [&](int s, uint4 w) {
-      __nv_bfloat16* d = pimg + (size_t)b * kPTile + s * 64 * kK;
+      __nv_bfloat16* d = sm.a + s * 64 * kK;
       const uint4 n = neg_bf16(w);
       *reinterpret_cast<uint2*>(d + o_re) = make_uint2(w.x, w.y);
       *reinterpret_cast<uint2*>(d + o_im) = make_uint2(n.z, n.w);
       *reinterpret_cast<uint2*>(d + o_re + 8) = make_uint2(w.z, w.w);
       *reinterpret_cast<uint2*>(d + o_im + 8) = make_uint2(w.x, w.y);
     });
+  }
+  __syncthreads();
+  if (warp == 0) {
+    float2 v[kNB];
+#pragma unroll
+    for (int c = 0; c < kNB; ++c) v[c] = sm.xt[c][lane];
+    bool good = true;
+#pragma unroll 1
+    for (int k = 0; k < kNB; ++k) {
+      if (lane == k) {
+#pragma unroll
+        for (int c = 0; c < kNB / 2; ++c) {
+          sm.prow[c] = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
+          v[2 * c] = v[2 * c + 1] = make_float2(0.f, 0.f);
+        }
+      }
+      __syncwarp();
+      const float4 p0 = sm.prow[0];
+      const float pm = p0.x * p0.x + p0.y * p0.y;
+      good = good && pm > 1e-30f;
+      float rm;
+      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rm) : "f"(pm));
+      const float2 pinv = make_float2(p0.x * rm, -p0.y * rm);
+      // row k: f = -1 / pivot on a zero row; the others: their entry over the pivot
+      float2 f = make_float2(v[0].x * pinv.x - v[0].y * pinv.y, v[0].x * pinv.y + v[0].y * pinv.x);
+      if (lane == k) f = make_float2(-pinv.x, -pinv.y);
+      const float2 nf = make_float2(-f.x, -f.y);
+#pragma unroll
+      for (int c = 0; c < kNB / 2; ++c) {
+        const float4 z = c == 0 ? p0 : sm.prow[c];
+        if (c > 0) {
+          v[2 * c - 1] = v[2 * c];
+          cfmaf(v[2 * c - 1], nf, make_float2(z.x, z.y));
+        }
+        v[2 * c] = v[2 * c + 1];
+        cfmaf(v[2 * c], nf, make_float2(z.z, z.w));
+      }
+      v[kNB - 1] = nf;
+      __syncwarp();
+    }
+#pragma unroll
+    for (int c = 0; c < kNB; ++c) sm.xt[c][lane] = v[c];
+    if (!good) sm.bad = 1;
+  }
+  __syncthreads();
+  // from here on thread t holds rows c4 .. c4 + 3 of column r of X
+  const int j = r;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) out[c] = make_double2(widen(sm.xt[j][c4 + c].x), widen(sm.xt[j][c4 + c].y));
+  if (sm.bad) return false;
+  for (int round = 0; round < 4; ++round) {
+    unsigned mx = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) mx = max(mx, max(mag_hi(out[c].x), mag_hi(out[c].y)));
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const int bx = row_biased(mx);
+    if ((t & 7) == 0) sm.xexp[j] = bx - 1022;
+    if (t == 0) sm.emax = 0;
+    long long y[8];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      y[c] = digit_word(out[c].x, bx);
+      y[4 + c] = digit_word(out[c].y, bx);
+    }
+    const int o_re = core_off(j, c4), o_im = core_off(j, 32 + c4);
+    put_digits(y, [&](int s, uint4 w) {
+      __nv_bfloat16* d = sm.x + s * kNB * kK;
+      *reinterpret_cast<uint2*>(d + o_re) = make_uint2(w.x, w.y);
+      *reinterpret_cast<uint2*>(d + o_im) = make_uint2(w.z, w.w);
+    });
+    fence_proxy_async();
+    __syncthreads();
+    if (t == 0) {
+      tc_fence_after();
+#pragma unroll
+      for (int a = 0; a < kS; ++a)
+#pragma unroll
+        for (int kk = 0; kk < kK / 16; ++kk)
+          mma_bf16(tmem + (uint32_t)(a * kNB), smem_desc(smem_u32(sm.a + a * 64 * kK) + kk * 256, 128, 1024),
+                   smem_desc(smem_u32(sm.x) + kk * 256, 128, 1024), idesc_bf16(128, (kS - a) * kNB),
+                   (a > 0 || kk > 0) ? 1u : 0u);
+      mma_commit(&sm.bar);
+    }
+    volatile int* abort_flag = &sm.abort;
+    bool ok = mbar_wait(&sm.bar, phase, abort_flag);
+    if (!ok) drain_wait(&sm.bar, phase);
+    phase ^= 1u;
+    if (!__syncthreads_and(ok)) return false;
+    tc_fence_after();
+    if ((warp & 3) < 2) {  // lanes 2 r, 2 r + 1 of the first two quarters hold Re, Im of row r; two warps halve the columns
+      const int row = (warp & 3) * 16 + (lane >> 1), part = lane & 1, j0 = 16 * (warp >> 2);
+      const int eb = 1023 + sm.aexp[row] - 53;
+      float big = 0.f;
+#pragma unroll 1
+      for (int g = 0; g < 16; g += 8) {
+        float c[kS][8];
+#pragma unroll
+        for (int o = 0; o < kS; ++o)
+          tmem_ld8(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(o * kNB + j0 + g), c[o]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int col = j0 + g + u;
+          const double d = orders_to_double(c[0][u], c[1][u], c[2][u], c[3][u], c[4][u], c[5][u], c[6][u],
+                                            eb + sm.xexp[col]);
+          // exact where it matters: near the diagonal's one the difference is (Sterbenz)
+          const float f = (float)((row == col && part == 0 ? 1.0 : 0.0) - d);
+          big = fmaxf(big, fabsf(f));
+          (&sm.e[row][col].x)[part] = f;
+          if (!(fabsf(f) < 1e30f)) big = 1e30f;
+        }
+      }
+      tc_fence_before();
+      const unsigned wb = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
+      if (lane == 0) atomicMax(&sm.emax, wb);
+    }
+    __syncthreads();
+    const float emax = __uint_as_float(sm.emax);
+    if (!(emax < 0.125f)) return false;
+    // X += X E
+    float2 acc[4] = {};
+#pragma unroll 8
+    for (int l = 0; l < kNB; ++l) {
+      const float2 b = sm.e[l][j];
+      const float4 x01 = *reinterpret_cast<const float4*>(&sm.xt[l][c4]);
+      const float4 x23 = *reinterpret_cast<const float4*>(&sm.xt[l][c4 + 2]);
+      cfmaf(acc[0], make_float2(x01.x, x01.y), b);
+      cfmaf(acc[1], make_float2(x01.z, x01.w), b);
+      cfmaf(acc[2], make_float2(x23.x, x23.y), b);
+      cfmaf(acc[3], make_float2(x23.z, x23.w), b);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      out[c].x += widen(acc[c].x);
+      out[c].y += widen(acc[c].y);
+    }
+    const bool last = emax < 9.3e-10f;  // 2^-30: what is left is E^2 and the product's FP32 rounding
+    if (last) {
+      if (e != 0) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) out[c] = make_double2(out[c].x * sc, out[c].y * sc);
+      }
+      return true;
+    }
+    __syncthreads();  // every thread has read xt and e
+#pragma unroll
+    for (int c = 0; c < 4; ++c) sm.xt[j][c4 + c] = make_float2((float)out[c].x, (float)out[c].y);
+  }
+  return false;
+}
+
+// P = inv of a 32 x 32 block by FP64 elimination, 256 threads, a warp per four
+// rows (v), lane = column.  Step k: the pivot row, divided by its pivot (its own
+// entry replaced by the pivot's inverse), is in shared memory (two buffers, one
+// barrier per step); every other row subtracts its entry of column k times it,
+// that entry counted as zero before.  The warp of the next pivot row takes that
+// row first and publishes it.  FP64 bound: 32 rows x 4 FMAs x 16 cycles per step.
+__device__ __forceinline__ void fp64_inverse(double2 (&v)[4], double2 (&rowb)[2][32], int* status) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // row (warp, kq) as step k's pivot row: divided by its pivot and published
+  auto publish = [&](double2& z, int k) {
+    const double2 d = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+    double2 pinv;
+    if (!recip(d, pinv) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
+    z = lane == k ? pinv : cmul(z, pinv);
+    rowb[k & 1][lane] = z;
+  };
+  if (warp == 0) publish(v[0], 0);
+  __syncthreads();
+  for (int kw = 0; kw < 8; ++kw)
+#pragma unroll
+    for (int kq = 0; kq < 4; ++kq) {
+      const int k = 4 * kw + kq;
+      const double2 rb = rowb[k & 1][lane];
+      auto eliminate = [&](double2& z) {
+        const double2 c = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
+        const double2 o = lane == k ? make_double2(0.0, 0.0) : z;
+        z = make_double2(fma(-c.x, rb.x, fma(c.y, rb.y, o.x)), fma(-c.x, rb.y, fma(-c.y, rb.x, o.y)));
+      };
+      constexpr int kNext[4] = {1, 2, 3, 0};  // the next pivot row's place in its warp
+      const int nq = kNext[kq];
+      const bool mine = k + 1 < 32 && warp == (kq == 3 ? kw + 1 : kw);
+      if (mine) {  // the next pivot row first: its reciprocal runs beside the other warps' rows
+        eliminate(v[nq]);
+        publish(v[nq], k + 1);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (!(warp == kw && q == kq) && !(mine && q == nq)) eliminate(v[q]);
+      __syncthreads();
+    }
+}
+
+// Matrix b's P (rows in shared memory) to Pbuf, and the digits of its 64 real
+// rows, eight threads per row r, four entries each: row 2r = [Re P_r | -Im P_r],
+// row 2r + 1 = [Im P_r | Re P_r].
+__device__ __forceinline__ void write_p(const double2 (*prow)[kNB + 1], int b, double2* __restrict__ Pbuf,
+                                        __nv_bfloat16* __restrict__ pimg, int* __restrict__ pexp, int* status) {
+  const int t = threadIdx.x;
+  const int r = t >> 3, c4 = 4 * (t & 7);
+  double2 p[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    p[c] = prow[r][c4 + c];
+    Pbuf[(size_t)b * kNB * kNB + r * kNB + c4 + c] = p[c];
+  }
+  unsigned m = 0;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) m = max(m, max(mag_hi(p[c].x), mag_hi(p[c].y)));
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int be = row_biased(m);
+  if ((t & 7) == 0) pexp[b * kNB + r] = be - 1022;
+  if (m >= 0x7ff00000u && status) atomicCAS(status, 0, DS_SINGULAR);
+  long long y[8];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    y[c] = digit_word(p[c].x, be);
+    y[4 + c] = digit_word(p[c].y, be);
+  }
+  const int o_re = core_off(2 * r, c4), o_im = core_off(2 * r, 32 + c4);  // row 2r + 1: 8 elements on
+  put_digits(y, [&](int s, uint4 w) {
+    __nv_bfloat16* d = pimg + (size_t)b * kPTile + s * 64 * kK;
+    const uint4 n = neg_bf16(w);
+    *reinterpret_cast<uint2*>(d + o_re) = make_uint2(w.x, w.y);
+    *reinterpret_cast<uint2*>(d + o_im) = make_uint2(n.z, n.w);
+    *reinterpret_cast<uint2*>(d + o_re + 8) = make_uint2(w.z, w.w);
+    *reinterpret_cast<uint2*>(d + o_im + 8) = make_uint2(w.x, w.y);
+  });
+}
+
+// CTAs 0 .. nb-1: P = inv(A_KK) of matrix b and its digits.
+// CTAs nb ..: digits of 128 rows of C, two threads per row; this work hides
+// behind the pivot blocks' latency.
+__global__ void __launch_bounds__(256, 2)
+    gj64_pivot_kernel(const double2* __restrict__ A, int np, int mtiles, int k0, int nb, double2* __restrict__ Pbuf,
+                      __nv_bfloat16* __restrict__ pimg, int* __restrict__ pexp, __nv_bfloat16* __restrict__ cimg,
+                      int* __restrict__ cexp, int* status) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  if ((int)blockIdx.x < nb) {
+    BlockSmem& sm = *reinterpret_cast<BlockSmem*>(smem_raw);
+    const int b = blockIdx.x;
+    const double2* a = A + (size_t)b * np * np + (size_t)k0 * np + k0;
+    const int r = t >> 3, c4 = 4 * (t & 7);
+    double2 in[4], out[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) in[c] = a[(size_t)r * np + c4 + c];
+    if (t == 0) {
+      mbar_init(&sm.bar, 1);
+      sm.abort = 0;
+      fence_barrier_init();
+    }
+    if (warp == 0) tmem_alloc(&sm.tmem_slot, 256);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = sm.tmem_slot;
+    uint32_t phase = 0;
+    const bool found = refined_inverse(sm, in, out, tmem, phase);
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+      tc_fence_after();
+      tmem_dealloc(tmem, 256);
+    }
+    if (t == 0 && sm.abort && status) atomicCAS(status, 0, DS_TIMEOUT);
+    // P by rows through shared memory (over the digits, which nobody reads any more)
+    double2 (*prow)[kNB + 1] = reinterpret_cast<double2 (*)[kNB + 1]>(sm.a);
+    if (found) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) prow[c4 + c][r] = out[c];
+    } else {
+      double2 v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = a[(size_t)(4 * warp + q) * np + lane];
+      fp64_inverse(v, *reinterpret_cast<double2 (*)[2][32]>(sm.x), status);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) prow[4 * warp + q][lane] = v[q];
+    }
+    __syncthreads();
+    write_p(prow, b, Pbuf, pimg, pexp, status);
     return;
   }
   const int u = blockIdx.x - nb, b = u / mtiles, mt = u % mtiles;
-  pack_c_rows<2>(A + (size_t)b * np * np, np, k0, mt, nullptr, cimg + (size_t)u * kATile, cexp + (size_t)b * np,
+  pack_c_rows<2>(A + (size_t)b * np * np, np, k0, mt, nullptr, reinterpret_cast<double2*>(smem_raw),
+                 cimg + (size_t)u * kATile, cexp + (size_t)b * np,
                  status);
 }
 
@@ -355,6 +636,7 @@ __global__ void __launch_bounds__(512, 1)
                        const __nv_bfloat16* __restrict__ pimg, const int* __restrict__ pexp,
                        __nv_bfloat16* __restrict__ rimg, int* __restrict__ rexp, const RowSwaps* __restrict__ sw,
                        __nv_bfloat16* __restrict__ cimg, int* __restrict__ cexp, int* status) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
   if ((int)blockIdx.x >= mtiles) {
     __shared__ int src[128];
     const int mt = blockIdx.x - mtiles, t = threadIdx.x;
@@ -362,10 +644,9 @@ __global__ void __launch_bounds__(512, 1)
     __syncthreads();
     if (t < sw->moved && sw->to[t] / 128 == mt) src[sw->to[t] % 128] = sw->from[t];
     __syncthreads();
-    pack_c_rows<4>(A, np, k0, mt, src, cimg + (size_t)mt * kATile, cexp, status);
+    pack_c_rows<4>(A, np, k0, mt, src, reinterpret_cast<double2*>(smem_raw), cimg + (size_t)mt * kATile, cexp, status);
     return;
   }
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __nv_bfloat16* sa = reinterpret_cast<__nv_bfloat16*>(smem);
   __nv_bfloat16* sp = reinterpret_cast<__nv_bfloat16*>(smem + RSmem::kA);
@@ -530,7 +811,8 @@ static_assert(sizeof(UBars) <= USmem::kBars, "barrier block");
 // cycles per tile of 4400, epilogue about 1700 issue cycles.  Measured before
 // it: old values loaded by TMA in 64-byte rows two boxes ahead, subtracted and
 // stored, 292 us (the shared memory left for boxes does not cover the latency);
-// half of the boxes each way, 274 us.
+// half of the boxes each way, 274 us; every other tile of six warps loaded in
+// 128-byte rows one tile ahead, 359 us.
 __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
     gj64_update_kernel(const __grid_constant__ CUtensorMap amap, int np, int mtiles, int ntn, int total, int k0,
                        int jskip, int nskip, const __nv_bfloat16* __restrict__ cimg, const int* __restrict__ cexp,
@@ -770,12 +1052,13 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
   int rc = encode_f64_boxes(&map, A, np, (uint64_t)np * nb);
   int sms = 0;
   if (!rc) rc = device_sm_count(&sms);
+  if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_pivot_kernel), (int)sizeof(BlockSmem));
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_rpanel_kernel), RSmem::kBytes);
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_update_kernel), USmem::kBytes);
   if (rc) return rc;
   const int mtiles = np / 128, ntn = ceil_div(n, kTn), total = nb * mtiles * ntn;
   for (int k0 = 0; k0 < n; k0 += kNB) {
-    gj64_pivot_kernel<<<nb + nb * mtiles, 256, 0, st>>>(A, np, mtiles, k0, nb, pbuf, pimg, pexp, cimg,
+    gj64_pivot_kernel<<<nb + nb * mtiles, 256, sizeof(BlockSmem), st>>>(A, np, mtiles, k0, nb, pbuf, pimg, pexp, cimg,
                                                           cexp, status);
     NED_LAUNCH_CHECK("gj64_pivot_kernel");
     gj64_rpanel_kernel<<<dim3(mtiles, nb), 512, RSmem::kBytes, st>>>(A, np, mtiles, k0, pbuf, pimg, pexp, rimg, rexp,
@@ -867,7 +1150,7 @@ __global__ void __cluster_dims__(kPanCtas, 1, 1) __launch_bounds__(256, 1)
       v[e] = make_float2((float)z.x, (float)z.y);
     }
   }
-  bool live = row >= 0, ok = true;
+  bool live = row >= 0;
   __syncthreads();
   cluster_barrier();  // every CTA's barriers are set before another counts on them
 #pragma unroll 1
@@ -901,21 +1184,19 @@ __global__ void __cluster_dims__(kPanCtas, 1, 1) __launch_bounds__(256, 1)
       if (lane < kPanCtas)
         st_async(&sm.cand[j][q], &sm.bar[j], lane, make_uint4((uint32_t)top, (uint32_t)srow, 0u, 0u));
     }
-    ok = mbar_wait(&sm.bar[j], 0, abort_flag);
-    if (!__syncthreads_and(ok)) {
-      ok = false;
-      break;
-    }
+    mbar_wait(&sm.bar[j], 0, abort_flag);  // after a failed wait the steps run on without waiting; rows are checked
     const uint4 y = sm.cand[j][lane & (kPanCtas - 1)];
     const int best = __reduce_max_sync(0xffffffffu, (int)y.x);
     const int qtop = __ffs(__ballot_sync(0xffffffffu, (int)y.x == best)) - 1;
     const int wrow = (int)sm.cand[j][qtop].y;
-    if (t == 0) sm.win[j] = best >= 0 ? wrow : -1;  // -1: no candidate left, or none finite
+    if (t == 0) sm.win[j] = best >= 0 && wrow >= k0 && wrow < n ? wrow : -1;  // -1: none left, or none finite
     if (best >= 0 && row == wrow) live = false;
     const float4* pr = sm.row[j][qtop];
     const float4 p0 = pr[0];
     const float pm = p0.x * p0.x + p0.y * p0.y;
-    const float rm = pm > 0.f ? 1.f / pm : 0.f;
+    float rm;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rm) : "f"(pm));
+    rm = pm > 1e-37f ? rm : 0.f;
     const float2 f = make_float2((v[0].x * p0.x + v[0].y * p0.y) * rm, (v[0].y * p0.x - v[0].x * p0.y) * rm);
 #pragma unroll
     for (int e = 0; e < kNB / 2; ++e) {
