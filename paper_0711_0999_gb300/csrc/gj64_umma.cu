@@ -235,8 +235,8 @@ __device__ __forceinline__ void pack_c_rows(const double2* __restrict__ A, int n
 struct BlockSmem {
   __nv_bfloat16 a[kS * 64 * kK];   // digits of the block: row 2r = [Re | -Im], 2r + 1 = [Im | Re]
   __nv_bfloat16 x[kS * kNB * kK];  // digits of X: row j = [Re X_j | Im X_j], column j over k
-  float2 xt[kNB][kNB], e[kNB][kNB + 1];  // X by columns, the residual by rows
-  float4 prow[kNB / 2];
+  float2 xt[kNB][kNB], e[kNB][kNB + 2];  // X by columns, the residual by rows
+  float2 mult[2][kNB];
   uint64_t bar;
   uint32_t tmem_slot;
   int aexp[kNB], xexp[kNB];
@@ -264,8 +264,7 @@ __device__ __forceinline__ void cfmaf(float2& acc, float2 a, float2 b) {
 // in[0 .. 3] = (row t / 8, columns 4 (t % 8) ..) and gets out[0 .. 3] = (rows
 // 4 (t % 8) .., column t / 8) of the inverse.  False: not found to FP64 accuracy
 // this way (a pivot vanished in FP32, or the first residual is not small).
-// An FP32 Gauss-Jordan elimination by one warp, a lane per row (rows rotate one
-// register down per step, so the loop is rolled), then X <- X + X E with the
+// An FP32 Gauss-Jordan elimination by four warps, then X <- X + X E with the
 // residual E = I - A X from the digit products on the tensor cores, exact to
 // 2^-54 of the row and column maxima as in the update, and the small product X E
 // in FP32: E squares from round to round (1e-5, 1e-10 as a rule), and below
@@ -314,46 +313,43 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
     });
   }
   __syncthreads();
-  if (warp == 0) {
-    float2 v[kNB];
+  if (warp < 4) {
+    // lane = row, eight columns per warp; the step's column's warp sends every row's multiplier
+    float2 v[8];
 #pragma unroll
-    for (int c = 0; c < kNB; ++c) v[c] = sm.xt[c][lane];
+    for (int c = 0; c < 8; ++c) v[c] = sm.xt[8 * warp + c][lane];
     bool good = true;
 #pragma unroll 1
-    for (int k = 0; k < kNB; ++k) {
-      if (lane == k) {
+    for (int kw = 0; kw < 4; ++kw)
 #pragma unroll
-        for (int c = 0; c < kNB / 2; ++c) {
-          sm.prow[c] = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
-          v[2 * c] = v[2 * c + 1] = make_float2(0.f, 0.f);
+      for (int kc = 0; kc < 8; ++kc) {
+        const int k = 8 * kw + kc;
+        float2 p[8];  // this warp's part of the pivot row
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          p[c] = make_float2(__shfl_sync(0xffffffffu, v[c].x, k), __shfl_sync(0xffffffffu, v[c].y, k));
+        if (warp == kw) {
+          const float pm = p[kc].x * p[kc].x + p[kc].y * p[kc].y;
+          good = good && pm > 1e-30f;
+          float rm;
+          asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rm) : "f"(pm));
+          const float2 pinv = make_float2(p[kc].x * rm, -p[kc].y * rm);
+          // row k: -1 / pivot, on a row taken as zero; the others: their entry over the pivot
+          sm.mult[kc & 1][lane] = lane == k ? make_float2(-pinv.x, -pinv.y)
+                                            : make_float2(v[kc].x * pinv.x - v[kc].y * pinv.y,
+                                                          v[kc].x * pinv.y + v[kc].y * pinv.x);
         }
-      }
-      __syncwarp();
-      const float4 p0 = sm.prow[0];
-      const float pm = p0.x * p0.x + p0.y * p0.y;
-      good = good && pm > 1e-30f;
-      float rm;
-      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rm) : "f"(pm));
-      const float2 pinv = make_float2(p0.x * rm, -p0.y * rm);
-      // row k: f = -1 / pivot on a zero row; the others: their entry over the pivot
-      float2 f = make_float2(v[0].x * pinv.x - v[0].y * pinv.y, v[0].x * pinv.y + v[0].y * pinv.x);
-      if (lane == k) f = make_float2(-pinv.x, -pinv.y);
-      const float2 nf = make_float2(-f.x, -f.y);
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        const float2 f = sm.mult[kc & 1][lane], nf = make_float2(-f.x, -f.y);
 #pragma unroll
-      for (int c = 0; c < kNB / 2; ++c) {
-        const float4 z = c == 0 ? p0 : sm.prow[c];
-        if (c > 0) {
-          v[2 * c - 1] = v[2 * c];
-          cfmaf(v[2 * c - 1], nf, make_float2(z.x, z.y));
+        for (int c = 0; c < 8; ++c) {
+          if (lane == k) v[c] = make_float2(0.f, 0.f);
+          cfmaf(v[c], nf, p[c]);
         }
-        v[2 * c] = v[2 * c + 1];
-        cfmaf(v[2 * c], nf, make_float2(z.z, z.w));
+        if (warp == kw) v[kc] = nf;
       }
-      v[kNB - 1] = nf;
-      __syncwarp();
-    }
 #pragma unroll
-    for (int c = 0; c < kNB; ++c) sm.xt[c][lane] = v[c];
+    for (int c = 0; c < 8; ++c) sm.xt[8 * warp + c][lane] = v[c];
     if (!good) sm.bad = 1;
   }
   __syncthreads();
@@ -432,22 +428,28 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
     __syncthreads();
     const float emax = __uint_as_float(sm.emax);
     if (!(emax < 0.125f)) return false;
-    // X += X E
+    // X += X E: lane = row of the product, four columns per warp (X by columns and
+    // broadcasts of E: four shared-memory wavefronts per l), then back to this thread's entries
     float2 acc[4] = {};
 #pragma unroll 8
     for (int l = 0; l < kNB; ++l) {
-      const float2 b = sm.e[l][j];
-      const float4 x01 = *reinterpret_cast<const float4*>(&sm.xt[l][c4]);
-      const float4 x23 = *reinterpret_cast<const float4*>(&sm.xt[l][c4 + 2]);
-      cfmaf(acc[0], make_float2(x01.x, x01.y), b);
-      cfmaf(acc[1], make_float2(x01.z, x01.w), b);
-      cfmaf(acc[2], make_float2(x23.x, x23.y), b);
-      cfmaf(acc[3], make_float2(x23.z, x23.w), b);
+      const float2 x = sm.xt[l][lane];
+      const float4 e01 = *reinterpret_cast<const float4*>(&sm.e[l][4 * warp]);
+      const float4 e23 = *reinterpret_cast<const float4*>(&sm.e[l][4 * warp + 2]);
+      cfmaf(acc[0], x, make_float2(e01.x, e01.y));
+      cfmaf(acc[1], x, make_float2(e01.z, e01.w));
+      cfmaf(acc[2], x, make_float2(e23.x, e23.y));
+      cfmaf(acc[3], x, make_float2(e23.z, e23.w));
     }
+    __syncthreads();  // every thread has read xt and e
+#pragma unroll
+    for (int c = 0; c < 4; ++c) sm.xt[4 * warp + c][lane] = acc[c];
+    __syncthreads();
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      out[c].x += widen(acc[c].x);
-      out[c].y += widen(acc[c].y);
+      const float2 d = sm.xt[j][c4 + c];
+      out[c].x += widen(d.x);
+      out[c].y += widen(d.y);
     }
     const bool last = emax < 9.3e-10f;  // 2^-30: what is left is E^2 and the product's FP32 rounding
     if (last) {
@@ -457,7 +459,6 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
       }
       return true;
     }
-    __syncthreads();  // every thread has read xt and e
 #pragma unroll
     for (int c = 0; c < 4; ++c) sm.xt[j][c4 + c] = make_float2((float)out[c].x, (float)out[c].y);
   }
