@@ -23,6 +23,8 @@
 // orders a .. 6 back to back in TMEM.
 #include <stddef.h>
 
+#include <type_traits>
+
 #include "lattice.cuh"
 #include "umma_core.cuh"
 
@@ -122,6 +124,23 @@ __device__ __forceinline__ int core_off(int row, int k) { return ((row >> 3) * 8
 
 // ------------------------------------------------------------------ order sums to FP64
 
+constexpr unsigned long long kPairOff = 0x8B400000ull;  // 0x4B400000 * 257 mod 2^32: the offset of a pair's word
+constexpr unsigned long long kLess = 0ull - kPairOff * ((1ull << 31) + (1ull << 15) + 1ull);
+// the orders in pairs, each word kPairOff above its value: T = u0 2^31 + u1 2^15 + u2 + kLess
+__device__ __forceinline__ void order_words(float c0, float c1, float c2, float c3, float c4, float c5, float c6,
+                                            uint32_t& u0, uint32_t& u1, uint32_t& u2) {
+  constexpr float kM = 12582912.f;
+  const uint32_t b0 = __float_as_uint(c0 + kM), b1 = __float_as_uint(c1 + kM);
+  const uint32_t b2 = __float_as_uint(c2 + kM), b3 = __float_as_uint(c3 + kM);
+  const float t4 = fmaf(c4, 0.5f, kM);
+  const float rem = fmaf(c4, 0.5f, kM - t4);
+  const float g = fmaf(rem, 512.f, fmaf(c6, 0.00390625f, c5));
+  const uint32_t b4 = __float_as_uint(t4), b5 = __float_as_uint(fmaf(g, 0.5f, kM));
+  u0 = b0 * 256u + b1;
+  u1 = b2 * 256u + b3;
+  u2 = b4 * 256u + b5;
+}
+
 // 2^(e-53) sum_o c_o 2^(8(5-o)) / 2 as a double, rounded once; c_o, o = 0 .. 6,
 // are integers with |c_o| <= (o + 1) 2^20.  ebase = 1023 + e - 53.
 // Float to int by adding 1.5 2^23 (below 2^22; conversion instructions run at
@@ -134,16 +153,8 @@ __device__ __forceinline__ int core_off(int row, int k) { return ((row >> 3) * 8
 // and conditionals took twice as many.
 __device__ __forceinline__ double orders_to_double(float c0, float c1, float c2, float c3, float c4, float c5,
                                                    float c6, int ebase) {
-  constexpr float kM = 12582912.f;
-  constexpr unsigned long long kOff = 0x8B400000ull;  // 0x4B400000 * 257 mod 2^32: the offset of a pair's word
-  constexpr unsigned long long kLess = 0ull - kOff * ((1ull << 31) + (1ull << 15) + 1ull);
-  const uint32_t b0 = __float_as_uint(c0 + kM), b1 = __float_as_uint(c1 + kM);
-  const uint32_t b2 = __float_as_uint(c2 + kM), b3 = __float_as_uint(c3 + kM);
-  const float t4 = fmaf(c4, 0.5f, kM);
-  const float rem = fmaf(c4, 0.5f, kM - t4);
-  const float g = fmaf(rem, 512.f, fmaf(c6, 0.00390625f, c5));
-  const uint32_t b4 = __float_as_uint(t4), b5 = __float_as_uint(fmaf(g, 0.5f, kM));
-  const uint32_t u0 = b0 * 256u + b1, u1 = b2 * 256u + b3, u2 = b4 * 256u + b5;  // the pairs + kOff
+  uint32_t u0, u1, u2;
+  order_words(c0, c1, c2, c3, c4, c5, c6, u0, u1, u2);
   uint32_t rh, ql;
   asm("{\n\t"
       ".reg .u64 t;\n\t.reg .u32 lo, hi, s, n, ld, e, qh;\n\t.reg .f32 fh, fl;\n\t.reg .pred z;\n\t"
@@ -169,6 +180,18 @@ __device__ __forceinline__ double orders_to_double(float c0, float c1, float c2,
       : "=&r"(rh), "=&r"(ql)
       : "r"(u0), "r"(u1), "r"(u2), "l"(kLess), "r"(ebase - 128));
   return __hiloint2double((int)rh, (int)ql);
+}
+
+// the same sum plus `more` (in its units), as a float of about 24 bits, times `scale`
+__device__ __forceinline__ float orders_to_float(float c0, float c1, float c2, float c3, float c4, float c5, float c6,
+                                                 unsigned long long more, float scale) {
+  uint32_t u0, u1, u2;
+  order_words(c0, c1, c2, c3, c4, c5, c6, u0, u1, u2);
+  const long long T = (long long)((unsigned long long)u0 * 0x80000000ull +
+                                  ((unsigned long long)u1 * 32768ull + ((unsigned long long)u2 + (kLess + more))));
+  const unsigned long long a = (unsigned long long)(T < 0 ? -T : T);
+  const float f = __fmaf_rz(__uint2float_rz((uint32_t)(a >> 32)), 4294967296.f, __uint2float_rz((uint32_t)a));
+  return (T < 0 ? -f : f) * scale;
 }
 
 // ------------------------------------------------------------------ pivot block and C digits
@@ -205,8 +228,9 @@ __device__ __forceinline__ void pack_c_rows(const double2* __restrict__ A, int n
 #pragma unroll 8
   for (int r = warp; r < 128; r += kWarps) {
     const int g = mt * 128 + r;
-    stage[r * kStageRow + lane] = g >= k0 && g < k0 + kNB ? make_double2(lane == g - k0 ? -1.0 : 0.0, 0.0)
-                                                          : A[(size_t)(src ? src[r] : g) * np + k0 + lane];
+    double2 z = A[(size_t)(src ? src[r] : g) * np + k0 + lane];
+    if (g >= k0 && g < k0 + kNB) z = make_double2(lane == g - k0 ? -1.0 : 0.0, 0.0);
+    stage[r * kStageRow + lane] = z;
   }
   __syncthreads();
   double2 z[CNT];
@@ -255,6 +279,16 @@ __device__ __forceinline__ double widen(float x) {
   const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
   return a < 0x00800000u ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(u << 29));
 }
+// x as a float, rounded towards zero, on the integer units; below the range
+// zero, above it and for a NaN a NaN.
+__device__ __forceinline__ float narrow(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t e = (hi >> 20) & 0x7ffu;
+  uint32_t u = __funnelshift_l(lo, hi, 3) - (896u << 23);
+  u = e < 897u ? 0u : e > 896u + 254u ? 0x7fffffffu : u;
+  return __uint_as_float((u & 0x7fffffffu) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float2 narrow(double2 z) { return make_float2(narrow(z.x), narrow(z.y)); }
 __device__ __forceinline__ void cfmaf(float2& acc, float2 a, float2 b) {
   acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
   acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
@@ -298,8 +332,7 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
     for (int c = 0; c < 4; ++c) {
       y[c] = digit_word(in[c].x, be);
       y[4 + c] = digit_word(in[c].y, be);
-      sm.xt[c4 + c][r] = e == 0 ? make_float2((float)in[c].x, (float)in[c].y)
-                                : make_float2((float)(in[c].x * sc), (float)(in[c].y * sc));
+      sm.xt[c4 + c][r] = narrow(e == 0 ? in[c] : make_double2(in[c].x * sc, in[c].y * sc));
     }
     if ((t & 7) == 0) sm.aexp[r] = be - 1022 - e;
     const int o_re = core_off(2 * r, c4), o_im = core_off(2 * r, 32 + c4);
@@ -400,7 +433,6 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
     tc_fence_after();
     if ((warp & 3) < 2) {  // lanes 2 r, 2 r + 1 of the first two quarters hold Re, Im of row r; two warps halve the columns
       const int row = (warp & 3) * 16 + (lane >> 1), part = lane & 1, j0 = 16 * (warp >> 2);
-      const int eb = 1023 + sm.aexp[row] - 53;
       float big = 0.f;
 #pragma unroll 1
       for (int g = 0; g < 16; g += 8) {
@@ -411,14 +443,15 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
         tmem_wait_ld();
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int col = j0 + g + u;
-          const double d = orders_to_double(c[0][u], c[1][u], c[2][u], c[3][u], c[4][u], c[5][u], c[6][u],
-                                            eb + sm.xexp[col]);
-          // exact where it matters: near the diagonal's one the difference is (Sterbenz)
-          const float f = (float)((row == col && part == 0 ? 1.0 : 0.0) - d);
+          // A X - I in units of 2^(ex - 53), the one taken off before any rounding
+          const int col = j0 + g + u, ex = sm.aexp[row] + sm.xexp[col];
+          const bool one = row == col && part == 0;
+          if (one && (ex < -8 || ex > 50)) big = 1e30f;  // not an inverse: a column of X or a row of A is lost
+          const float f = -orders_to_float(c[0][u], c[1][u], c[2][u], c[3][u], c[4][u], c[5][u], c[6][u],
+                                           one ? 0ull - (1ull << ((53 - ex) & 63)) : 0ull,
+                                           __int_as_float((127 - 53 + max(min(ex, 100), -60)) << 23));
           big = fmaxf(big, fabsf(f));
           (&sm.e[row][col].x)[part] = f;
-          if (!(fabsf(f) < 1e30f)) big = 1e30f;
         }
       }
       tc_fence_before();
@@ -460,7 +493,7 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
       return true;
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) sm.xt[j][c4 + c] = make_float2((float)out[c].x, (float)out[c].y);
+    for (int c = 0; c < 4; ++c) sm.xt[j][c4 + c] = narrow(out[c]);
   }
   return false;
 }
@@ -545,6 +578,52 @@ __device__ __forceinline__ void write_p(const double2 (*prow)[kNB + 1], int b, d
   });
 }
 
+// P = inv of the block whose row k starts at row_of(k), by 256 threads, and its
+// digits; all of the CTA's threads, with the shared memory to themselves.
+template <class RowOf>
+__device__ __forceinline__ void invert_block(BlockSmem& sm, RowOf&& row_of, int b, double2* __restrict__ Pbuf,
+                                             __nv_bfloat16* __restrict__ pimg, int* __restrict__ pexp, int* status) {
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int r = t >> 3, c4 = 4 * (t & 7);
+  double2 in[4], out[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) in[c] = row_of(r)[c4 + c];
+  if (t == 0) {
+    mbar_init(&sm.bar, 1);
+    sm.abort = 0;
+    fence_barrier_init();
+  }
+  if (warp == 0) tmem_alloc(&sm.tmem_slot, 256);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = sm.tmem_slot;
+  uint32_t phase = 0;
+  const bool found = refined_inverse(sm, in, out, tmem, phase);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 256);
+  }
+  if (t == 0 && sm.abort && status) atomicCAS(status, 0, DS_TIMEOUT);
+  // P by rows through shared memory (over the digits, which nobody reads any more)
+  double2 (*prow)[kNB + 1] = reinterpret_cast<double2 (*)[kNB + 1]>(sm.a);
+  if (found) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) prow[c4 + c][r] = out[c];
+  } else {
+    double2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = row_of(4 * warp + q)[lane];
+    fp64_inverse(v, *reinterpret_cast<double2 (*)[2][32]>(sm.x), status);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) prow[4 * warp + q][lane] = v[q];
+  }
+  __syncthreads();
+  write_p(prow, b, Pbuf, pimg, pexp, status);
+}
+
 // CTAs 0 .. nb-1: P = inv(A_KK) of matrix b and its digits.
 // CTAs nb ..: digits of 128 rows of C, two threads per row; this work hides
 // behind the pivot blocks' latency.
@@ -553,49 +632,10 @@ __global__ void __launch_bounds__(256, 2)
                       __nv_bfloat16* __restrict__ pimg, int* __restrict__ pexp, __nv_bfloat16* __restrict__ cimg,
                       int* __restrict__ cexp, int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   if ((int)blockIdx.x < nb) {
-    BlockSmem& sm = *reinterpret_cast<BlockSmem*>(smem_raw);
-    const int b = blockIdx.x;
-    const double2* a = A + (size_t)b * np * np + (size_t)k0 * np + k0;
-    const int r = t >> 3, c4 = 4 * (t & 7);
-    double2 in[4], out[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) in[c] = a[(size_t)r * np + c4 + c];
-    if (t == 0) {
-      mbar_init(&sm.bar, 1);
-      sm.abort = 0;
-      fence_barrier_init();
-    }
-    if (warp == 0) tmem_alloc(&sm.tmem_slot, 256);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = sm.tmem_slot;
-    uint32_t phase = 0;
-    const bool found = refined_inverse(sm, in, out, tmem, phase);
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-      tc_fence_after();
-      tmem_dealloc(tmem, 256);
-    }
-    if (t == 0 && sm.abort && status) atomicCAS(status, 0, DS_TIMEOUT);
-    // P by rows through shared memory (over the digits, which nobody reads any more)
-    double2 (*prow)[kNB + 1] = reinterpret_cast<double2 (*)[kNB + 1]>(sm.a);
-    if (found) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) prow[c4 + c][r] = out[c];
-    } else {
-      double2 v[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] = a[(size_t)(4 * warp + q) * np + lane];
-      fp64_inverse(v, *reinterpret_cast<double2 (*)[2][32]>(sm.x), status);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) prow[4 * warp + q][lane] = v[q];
-    }
-    __syncthreads();
-    write_p(prow, b, Pbuf, pimg, pexp, status);
+    const double2* a = A + (size_t)blockIdx.x * np * np + (size_t)k0 * np + k0;
+    invert_block(*reinterpret_cast<BlockSmem*>(smem_raw), [&](int k) { return a + (size_t)k * np; }, blockIdx.x, Pbuf,
+                 pimg, pexp, status);
     return;
   }
   const int u = blockIdx.x - nb, b = u / mtiles, mt = u % mtiles;
@@ -1079,220 +1119,209 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
 
 namespace {
 
-constexpr int kPanCtas = 8;     // CTAs of a panel cluster
-constexpr int kPanRows = 2048;  // most rows of one: 256 threads, a row each
+constexpr int kPanThreads = 256;
+constexpr int kPanCand = 256;  // candidate rows of a CTA
+constexpr int kPanCtas = 8;    // most CTAs of a cluster
+constexpr int kPanRows = kPanCand * kPanCtas;
 
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// 16 bytes into CTA `rank`'s copy of *p, counted on its copy of `bar`
-__device__ __forceinline__ void st_async(const void* p, const uint64_t* bar, uint32_t rank, uint4 v) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(
-                   cluster_addr(p, rank)),
-               "r"(cluster_addr(bar, rank)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
 
+constexpr int kStagePitch = kNB + 1;  // staged candidate rows: conflict-free with a lane per row
 struct PanSmem {
-  float4 row[kNB][kPanCtas][kNB / 2];  // per step: the CTAs' candidate rows, from the step's column on
-  uint4 cand[kNB][kPanCtas];           // their |entry|^2 as ordered bits, and row
-  double2 prow[kNB][kNB];              // the block inverse's pivot rows, divided by their pivots
-  uint64_t bar[kNB], pbar[kNB];
-  int wtop[2][8];
+  float4 prow[2][kNB / 2];  // the pivot row, from the step's column on (by step parity)
+  int4 key[2];              // the four warps' largest |entry|^2 as ordered bits
   int win[kNB];
-  int abort;
+  int cand[kPanCand];
 };
 
+// Partial pivoting in FP32 on a CTA's candidate rows sm.cand (-1: none) over the
+// 32 columns from k0 on; the rows chosen, in order, to sm.win.  The rows come in
+// coalesced, through `stage` (256 x kStagePitch float2); then four warps keep two
+// rows per lane in registers.  Per column: a warp maximum, one over the four
+// warps, the chosen row to shared memory, and every lane eliminates its rows,
+// writing the result one register down, so that the column in hand is always
+// register 0 and the loop needs no unrolling.  A step is latency and the pivot
+// row's broadcast (256 bytes per lane, hence two rows per lane): 720 cycles on
+// average; 1230 with a row per thread in eight warps and every warp's best row
+// published before one barrier; 1830 with one exchange per column through a
+// cluster of eight CTAs, which saves the second round (the same 9.5 ms per
+// impurity step at N_c = 1500, but 542 us against 470 at N_c = 80).
+__device__ __forceinline__ void choose_rows(PanSmem& sm, float2* stage, const double2* __restrict__ A, int np, int n,
+                                            int k0) {
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int ncol = min(kNB, n - k0);
+#pragma unroll 8
+  for (int r = warp; r < kPanCand; r += kPanThreads / 32) {
+    const int row = sm.cand[r];
+    const float2 f = narrow(A[(size_t)max(row, k0) * np + k0 + lane]);  // loaded either way: the loads overlap
+    stage[r * kStagePitch + lane] = row >= 0 && lane < ncol ? f : make_float2(0.f, 0.f);
+  }
+  if (t < kNB) sm.win[t] = -1;
+  __syncthreads();
+  if (warp < 4) {
+    float2 v[2][kNB];
+    bool live[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = 64 * warp + 32 * h + lane;
+      live[h] = sm.cand[r] >= 0;
+#pragma unroll
+      for (int e = 0; e < kNB; ++e) v[h][e] = stage[r * kStagePitch + e];
+    }
+    // columns past the panel's shift in as zeros: after 16 and 24 steps half and a quarter of the registers are left
+    auto steps = [&](auto width, int j0, int j1) {
+      constexpr int W = decltype(width)::value;
+#pragma unroll 1
+      for (int j = j0; j < j1; ++j) {
+        const int sb = j & 1;
+        // |entry|^2 as ordered bits, -1 below every magnitude; a NaN is never chosen
+        const float m0 = v[0][0].x * v[0][0].x + v[0][0].y * v[0][0].y;
+        const float m1 = v[1][0].x * v[1][0].x + v[1][0].y * v[1][0].y;
+        const int k_0 = live[0] && m0 >= 0.f ? __float_as_int(m0) : -1;
+        const int k_1 = live[1] && m1 >= 0.f ? __float_as_int(m1) : -1;
+        const bool second = k_1 > k_0;
+        const int key = second ? k_1 : k_0;
+        const int top = __reduce_max_sync(0xffffffffu, key);
+        const int src = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
+        if (lane == src) (&sm.key[sb].x)[warp] = top;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        const int4 y = sm.key[sb];
+        const int best = max(max(y.x, y.y), max(y.z, y.w));
+        const int wtop = best == y.x ? 0 : best == y.y ? 1 : best == y.z ? 2 : 3;
+        if (warp == wtop && lane == src) {
+          if (second) {
+#pragma unroll
+            for (int e = 0; e < W / 2; ++e)
+              sm.prow[sb][e] = make_float4(v[1][2 * e].x, v[1][2 * e].y, v[1][2 * e + 1].x, v[1][2 * e + 1].y);
+            live[1] = false;
+          } else {
+#pragma unroll
+            for (int e = 0; e < W / 2; ++e)
+              sm.prow[sb][e] = make_float4(v[0][2 * e].x, v[0][2 * e].y, v[0][2 * e + 1].x, v[0][2 * e + 1].y);
+            live[0] = false;
+          }
+          if (best >= 0) sm.win[j] = sm.cand[64 * warp + (second ? 32 : 0) + lane];  // else none left, or none finite
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        const float4* pr = sm.prow[sb];
+        const float4 p0 = pr[0];
+        const float pm = p0.x * p0.x + p0.y * p0.y;
+        float rm;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rm) : "f"(pm));
+        rm = pm > 1e-37f ? rm : 0.f;
+        float2 f[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          f[h] = make_float2((v[h][0].x * p0.x + v[h][0].y * p0.y) * rm, (v[h][0].y * p0.x - v[h][0].x * p0.y) * rm);
+#pragma unroll
+        for (int e = 0; e < W / 2; ++e) {
+          const float4 z = e == 0 ? p0 : pr[e];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (e > 0) v[h][2 * e - 1] = make_float2(fmaf(-f[h].x, z.x, fmaf(f[h].y, z.y, v[h][2 * e].x)),
+                                                     fmaf(-f[h].x, z.y, fmaf(-f[h].y, z.x, v[h][2 * e].y)));
+            v[h][2 * e] = make_float2(fmaf(-f[h].x, z.z, fmaf(f[h].y, z.w, v[h][2 * e + 1].x)),
+                                      fmaf(-f[h].x, z.w, fmaf(-f[h].y, z.z, v[h][2 * e + 1].y)));
+          }
+        }
+        v[0][W - 1] = v[1][W - 1] = make_float2(0.f, 0.f);
+      }
+    };
+    steps(std::integral_constant<int, 32>{}, 0, min(ncol, 16));
+    steps(std::integral_constant<int, 16>{}, 16, min(ncol, 24));
+    steps(std::integral_constant<int, 8>{}, 24, ncol);
+  }
+  __syncthreads();
+}
+
 // Pivot choice for the 32 columns from k0 on and, in the last round, the block's
-// inverse, on a cluster of eight CTAs.
-// Choice: partial pivoting in FP32 on up to 2048 candidate rows (rows k0 + i, or
-// in[i]), a thread per row with its entries in registers.  Per column: a warp
-// maximum, one over the warps, then the CTA's row goes to all eight CTAs'
-// shared memory (st.async, counted on the receivers' barrier of that step), every
-// thread picks the largest of the eight and eliminates its row, writing the
-// result one register down, so that the column in hand is always register 0 and
-// the loop needs no unrolling (unrolled with a row per thread, 200 KB of code
-// used once, the fetching alone bound it: 55 us per round of 256 rows; a warp
-// per R rows with two shuffles per row and a cluster barrier per column, 63 us
-// for R = 1 with the inverse, 88 for R = 6).
-// Last round: P = inv of the chosen rows' block in FP64, four rows per CTA, a
-// warp per row, the next pivot row first and sent the same way; its digits (the
-// B operand of gj64_rpanel_kernel); the row exchanges; the row permutation.
-// Every step has buffers and a barrier of its own, so nothing waits for a slot.
-// Both parts are latency bound, 32 exchanges each.
-__global__ void __cluster_dims__(kPanCtas, 1, 1) __launch_bounds__(256, 1)
+// inverse.  A tournament: each CTA of a cluster chooses 32 of its 256 candidate
+// rows (rows k0 + i, or in[i]), then the cluster's first CTA 32 of those.  Last
+// round: P = inv of the chosen rows' block and its digits, the row exchanges, the
+// row permutation.  Latency bound throughout.
+__global__ void __launch_bounds__(kPanThreads, 1)
     gj64_panel_kernel(const double2* __restrict__ A, int np, int n, int k0, const int* __restrict__ in, int count,
                       int* __restrict__ out, int last, double2* __restrict__ Pbuf, __nv_bfloat16* __restrict__ pimg,
                       int* __restrict__ pexp, RowSwaps* __restrict__ sw, int* __restrict__ rowperm, int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  PanSmem& sm = *reinterpret_cast<PanSmem*>(smem_raw);
-  volatile int* abort_flag = &sm.abort;
-  const int q = (int)cluster_ctarank(), c = blockIdx.x / kPanCtas;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nwarp = blockDim.x >> 5;
-  const int per = kPanCtas * blockDim.x, base = c * per, here = min(count - base, per);
-  const int ncol = min(kNB, n - k0), steps = min(ncol, here);
-  if (t < kNB) {
-    mbar_init(&sm.bar[t], 1);
-    mbar_init(&sm.pbar[t], 1);
-    fence_barrier_init();
-    mbar_arrive_expect_tx(&sm.bar[t], kPanCtas * (kNB * 8 + 16));
-    mbar_arrive_expect_tx(&sm.pbar[t], kNB * 16);
-    sm.win[t] = -1;
-  }
-  if (t == 0) sm.abort = 0;
-  const int i = base + q * (int)blockDim.x + t;
-  const int row = i < base + here ? (in ? in[i] : k0 + i) : -1;
-  float2 v[kNB];
-#pragma unroll
-  for (int e = 0; e < kNB; ++e) {
-    v[e] = make_float2(0.f, 0.f);
-    if (row >= 0 && e < ncol) {
-      const double2 z = A[(size_t)row * np + k0 + e];
-      v[e] = make_float2((float)z.x, (float)z.y);
-    }
-  }
-  bool live = row >= 0;
+  BlockSmem& blk = *reinterpret_cast<BlockSmem*>(smem_raw);
+  PanSmem& sm = *reinterpret_cast<PanSmem*>(smem_raw + (sizeof(BlockSmem) + 127) / 128 * 128);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  uint32_t nq;
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(nq));
+  const int q = (int)cluster_ctarank();
+  float2* stage = reinterpret_cast<float2*>(smem_raw);
+  const int i = blockIdx.x * kPanCand + t;
+  sm.cand[t] = i < count ? (in ? in[i] : k0 + i) : -1;
   __syncthreads();
-  cluster_barrier();  // every CTA's barriers are set before another counts on them
-#pragma unroll 1
-  for (int j = 0; j < steps; ++j) {
-    // largest |entry|^2, as ordered bits (-1 below every magnitude; a NaN is never chosen)
-    const float m = v[0].x * v[0].x + v[0].y * v[0].y;
-    const int key = live && m >= 0.f ? __float_as_int(m) : -1;
-    const int wk = __reduce_max_sync(0xffffffffu, key);
-    if (lane == 0) sm.wtop[j & 1][warp] = wk;
+  choose_rows(sm, stage, A, np, n, k0);
+  if (nq > 1) {
+    cluster_barrier();  // the first CTA has read its own candidates
+    if (t < kNB)
+      asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(cluster_addr(&sm.cand[q * kNB + t], 0)), "r"(sm.win[t])
+                   : "memory");
+    cluster_barrier();
+    if (q > 0) return;
+    if (t >= (int)nq * kNB) sm.cand[t] = -1;
     __syncthreads();
-    const int x = lane < nwarp ? sm.wtop[j & 1][lane] : -1;
-    const int top = __reduce_max_sync(0xffffffffu, x);
-    const int wtop = __ffs(__ballot_sync(0xffffffffu, x == top)) - 1;
-    if (warp == wtop) {
-      const int src = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
-      float4* mine = sm.row[j][q];
-      if (lane == src) {
-#pragma unroll
-        for (int e = 0; e < kNB / 2; ++e) mine[e] = make_float4(v[2 * e].x, v[2 * e].y, v[2 * e + 1].x, v[2 * e + 1].y);
-      }
-      const int srow = __shfl_sync(0xffffffffu, row, src);
-      __syncwarp();
-      // lane: CTA lane / 4, a quarter of the row (its own CTA's copy is rewritten with the same values)
-      const uint32_t d = lane >> 2;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float4 z = mine[4 * (lane & 3) + e];
-        st_async(&mine[4 * (lane & 3) + e], &sm.bar[j], d,
-                 make_uint4(__float_as_uint(z.x), __float_as_uint(z.y), __float_as_uint(z.z), __float_as_uint(z.w)));
-      }
-      if (lane < kPanCtas)
-        st_async(&sm.cand[j][q], &sm.bar[j], lane, make_uint4((uint32_t)top, (uint32_t)srow, 0u, 0u));
-    }
-    mbar_wait(&sm.bar[j], 0, abort_flag);  // after a failed wait the steps run on without waiting; rows are checked
-    const uint4 y = sm.cand[j][lane & (kPanCtas - 1)];
-    const int best = __reduce_max_sync(0xffffffffu, (int)y.x);
-    const int qtop = __ffs(__ballot_sync(0xffffffffu, (int)y.x == best)) - 1;
-    const int wrow = (int)sm.cand[j][qtop].y;
-    if (t == 0) sm.win[j] = best >= 0 && wrow >= k0 && wrow < n ? wrow : -1;  // -1: none left, or none finite
-    if (best >= 0 && row == wrow) live = false;
-    const float4* pr = sm.row[j][qtop];
-    const float4 p0 = pr[0];
-    const float pm = p0.x * p0.x + p0.y * p0.y;
-    float rm;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rm) : "f"(pm));
-    rm = pm > 1e-37f ? rm : 0.f;
-    const float2 f = make_float2((v[0].x * p0.x + v[0].y * p0.y) * rm, (v[0].y * p0.x - v[0].x * p0.y) * rm);
-#pragma unroll
-    for (int e = 0; e < kNB / 2; ++e) {
-      const float4 z = e == 0 ? p0 : pr[e];
-      if (e > 0) v[2 * e - 1] = make_float2(fmaf(-f.x, z.x, fmaf(f.y, z.y, v[2 * e].x)),
-                                            fmaf(-f.x, z.y, fmaf(-f.y, z.x, v[2 * e].y)));
-      v[2 * e] = make_float2(fmaf(-f.x, z.z, fmaf(f.y, z.w, v[2 * e + 1].x)),
-                             fmaf(-f.x, z.w, fmaf(-f.y, z.z, v[2 * e + 1].y)));
-    }
-    v[kNB - 1] = make_float2(0.f, 0.f);
+    choose_rows(sm, stage, A, np, n, k0);
   }
-  __syncthreads();
   if (!last) {
-    if (q == 0 && t < kNB) out[c * kNB + t] = sm.win[t];
-  } else if (warp < 4) {
-    // P = inv of the chosen block, row r of it in warp r & 3 of CTA r / 4
-    const int pr = 4 * q + warp;
-    double2 z = A[(size_t)(sm.win[pr] >= 0 ? sm.win[pr] : k0 + pr) * np + k0 + lane];
-    auto publish = [&](int k) {
-      const double2 d = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
-      double2 pinv;
-      if (!recip(d, pinv) && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
-      z = lane == k ? pinv : cmul(z, pinv);
-      const uint4 w = make_uint4((uint32_t)__double2loint(z.x), (uint32_t)__double2hiint(z.x),
-                                 (uint32_t)__double2loint(z.y), (uint32_t)__double2hiint(z.y));
-#pragma unroll
-      for (uint32_t d8 = 0; d8 < (uint32_t)kPanCtas; ++d8) st_async(&sm.prow[k][lane], &sm.pbar[k], d8, w);
-    };
-    if (pr == 0) publish(0);
-    for (int k = 0; k < kNB; ++k) {
-      if (pr == k) continue;
-      if (!__all_sync(0xffffffffu, mbar_wait(&sm.pbar[k], 0, abort_flag))) break;
-      const double2 rb = sm.prow[k][lane];
-      const double2 f = make_double2(__shfl_sync(0xffffffffu, z.x, k), __shfl_sync(0xffffffffu, z.y, k));
-      const double2 o = lane == k ? make_double2(0.0, 0.0) : z;
-      z = make_double2(fma(-f.x, rb.x, fma(f.y, rb.y, o.x)), fma(-f.x, rb.y, fma(-f.y, rb.x, o.y)));
-      if (pr == k + 1) publish(k + 1);
-    }
-    Pbuf[pr * kNB + lane] = z;
-    // digits of rows 2 pr = [Re | -Im] and 2 pr + 1 = [Im | Re], two columns per even lane
-    const unsigned m = __reduce_max_sync(0xffffffffu, max(mag_hi(z.x), mag_hi(z.y)));
-    const int be = row_biased(m);
-    if (m >= 0x7ff00000u && lane == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
-    if (lane == 0) pexp[pr] = be - 1022;
-    const long long yr = digit_word(z.x, be), yi = digit_word(z.y, be);
-    const long long yr1 = __shfl_down_sync(0xffffffffu, yr, 1), yi1 = __shfl_down_sync(0xffffffffu, yi, 1);
-    if ((lane & 1) == 0) {
-      const long long y[8] = {yr, yr1, yi, yi1, 0, 0, 0, 0};
-      const int o_re = core_off(2 * pr, lane), o_im = core_off(2 * pr, 32 + lane);
-      put_digits(y, [&](int s, uint4 w) {
-        __nv_bfloat16* d = pimg + s * 64 * kK;
-        *reinterpret_cast<uint32_t*>(d + o_re) = w.x;
-        *reinterpret_cast<uint32_t*>(d + o_im) = w.y ^ 0x80008000u;
-        *reinterpret_cast<uint32_t*>(d + o_re + 8) = w.y;
-        *reinterpret_cast<uint32_t*>(d + o_im + 8) = w.x;
-      });
-    }
-    if (pr == 0) {
-      // place k0 + lane takes row w; a winner from outside the block leaves its
-      // place to a row of the block that was not chosen (the t-th such place gets
-      // the t-th such row)
-      const int w = sm.win[lane] >= 0 ? sm.win[lane] : k0 + lane;
-      const bool inside = w >= k0 && w < k0 + kNB;
-      if (sm.win[lane] < 0 && k0 + lane < n && status) atomicCAS(status, 0, DS_SINGULAR);  // too few candidates
-      const unsigned chosen = __reduce_or_sync(0xffffffffu, inside ? 1u << (w - k0) : 0u);
-      const unsigned outs = __ballot_sync(0xffffffffu, !inside);
-      const int at = __popc(outs & ((1u << lane) - 1u));
-      unsigned left = ~chosen;
-      for (int u = 0; u < at; ++u) left &= left - 1;  // drop the lowest
-      const int from = k0 + __ffs(left) - 1;
-      const int pw = rowperm[w], pf = inside ? 0 : rowperm[from];
-      __syncwarp();
-      rowperm[k0 + lane] = pw;
-      sw->win[lane] = w;
-      if (!inside) {
-        rowperm[w] = pf;
-        sw->to[at] = w;
-        sw->from[at] = from;
-      }
-      if (lane == 0) sw->moved = __popc(outs);
-    }
+    if (t < kNB) out[(blockIdx.x / nq) * kNB + t] = sm.win[t];
+    return;
   }
-  __syncthreads();
-  if (t == 0 && sm.abort && status) atomicCAS(status, 0, DS_TIMEOUT);
-  cluster_barrier();  // nobody leaves while another may still write to it
+  invert_block(blk, [&](int k) { return A + (size_t)(sm.win[k] >= 0 ? sm.win[k] : k0 + k) * np + k0; }, 0, Pbuf, pimg,
+               pexp, status);
+  if (warp == 0) {
+    // place k0 + lane takes row w; a winner from outside the block leaves its
+    // place to a row of the block that was not chosen (the t-th such place gets
+    // the t-th such row)
+    const int w = sm.win[lane] >= 0 ? sm.win[lane] : k0 + lane;
+    const bool inside = w >= k0 && w < k0 + kNB;
+    if (sm.win[lane] < 0 && k0 + lane < n && status) atomicCAS(status, 0, DS_SINGULAR);  // too few candidates
+    const unsigned chosen = __reduce_or_sync(0xffffffffu, inside ? 1u << (w - k0) : 0u);
+    const unsigned outs = __ballot_sync(0xffffffffu, !inside);
+    const int at = __popc(outs & ((1u << lane) - 1u));
+    unsigned left = ~chosen;
+    for (int u = 0; u < at; ++u) left &= left - 1;  // drop the lowest
+    const int from = k0 + __ffs(left) - 1;
+    const int pw = rowperm[w], pf = inside ? 0 : rowperm[from];
+    __syncwarp();
+    rowperm[k0 + lane] = pw;
+    sw->win[lane] = w;
+    if (!inside) {
+      rowperm[w] = pf;
+      sw->to[at] = w;
+      sw->from[at] = from;
+    }
+    if (lane == 0) sw->moved = __popc(outs);
+  }
 }
+
+static_assert(kPanCand * kStagePitch * sizeof(float2) <= sizeof(BlockSmem), "candidate rows are staged in the block's space");
+constexpr int kPanSmem = (int)((sizeof(BlockSmem) + 127) / 128 * 128 + sizeof(PanSmem));
 
 int launch_panel(const double2* A, int np, int n, int k0, const int* in, int count, int* out, bool last, double2* pbuf,
                  __nv_bfloat16* pimg, int* pexp, RowSwaps* sw, int* rowperm, int* status, cudaStream_t s) {
-  // a thread per candidate row over the cluster's eight CTAs, 128 to 256 threads each
-  int threads = ceil_div(count < kPanRows ? count : kPanRows, kPanCtas * 32) * 32;
-  if (threads < 128) threads = 128;
-  gj64_panel_kernel<<<ceil_div(count, kPanCtas * threads) * kPanCtas, threads, sizeof(PanSmem), s>>>(
-      A, np, n, k0, in, count, out, last, pbuf, pimg, pexp, sw, rowperm, status);
-  NED_LAUNCH_CHECK("gj64_panel_kernel");
+  // 256 candidate rows per CTA: clusters of 1, 2, 4 or 8 CTAs, the fewest that hold them
+  int ctas = 1;
+  while (ctas < kPanCtas && ctas * kPanCand < count) ctas *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ceil_div(count, ctas * kPanCand) * ctas);
+  cfg.blockDim = dim3(kPanThreads);
+  cfg.dynamicSmemBytes = kPanSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = ctas;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  NED_CUDA(cudaLaunchKernelEx(&cfg, gj64_panel_kernel, A, np, n, k0, in, count, out, (int)last, pbuf, pimg, pexp, sw,
+                              rowperm, status));
+  instr_count();
   return NEDMFT_OK;
 }
 
@@ -1398,7 +1427,7 @@ int pivot_inverse_prepare() {
   LookAhead* la = nullptr;
   int rc = look_ahead(&la), sms = 0;
   if (!rc) rc = device_sm_count(&sms);
-  if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_panel_kernel), (int)sizeof(PanSmem));
+  if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_panel_kernel), kPanSmem);
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_rpanel_kernel), RSmem::kBytes);
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_update_kernel), USmem::kBytes);
   return rc;
