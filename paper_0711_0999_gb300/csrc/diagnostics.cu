@@ -98,8 +98,12 @@ __global__ void __launch_bounds__(32 * kDosWarps)
       }
     }
     if (l0 < cnt) {
-      sincos(om * ((k0 + l0) * h), &ls, &lc);
-      im += lc * p.y + ls * p.x;  // Im(e^{i om s} G^R)
+      // one phase for B terms: the rounding of its angle, which they would share, is put back
+      const double k = (double)(k0 + l0), t = k * h, te = fma(k, h, -t);
+      const double an = om * t, ae = fma(om, t, -an) + om * te;
+      sincos(an, &ls, &lc);
+      const double s1 = fma(lc, ae, ls), c1 = fma(-ls, ae, lc);
+      im += c1 * p.y + s1 * p.x;  // Im(e^{i om s} G^R)
     }
   }
 #pragma unroll

@@ -44,13 +44,20 @@ __global__ void norm_pass1(const double2* __restrict__ a, const double2* __restr
 }
 
 __global__ void norm_pass2(const double* __restrict__ part, int nblocks, double* __restrict__ err) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  // one warp: strided loads, then a warp maximum (49 us with one thread over the 304 pairs)
+  const int lane = threadIdx.x;
   double md = 0.0, ma = 0.0;
-  for (int i = 0; i < nblocks; ++i) {
+#pragma unroll 4
+  for (int i = lane; i < nblocks; i += 32) {
     md = fmax(md, part[2 * i]);
     ma = fmax(ma, part[2 * i + 1]);
   }
-  *err = ma > 0.0 ? md / ma : (md > 0.0 ? INFINITY : 0.0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    md = fmax(md, __shfl_xor_sync(0xffffffffu, md, o));
+    ma = fmax(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+  }
+  if (lane == 0) *err = ma > 0.0 ? md / ma : (md > 0.0 ? INFINITY : 0.0);
 }
 
 struct DmftLayout {

@@ -42,14 +42,14 @@ __global__ void imp_build_kernel(ContourDev c, ModelDev m, const double2* __rest
 }
 
 // sigma_new = W^-1 [-w1 D + w1 (1 - w1) D X_h D] W^-1 with X_h = inv(A_h); if
-// g is given, g = A0 - W sigma_new W (= inv(G_imp)).  16 rows of 256 columns per
+// g is given, g = A0 - W sigma_new W (= inv(G_imp)).  Four rows of 256 columns per
 // CTA: the factors d_i / W_i and d_{j+1} / W_j are formed once per row and
 // column, so an entry costs two complex products (240 us at N_c = 1500 when
 // every entry formed and divided by W_i W_j in FP64).
+constexpr int kRowsPer = 4;
 __global__ void __launch_bounds__(256) imp_sigma_kernel(ContourDev c, ModelDev m, const double2* __restrict__ xh,
                                                         const double2* __restrict__ a0,
                                                         double2* __restrict__ sigma_new, double2* __restrict__ g) {
-  constexpr int kRowsPer = 16;
   __shared__ double2 fi[kRowsPer];
   const int n = c.n, i0 = blockIdx.y * kRowsPer;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,7 +127,7 @@ extern "C" int nedmft_impurity_update(const nedmft_contour* c, const nedmft_mode
   imp_build_kernel<<<bx, 256, 0, st>>>(cd, md, reinterpret_cast<const double2*>(sigma_d), a0, ah);
   NED_LAUNCH_CHECK("imp_build_kernel");
   if ((rc = pivot_inverse(ah, n, pws, st, status))) return rc;  // ah = X_h = inv(A_h)
-  imp_sigma_kernel<<<dim3(ceil_div(n, 256), ceil_div(n, 16)), 256, 0, st>>>(
+  imp_sigma_kernel<<<dim3(ceil_div(n, 256), ceil_div(n, kRowsPer)), 256, 0, st>>>(
       cd, md, ah, a0, reinterpret_cast<double2*>(sigma_new_d), gimp_d ? g : nullptr);
   NED_LAUNCH_CHECK("imp_sigma_kernel");
   if (gimp_d) {

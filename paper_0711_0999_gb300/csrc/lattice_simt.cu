@@ -201,49 +201,54 @@ int launch_gj_small_fp64(const ContourDev& c, const ModelDev& m, const double* e
 
 // ------------------------------------------------------------------ FP64 reductions over the points
 
-// gloc[i][j] (= or +=) sum_b wq[q0+b] X[b][i][col(j)], b ascending, col =
-// unshift_col if `cycled` (the batch holds X' = (P A)^-1).  A thread per entry
-// with eight matrices' loads in flight, the weights of 256 points at a time in
-// shared memory; small blocks, so that an 80 x 80 result covers the SMs (100 us
-// with one load in flight and 25 blocks, 256 points of 80 x 80).
-constexpr int kRedPts = 256;
-__global__ void __launch_bounds__(128) reduce_gloc_kernel(ContourDev c, ModelDev m, const double* __restrict__ eps_d,
-                                                          const double* __restrict__ wq_d, int q0, int nb,
-                                                          const double2* __restrict__ X, int ldx, bool cycled,
-                                                          bool first, double2* __restrict__ gloc) {
-  __shared__ double w[kRedPts];
-  __shared__ bool sh[kRedPts];
+// gloc[i][j] (= or +=) sum_b wq[q0+b] X[b][i][col(j)], col = unshift_col if
+// `cycled` (the batch holds X' = (P A)^-1).  32 consecutive entries per CTA, a
+// warp per eighth of the points: each sums its consecutive points in ascending
+// order with eight loads in flight, then the eighths are added in order (a fixed
+// order).  Bound by the loads' latency while the result is small: 135 us with a
+// thread per entry over all 256 points of 80 x 80.
+constexpr int kRedGroups = 8;
+__global__ void __launch_bounds__(32 * kRedGroups)
+    reduce_gloc_kernel(ContourDev c, ModelDev m, const double* __restrict__ eps_d, const double* __restrict__ wq_d,
+                       int q0, int nb, const double2* __restrict__ X, int ldx, bool cycled, bool first,
+                       double2* __restrict__ gloc) {
+  __shared__ double2 part[kRedGroups][32];
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const size_t total = (size_t)c.n * c.n, bstride = (size_t)ldx * ldx;
-  const size_t span = (size_t)gridDim.x * blockDim.x;
-  for (size_t e0 = (size_t)blockIdx.x * blockDim.x; e0 < total; e0 += span) {  // the same trips for a whole block
-    const size_t e = e0 + threadIdx.x;
-    const bool live = e < total;
-    const int i = (int)((live ? e : 0) / c.n), j = (int)((live ? e : 0) % c.n);
-    const size_t off0 = (size_t)i * ldx + j, off1 = (size_t)i * ldx + unshift_col(j, c.n, true);
-    double2 acc = first || !live ? make_double2(0.0, 0.0) : gloc[e];
-    for (int p0 = 0; p0 < nb; p0 += kRedPts) {
-      const int np = nb - p0 < kRedPts ? nb - p0 : kRedPts;
-      __syncthreads();
-      for (int b = threadIdx.x; b < np; b += blockDim.x) {
-        w[b] = wq_d[q0 + p0 + b];
-        sh[b] = cycled && shifted_point(m, eps_d[q0 + p0 + b]);
-      }
-      __syncthreads();
-      constexpr int U = 8;
-      for (int b0 = 0; b0 < np && live; b0 += U) {
-        double2 v[U];
+  const int b0 = (int)((long long)g * nb / kRedGroups), b1 = (int)((long long)(g + 1) * nb / kRedGroups);
+  for (size_t e0 = (size_t)blockIdx.x * 32; e0 < total; e0 += (size_t)gridDim.x * 32) {  // the same trips for a CTA
+    const size_t e = e0 + lane, ec = e < total ? e : 0;
+    const int i = (int)(ec / c.n), j = (int)(ec - (size_t)i * c.n);
+    const double2* x0 = X + (size_t)i * ldx + j;
+    const double2* x1 = X + (size_t)i * ldx + unshift_col(j, c.n, true);
+    double2 acc = make_double2(0.0, 0.0);
+    constexpr int U = 8;
+    for (int b = b0; b < b1; b += U) {
+      double2 v[U];
+      double w[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          v[u] = b0 + u < np ? X[(size_t)(p0 + b0 + u) * bstride + (sh[b0 + u] ? off1 : off0)] : make_double2(0.0, 0.0);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (b0 + u < np) {
-            acc.x = fma(w[b0 + u], v[u].x, acc.x);
-            acc.y = fma(w[b0 + u], v[u].y, acc.y);
-          }
+      for (int u = 0; u < U; ++u) {
+        const int q = min(b + u, b1 - 1);
+        const bool sh = cycled && shifted_point(m, eps_d[q0 + q]);
+        v[u] = (sh ? x1 : x0)[(size_t)q * bstride];
+        w[u] = wq_d[q0 + q];
       }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (b + u < b1) {
+          acc.x = fma(w[u], v[u].x, acc.x);
+          acc.y = fma(w[u], v[u].y, acc.y);
+        }
     }
-    if (live) gloc[e] = acc;
+    part[g][lane] = acc;
+    __syncthreads();
+    if (g == 0 && e < total) {
+      double2 s = first ? make_double2(0.0, 0.0) : gloc[e];
+#pragma unroll
+      for (int k = 0; k < kRedGroups; ++k) s = cadd(s, part[k][lane]);
+      gloc[e] = s;
+    }
+    __syncthreads();
   }
 }
 
@@ -298,9 +303,9 @@ int launch_reduce(const ContourDev& c, const ModelDev& m, const double* eps, con
                   int q0, int nb, const double2* X, int ldx, bool cycled, bool first, double2* gloc, double2* jacc,
                   cudaStream_t st) {
   const size_t total = (size_t)c.n * c.n;
-  const size_t blocks = (total + 127) / 128;
-  reduce_gloc_kernel<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 128, 0, st>>>(c, m, eps, wq, q0, nb, X, ldx,
-                                                                                   cycled, first, gloc);
+  const size_t blocks = (total + 31) / 32;
+  reduce_gloc_kernel<<<(int)(blocks < 152 * 32 ? blocks : 152 * 32), 32 * kRedGroups, 0, st>>>(
+      c, m, eps, wq, q0, nb, X, ldx, cycled, first, gloc);
   NED_LAUNCH_CHECK("reduce_gloc_kernel");
   if (jacc) {
     reduce_current_kernel<<<ceil_div(c.nt, 4), 128, 0, st>>>(c, m, eps, ebar, wq, q0, nb, X, ldx, cycled, first, jacc);
