@@ -1467,17 +1467,29 @@ __global__ void __launch_bounds__(256) oz_pack_sd_kernel(ContourDev c, const dou
 // <= kRefineTail * sum(w) (weights taken as w_q (1 + |eps| + |ebar|), which
 // also bounds the current's quadrature factor).  One CTA; bisection on the
 // threshold in log space.
+//
+// The weights are sorted in shared memory (bitonic) and summed up in that order:
+// the threshold lies below the first weight whose running sum exceeds the tail,
+// and the bisection, which fixes its last bits, only compares with that weight,
+// by logarithms until the interval is within 1e-9 of it.  (Every step of the
+// bisection summing the weights below its threshold took 840 us for 1024 points,
+// up to a quarter of a small lattice step.)  More points than the shared memory
+// holds are summed anew for every step.
+constexpr int kSelectMax = 8192;
 __global__ void __launch_bounds__(1024) refine_select_kernel(const double* __restrict__ eps,
                                                              const double* __restrict__ ebar,
-                                                             const double* __restrict__ wq, int nq,
+                                                             const double* __restrict__ wq, int nq, int npow,
                                                              int* __restrict__ flags) {
+  extern __shared__ double sorted[];  // npow values, a power of two >= nq, if it fits; else npow = 0
   __shared__ double red[1024];
+  __shared__ double sh_lo, sh_cut;
+  const int t = threadIdx.x;
   auto wt = [&](int q) { return fabs(wq[q]) * (1.0 + fabs(eps[q]) + fabs(ebar[q])); };
   auto block_sum = [&](double v) {
-    red[threadIdx.x] = v;
+    red[t] = v;
     __syncthreads();
     for (int s = 512; s > 0; s >>= 1) {
-      if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+      if (t < s) red[t] += red[t + s];
       __syncthreads();
     }
     const double r = red[0];
@@ -1485,22 +1497,71 @@ __global__ void __launch_bounds__(1024) refine_select_kernel(const double* __res
     return r;
   };
   double tot = 0.0;
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) tot += wt(q);
-  const double total = block_sum(tot);
+  for (int q = t; q < nq; q += blockDim.x) tot += wt(q);
+  const double total = block_sum(tot), tail = kRefineTail * total;
   double lo = -800.0, hi = 10.0;  // log2 of the threshold
-  for (int it = 0; it < 80; ++it) {
-    const double mid = 0.5 * (lo + hi);
-    const double th = exp2(mid);
-    double part = 0.0;
-    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-      const double w = wt(q);
-      if (w <= th) part += w;
+  if (npow) {
+    for (int q = t; q < npow; q += blockDim.x) sorted[q] = q < nq ? wt(q) : INFINITY;
+    __syncthreads();
+    for (int k = 2; k <= npow; k <<= 1)
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int i = t; i < npow / 2; i += blockDim.x) {
+          const int x = 2 * i - (i & (j - 1)), y = x + j;  // the pair whose indices differ in bit j
+          const double a = sorted[x], b = sorted[y];
+          if ((a > b) == ((x & k) == 0)) {
+            sorted[x] = b;
+            sorted[y] = a;
+          }
+        }
+        __syncthreads();
+      }
+    // running sums: every thread its run of weights, after the runs before it
+    const int per = (nq + 1023) / 1024, i0 = min(nq, t * per), i1 = min(nq, i0 + per);
+    double run = 0.0;
+    for (int i = i0; i < i1; ++i) run += sorted[i];
+    red[t] = run;
+    if (t == 0) sh_cut = isnan(tail) ? -1.0 : INFINITY;  // a NaN among the weights: nothing is skipped
+    __syncthreads();
+    for (int s = 1; s < 1024; s <<= 1) {  // inclusive scan
+      const double add = t >= s ? red[t - s] : 0.0;
+      __syncthreads();
+      red[t] += add;
+      __syncthreads();
     }
-    const double skipped = block_sum(part);
-    if (skipped <= kRefineTail * total) lo = mid; else hi = mid;
+    double sum = t > 0 ? red[t - 1] : 0.0;
+    for (int i = i0; i < i1; ++i) {  // one thread finds the first weight past the tail
+      const double next = sum + sorted[i];
+      if (sum <= tail && !(next <= tail)) sh_cut = sorted[i];
+      sum = next;
+    }
+    __syncthreads();
+    if (t == 0) {
+      const double cut = sh_cut, l2 = log2(cut);
+      for (int it = 0; it < 80; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (mid == lo || mid == hi) break;  // nothing moves any more
+        const bool below = mid < l2 - 1e-9 ? true : mid > l2 + 1e-9 ? false : exp2(mid) < cut;
+        if (below) lo = mid; else hi = mid;
+      }
+      sh_lo = lo;
+    }
+    __syncthreads();
+    lo = sh_lo;
+  } else {
+    for (int it = 0; it < 80; ++it) {
+      const double mid = 0.5 * (lo + hi);
+      const double th = exp2(mid);
+      double part = 0.0;
+      for (int q = t; q < nq; q += blockDim.x) {
+        const double w = wt(q);
+        if (w <= th) part += w;
+      }
+      const double skipped = block_sum(part);
+      if (skipped <= tail) lo = mid; else hi = mid;
+    }
   }
   const double th = exp2(lo);
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) flags[q] = wt(q) > th ? 1 : 0;
+  for (int q = t; q < nq; q += blockDim.x) flags[q] = wt(q) > th ? 1 : 0;
 }
 
 // Per matrix: the (B - S_sp) coefficients of every row in double-float,
@@ -2175,7 +2236,12 @@ int umma_prepare_shared(const ContourDev& c, const double2* S, int np, const dou
   NED_LAUNCH_CHECK("base_neg_s_kernel");
   oz_pack_sd_kernel<<<np, 256, 0, st>>>(c, S, np, r.sd_img, r.sd_slice, r.sd_exp);
   NED_LAUNCH_CHECK("oz_pack_sd_kernel");
-  refine_select_kernel<<<1, 1024, 0, st>>>(eps, ebar, wq, nq, r.flags);
+  int npow = 2;
+  while (npow < nq && npow <= kSelectMax) npow *= 2;
+  if (npow > kSelectMax) npow = 0;
+  if (int rc = ensure_dyn_smem(reinterpret_cast<const void*>(refine_select_kernel), kSelectMax * (int)sizeof(double)))
+    return rc;
+  refine_select_kernel<<<1, 1024, npow * sizeof(double), st>>>(eps, ebar, wq, nq, npow, r.flags);
   NED_LAUNCH_CHECK("refine_select_kernel");
   return NEDMFT_OK;
 }
