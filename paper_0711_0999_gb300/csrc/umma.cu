@@ -2220,7 +2220,12 @@ int umma_padded(int n, int width) {
 size_t umma_batch_bytes_per_matrix(int np, int width) {
   return gj_buffers_for(np, width).total + refine_layout(np, 1).total;
 }
-int umma_default_batch(int np) { return np <= 2048 ? 152 : 76; }
+// Points per batch: 152, one pivot block per SM at a time; three times that while
+// the matrices are small, where a launch's fixed cost and the last wave count
+// (1024 points, batches of 152 / 304 / 456: N_c = 100 2.04 / 1.85 / 1.78 ms, 400
+// 16.3 / 15.6 / 15.3, 700 33.1 / 32.0 / 31.6; 576 points of 1500 94.7 / 93.6 /
+// 93.7, not worth 60 GB of workspace); half above 2048 rows for the workspace.
+int umma_default_batch(int np) { return np <= 768 ? 456 : np <= 2048 ? 152 : 76; }
 size_t umma_shared_bytes(int np, int nq) {
   return align1k(kOzS * sizeof(__nv_bfloat16) * (size_t)np * 2 * np) + align1k(sizeof(int) * (size_t)np) +
          flags_bytes(nq) + align1k(sizeof(float2) * (size_t)np * np);
