@@ -49,6 +49,16 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
   while (!mbar_test(bar, parity) && global_ns() - t0 < kDrainNs) {
   }
 }
+// shared -> global bulk copy and FP64 reduction (add at L2), tracked by bulk groups
+__device__ __forceinline__ void bulk_store(double2* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_add_f64(double2* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f64 [%0], [%1], %2;" ::"l"(dst),
+               "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
 // eight TMEM columns of this warp's 32 lanes (wait with tmem_wait_ld)
 __device__ __forceinline__ void tmem_ld8(uint32_t addr, float (&v)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -228,7 +238,7 @@ __device__ __forceinline__ void pack_c_rows(const double2* __restrict__ A, int n
 #pragma unroll 8
   for (int r = warp; r < 128; r += kWarps) {
     const int g = mt * 128 + r;
-    double2 z = A[(size_t)(src ? src[r] : g) * np + k0 + lane];
+    double2 z = A[box_off(np, src ? src[r] : g, k0 + lane)];
     if (g >= k0 && g < k0 + kNB) z = make_double2(lane == g - k0 ? -1.0 : 0.0, 0.0);
     stage[r * kStageRow + lane] = z;
   }
@@ -578,16 +588,16 @@ __device__ __forceinline__ void write_p(const double2 (*prow)[kNB + 1], int b, d
   });
 }
 
-// P = inv of the block whose row k starts at row_of(k), by 256 threads, and its
+// P = inv of the block with entries entry(row, column), by 256 threads, and its
 // digits; all of the CTA's threads, with the shared memory to themselves.
-template <class RowOf>
-__device__ __forceinline__ void invert_block(BlockSmem& sm, RowOf&& row_of, int b, double2* __restrict__ Pbuf,
+template <class Entry>
+__device__ __forceinline__ void invert_block(BlockSmem& sm, Entry&& entry, int b, double2* __restrict__ Pbuf,
                                              __nv_bfloat16* __restrict__ pimg, int* __restrict__ pexp, int* status) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int r = t >> 3, c4 = 4 * (t & 7);
   double2 in[4], out[4];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) in[c] = row_of(r)[c4 + c];
+  for (int c = 0; c < 4; ++c) in[c] = entry(r, c4 + c);
   if (t == 0) {
     mbar_init(&sm.bar, 1);
     sm.abort = 0;
@@ -615,7 +625,7 @@ __device__ __forceinline__ void invert_block(BlockSmem& sm, RowOf&& row_of, int 
   } else {
     double2 v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = row_of(4 * warp + q)[lane];
+    for (int q = 0; q < 4; ++q) v[q] = entry(4 * warp + q, lane);
     fp64_inverse(v, *reinterpret_cast<double2 (*)[2][32]>(sm.x), status);
 #pragma unroll
     for (int q = 0; q < 4; ++q) prow[4 * warp + q][lane] = v[q];
@@ -633,9 +643,9 @@ __global__ void __launch_bounds__(256, 2)
                       int* __restrict__ cexp, int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   if ((int)blockIdx.x < nb) {
-    const double2* a = A + (size_t)blockIdx.x * np * np + (size_t)k0 * np + k0;
-    invert_block(*reinterpret_cast<BlockSmem*>(smem_raw), [&](int k) { return a + (size_t)k * np; }, blockIdx.x, Pbuf,
-                 pimg, pexp, status);
+    const double2* a = A + (size_t)blockIdx.x * np * np;
+    invert_block(*reinterpret_cast<BlockSmem*>(smem_raw), [&](int r, int c) { return a[box_off(np, k0 + r, k0 + c)]; },
+                 blockIdx.x, Pbuf, pimg, pexp, status);
     return;
   }
   const int u = blockIdx.x - nb, b = u / mtiles, mt = u % mtiles;
@@ -709,14 +719,14 @@ __global__ void __launch_bounds__(512, 1)
   if (t < 128) colmax[0][t] = colmax[1][t] = 0;
   if (warp == 0) tmem_alloc(&tmem_slot, kCols);
   double2 z[8];
-  double2* col = A + (size_t)b * np * np + j;
+  double2* mat = A + (size_t)b * np * np;
 #pragma unroll
-  for (int c = 0; c < 8; ++c) z[c] = col[(size_t)(sw ? sw->win[8 * h + c] : k0 + 8 * h + c) * np];
+  for (int c = 0; c < 8; ++c) z[c] = mat[box_off(np, sw ? sw->win[8 * h + c] : k0 + 8 * h + c, j)];
   tc_fence_before();
   __syncthreads();  // barriers, colmax, TMEM address; every row of A_K is read
   tc_fence_after();
   if (sw)
-    for (int e = h; e < sw->moved; e += 4) col[(size_t)sw->to[e] * np] = col[(size_t)sw->from[e] * np];
+    for (int e = h; e < sw->moved; e += 4) mat[box_off(np, sw->to[e], j)] = mat[box_off(np, sw->from[e], j)];
   const uint32_t tmem = tmem_slot;
   {
     unsigned m = 0;
@@ -855,7 +865,7 @@ static_assert(sizeof(UBars) <= USmem::kBars, "barrier block");
 // half of the boxes each way, 274 us; every other tile of six warps loaded in
 // 128-byte rows one tile ahead, 359 us.
 __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
-    gj64_update_kernel(const __grid_constant__ CUtensorMap amap, int np, int mtiles, int ntn, int total, int k0,
+    gj64_update_kernel(double2* __restrict__ A, int np, int mtiles, int ntn, int total, int k0,
                        int jskip, int nskip, const __nv_bfloat16* __restrict__ cimg, const int* __restrict__ cexp,
                        const __nv_bfloat16* __restrict__ rimg, const int* __restrict__ rexp, int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -1003,9 +1013,9 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) {
-        const int x = 2 * j, y = b * np + cur.mt * 128 + quarter * 32;
-        if (ik || (j >= k0 && j < k0 + kNB)) tma_store_2d(&amap, box, x, y);  // block K: nothing to add to
-        else tma_reduce_add_2d(&amap, box, x, y);
+        double2* dst = A + (size_t)b * np * np + box_off(np, i, j & ~7);  // lane 0: row 0 of the box
+        if (ik || (j >= k0 && j < k0 + kNB)) bulk_store(dst, box, kBoxBytes);  // block K: nothing to add to
+        else bulk_add_f64(dst, box, kBoxBytes);
         bulk_commit();
       }
       __syncwarp();
@@ -1020,31 +1030,6 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
     tmem_dealloc(tmem, kCols);
   }
   if (t == 0 && bars.abort && status) atomicCAS(status, 0, DS_TIMEOUT);
-}
-
-// The batch as one tensor of 2 np doubles per row, moved in boxes of four complex columns x 32 rows.
-int encode_f64_boxes(CUtensorMap* map, double2* base, uint64_t np, uint64_t rows) {
-  using Fn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                          const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                          CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static const Fn fn = [] {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      f = nullptr;
-    return reinterpret_cast<Fn>(f);
-  }();
-  if (!fn) return set_error(NEDMFT_ECUDA, "cuTensorMapEncodeTiled is not available from the CUDA driver");
-  const cuuint64_t dims[2] = {2 * np, rows};
-  const cuuint64_t strides[1] = {2 * np * sizeof(double)};
-  const cuuint32_t box[2] = {2 * kBoxCols, 32};
-  const cuuint32_t elem_strides[2] = {1, 1};
-  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, base, dims, strides, box, elem_strides,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return set_error(NEDMFT_ECUDA, "cuTensorMapEncodeTiled (FP64) failed (CUresult %d)", (int)r);
-  return NEDMFT_OK;
 }
 
 struct Gj64Layout {
@@ -1089,10 +1074,8 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
   __nv_bfloat16* rimg = reinterpret_cast<__nv_bfloat16*>(p); p += L.r;
   int* cexp = reinterpret_cast<int*>(p); p += L.ce;
   int* rexp = reinterpret_cast<int*>(p);
-  CUtensorMap map;
-  int rc = encode_f64_boxes(&map, A, np, (uint64_t)np * nb);
   int sms = 0;
-  if (!rc) rc = device_sm_count(&sms);
+  int rc = device_sm_count(&sms);
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_pivot_kernel), (int)sizeof(BlockSmem));
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_rpanel_kernel), RSmem::kBytes);
   if (!rc) rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj64_update_kernel), USmem::kBytes);
@@ -1107,7 +1090,7 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
     NED_LAUNCH_CHECK("gj64_rpanel_kernel");
     const int slot = instr_begin(st);
     gj64_update_kernel<<<total < sms ? total : sms, 64 + 32 * kEpiW, USmem::kBytes, st>>>(
-        map, np, mtiles, ntn, total, k0, ntn, 0, cimg, cexp, rimg, rexp, status);
+        A, np, mtiles, ntn, total, k0, ntn, 0, cimg, cexp, rimg, rexp, status);
     NED_LAUNCH_CHECK("gj64_update_kernel");
     const int live = n - k0 < kNB ? n - k0 : kNB;
     instr_end(slot, st, 8.0 * (double)n * n * live * nb, 2.0 * sizeof(double2) * (double)n * n * nb);
@@ -1155,7 +1138,7 @@ __device__ __forceinline__ void choose_rows(PanSmem& sm, float2* stage, const do
 #pragma unroll 8
   for (int r = warp; r < kPanCand; r += kPanThreads / 32) {
     const int row = sm.cand[r];
-    const float2 f = narrow(A[(size_t)max(row, k0) * np + k0 + lane]);  // loaded either way: the loads overlap
+    const float2 f = narrow(A[box_off(np, max(row, k0), k0 + lane)]);  // loaded either way: the loads overlap
     stage[r * kStagePitch + lane] = row >= 0 && lane < ncol ? f : make_float2(0.f, 0.f);
   }
   if (t < kNB) sm.win[t] = -1;
@@ -1272,8 +1255,8 @@ __global__ void __launch_bounds__(kPanThreads, 1)
     if (t < kNB) out[(blockIdx.x / nq) * kNB + t] = sm.win[t];
     return;
   }
-  invert_block(blk, [&](int k) { return A + (size_t)(sm.win[k] >= 0 ? sm.win[k] : k0 + k) * np + k0; }, 0, Pbuf, pimg,
-               pexp, status);
+  invert_block(blk, [&](int r, int c) { return A[box_off(np, sm.win[r] >= 0 ? sm.win[r] : k0 + r, k0 + c)]; }, 0, Pbuf,
+               pimg, pexp, status);
   if (warp == 0) {
     // place k0 + lane takes row w; a winner from outside the block leaves its
     // place to a row of the block that was not chosen (the t-th such place gets
@@ -1358,7 +1341,7 @@ __global__ void pad_identity_kernel(const double2* __restrict__ a, int n, double
       const double2 z = a[(size_t)i * n + j];
       v = make_double2(scalbn(z.x, sh), scalbn(z.y, sh));
     }
-    ap[(size_t)i * np + j] = v;
+    ap[box_off(np, i, j)] = v;
     if (i == 0) rowperm[j] = j;
   }
 }
@@ -1370,7 +1353,7 @@ __global__ void unpermute_kernel(const double2* __restrict__ x, int np, int n, c
   const int sh = -amax_exponent(amax);
   const int i = blockIdx.x;
   for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < n; c += gridDim.y * blockDim.x) {
-    const double2 z = x[(size_t)i * np + c];
+    const double2 z = x[box_off(np, i, c)];
     y[(size_t)i * n + rowperm[c]] = make_double2(scalbn(z.x, sh), scalbn(z.y, sh));
   }
 }
@@ -1463,8 +1446,6 @@ int pivot_inverse(double2* a, int n, void* ws, cudaStream_t st, int* status) {
   LookAhead* la = nullptr;
   int rc = look_ahead(&la);
   if (!rc) rc = pivot_inverse_prepare();
-  CUtensorMap map;
-  if (!rc) rc = encode_f64_boxes(&map, ap, np, np);
   int sms = 0;
   if (!rc) rc = device_sm_count(&sms);
   if (rc) return rc;
@@ -1479,7 +1460,7 @@ int pivot_inverse(double2* a, int n, void* ws, cudaStream_t st, int* status) {
     const int total = mtiles * tiles;
     if (total <= 0) return NEDMFT_OK;
     gj64_update_kernel<<<total < ctas ? total : ctas, 64 + 32 * kEpiW, USmem::kBytes, s>>>(
-        map, np, mtiles, tiles, total, k0, jskip, nskip, cimg, cexp, rimg, rexp, status);
+        ap, np, mtiles, tiles, total, k0, jskip, nskip, cimg, cexp, rimg, rexp, status);
     NED_LAUNCH_CHECK("gj64_update_kernel");
     return NEDMFT_OK;
   };

@@ -17,8 +17,16 @@ int small_path_max_n();
 int launch_gj_small_fp64(const ContourDev& c, const ModelDev& m, const double* eps, const double* ebar, int q0,
                          int nb, const double2* S, double2* out, int* status, cudaStream_t st);
 
-// Batched FP64 inverses on the tensor cores (gj64_umma.cu): nb matrices of np x np (np a multiple of 128, the
-// identity outside n x n), in place, scratch of gj64_scratch_bytes.
+// Element (i, j) of an np x np matrix of the FP64 tensor-core path: boxes of 32 rows x 8 columns, 4 KB each and
+// row-band major, so that the update adds a box by one contiguous bulk reduction; within a box a row's 128 bytes
+// with the columns exchanged by the row's low bits, the order in which a lane per row writes a box to shared memory
+// without bank conflicts.  Eight columns of a row from a multiple of 8 on stay one 128-byte line.
+__host__ __device__ __forceinline__ size_t box_off(int np, int i, int j) {
+  return ((size_t)(i >> 5) * (np >> 3) + (j >> 3)) * 256 + (i & 31) * 8 + ((j ^ i) & 7);
+}
+
+// Batched FP64 inverses on the tensor cores (gj64_umma.cu): nb matrices of np x np in that order (np a multiple of
+// 128, the identity outside n x n), in place, scratch of gj64_scratch_bytes.
 size_t gj64_scratch_bytes(int np, int nb);
 int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, cudaStream_t st);
 int gj64_set_wait_ns(uint64_t ns, cudaStream_t st);  // its bounded waits' limit on the current device

@@ -92,9 +92,10 @@ __global__ void __launch_bounds__(256) gen_a_kernel(ContourDev c, ModelDev m, co
   __syncthreads();
   for (int rr = warp; rr < kGenRows; rr += 8) {
     const int i = src_row[rr];
-    double2* dst = A + (size_t)b * np * np + (size_t)(r0 + rr) * np;
+    double2* dst = A + (size_t)b * np * np;
+    const int r = r0 + rr;
     if (i >= c.n) {  // padding
-      for (int j = lane; j < np; j += 32) dst[j] = make_double2(j == i ? 1.0 : 0.0, 0.0);
+      for (int j = lane; j < np; j += 32) dst[box_off(np, r, j)] = make_double2(j == i ? 1.0 : 0.0, 0.0);
       continue;
     }
     const double2* src = S + (size_t)i * c.n;
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(256) gen_a_kernel(ContourDev c, ModelDev m, co
         if (j == i) v.y += 1.0;
         if (j == js) v = cadd(v, sub[rr]);
       }
-      dst[j] = v;
+      dst[box_off(np, r, j)] = v;
     }
   }
 }
@@ -202,7 +203,7 @@ int launch_gj_small_fp64(const ContourDev& c, const ModelDev& m, const double* e
 // ------------------------------------------------------------------ FP64 reductions over the points
 
 // gloc[i][j] (= or +=) sum_b wq[q0+b] X[b][i][col(j)], col = unshift_col if
-// `cycled` (the batch holds X' = (P A)^-1).  32 consecutive entries per CTA, a
+// `cycled` (the batch holds X' = (P A)^-1 in boxes, box_off).  32 consecutive entries per CTA, a
 // warp per eighth of the points: each sums its consecutive points in ascending
 // order with eight loads in flight, then the eighths are added in order (a fixed
 // order).  Bound by the loads' latency while the result is small: 135 us with a
@@ -219,8 +220,8 @@ __global__ void __launch_bounds__(32 * kRedGroups)
   for (size_t e0 = (size_t)blockIdx.x * 32; e0 < total; e0 += (size_t)gridDim.x * 32) {  // the same trips for a CTA
     const size_t e = e0 + lane, ec = e < total ? e : 0;
     const int i = (int)(ec / c.n), j = (int)(ec - (size_t)i * c.n);
-    const double2* x0 = X + (size_t)i * ldx + j;
-    const double2* x1 = X + (size_t)i * ldx + unshift_col(j, c.n, true);
+    const double2* x0 = X + (cycled ? box_off(ldx, i, j) : (size_t)i * ldx + j);
+    const double2* x1 = X + (cycled ? box_off(ldx, i, unshift_col(j, c.n, true)) : 0);
     double2 acc = make_double2(0.0, 0.0);
     constexpr int U = 8;
     for (int b = b0; b < b1; b += U) {
@@ -273,8 +274,8 @@ __global__ void __launch_bounds__(128) reduce_current_kernel(ContourDev c, Model
   for (int b = lane; b < nb; b += 32) {
     const int q = q0 + b;
     const double eps = eps_d[q];
-    const double2 v = X[(size_t)b * ldx * ldx + (size_t)mm * ldx +
-                        unshift_col(jcol, c.n, cycled && shifted_point(mo, eps))];
+    const double2 v = X[(size_t)b * ldx * ldx + (cycled ? box_off(ldx, mm, unshift_col(jcol, c.n, shifted_point(mo, eps)))
+                                                        : (size_t)mm * ldx + jcol)];
     const double w = wq_d[q] * (ebar_d[q] * cs + eps * sn);
     part.x = fma(w, v.x, part.x);
     part.y = fma(w, v.y, part.y);
