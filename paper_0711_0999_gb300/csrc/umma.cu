@@ -822,8 +822,15 @@ struct EpiRPack {
 // the two 64 x 64 inversions unblocked (one barrier per pivot, 2 x 2 complex
 // entries per thread), the products by two halves of 512 threads (4 x 2
 // outputs each).
+// Bound by the FP32 pipe in the products (three operations per part and term, the order
+// and roundings of which are fixed: 93 of 230 thousand cycles, 74 at the pipe's rate) and by
+// the chain of pivots in the two inversions (118).  The image was read from rows 1024
+// bytes apart, every lane of a warp on the same bank (23.5 thousand cycles; 8.5 with rows two
+// entries longer and eight lanes on the eight rows of a core matrix): 456 blocks
+// 353 -> 335 us.
 constexpr int kPivH = kNb / 2;
-constexpr size_t kPivSmem = (size_t)(kNb * kNb + kPivH * kPivH) * sizeof(float2);  // 160 KB
+constexpr int kPivLd = kNb + 2;  // row stride: eight rows' 16-byte reads hit different banks
+constexpr size_t kPivSmem = (size_t)(kNb * kPivLd + kPivH * kPivH) * sizeof(float2);  // 162 KB
 
 struct alignas(16) PivShared {
   float4 rowb[2][2][kPivH / 2];  // [buffer][pivot row][column pair]
@@ -836,7 +843,7 @@ __device__ __forceinline__ float2 shfl_c(float2 v, int src) {
   return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-// unblocked in-place Gauss-Jordan of the 64 x 64 block of M (row stride kNb) at (o, o),
+// unblocked in-place Gauss-Jordan of the 64 x 64 block of M (row stride kPivLd) at (o, o),
 // two pivots per barrier: thread (warp w, lane l) holds rows 2w, 2w+1 x columns 2l, 2l+1,
 // so step s eliminates with the 2 x 2 pivot block P held by thread (s, s) (P^-1 by
 // two scalar pivots: p11 and the Schur complement p22 - p21 p11^-1 p12).  Warp s
@@ -851,7 +858,7 @@ __device__ __forceinline__ void piv_gj64(float2* M, int o, PivShared& sh) {
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) a[i][j] = M[(o + rr + i) * kNb + o + cc + j];
+    for (int j = 0; j < 2; ++j) a[i][j] = M[(o + rr + i) * kPivLd + o + cc + j];
   for (int s = 0; s < kPivH / 2; ++s) {
     const int buf = s & 1;
     if (lane == s)  // the rows' entries in the pivot columns, before the step
@@ -924,28 +931,42 @@ __device__ __forceinline__ void piv_gj64(float2* M, int o, PivShared& sh) {
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) M[(o + rr + i) * kNb + o + cc + j] = a[i][j];
+    for (int j = 0; j < 2; ++j) M[(o + rr + i) * kPivLd + o + cc + j] = a[i][j];
+}
+
+// a b with the roundings written out (one multiply and one fused multiply-add per
+// part), whatever the compiler makes of the code around it
+__device__ __forceinline__ float2 piv_mul(float2 a, float2 b) {
+  return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
 }
 
 // acc[a][c] = sum_{k0 <= k < k0 + kn} X[i0 + a][k] Y[k][j0 + c] (a < 4, c < 2)
 // for the 4 x 2 block of thread s (0 .. 511) of a 64 x 64 product (row
-// strides ldx, ldy): i0 = 4 (s / 32), j0 = 2 (s % 32), so a warp reads one X
-// entry per row (a broadcast) and one 512-byte row of Y per k.
+// strides ldx, ldy): i0 = 4 (s / 32), j0 = 2 (s % 32), so a warp reads two X
+// entries per row (a broadcast) for two k and one 512-byte row of Y per k.
 __device__ __forceinline__ void piv_mm(const float2* X, int ldx, const float2* Y, int ldy, int s, int k0, int kn,
                                        float2 (&acc)[4][2]) {
   const int i0 = 4 * (s >> 5), j0 = 2 * (s & 31);
 #pragma unroll
   for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = make_float2(0.f, 0.f);
-#pragma unroll 4
-  for (int k = k0; k < k0 + kn; ++k) {
-    const float4 y = *reinterpret_cast<const float4*>(Y + k * ldy + j0);
+#pragma unroll 2
+  for (int k = k0; k < k0 + kn; k += 2) {
+    float4 x2[4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const float2 x = X[(i0 + a) * ldx + k];
-      acc[a][0].x += x.x * y.x - x.y * y.y;
-      acc[a][0].y += x.x * y.y + x.y * y.x;
-      acc[a][1].x += x.x * y.z - x.y * y.w;
-      acc[a][1].y += x.x * y.w + x.y * y.z;
+    for (int a = 0; a < 4; ++a) x2[a] = *reinterpret_cast<const float4*>(X + (i0 + a) * ldx + k);
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      const float4 y = *reinterpret_cast<const float4*>(Y + (k + d) * ldy + j0);
+      const float2 y0 = make_float2(y.x, y.y), y1 = make_float2(y.z, y.w);
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const float2 x = d ? make_float2(x2[a].z, x2[a].w) : make_float2(x2[a].x, x2[a].y);
+        const float2 z0 = piv_mul(x, y0), z1 = piv_mul(x, y1);
+        acc[a][0].x = __fadd_rn(acc[a][0].x, z0.x);
+        acc[a][0].y = __fadd_rn(acc[a][0].y, z0.y);
+        acc[a][1].x = __fadd_rn(acc[a][1].x, z1.x);
+        acc[a][1].y = __fadd_rn(acc[a][1].y, z1.y);
+      }
     }
   }
 }
@@ -999,18 +1020,18 @@ __global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __res
                                                              size_t pslice, int* status) {
   extern __shared__ __align__(16) float2 piv_smem[];
   __shared__ PivShared sh;
-  float2* M = piv_smem;               // A_KK, row stride kNb
-  float2* T = piv_smem + kNb * kNb;   // 64 x 64 temporary
+  float2* M = piv_smem;                 // A_KK, row stride kPivLd
+  float2* T = piv_smem + kNb * kPivLd;  // 64 x 64 temporary
   float2* B11 = M;
   float2* B12 = M + kPivH;
-  float2* B21 = M + kPivH * kNb;
-  float2* B22 = M + kPivH * kNb + kPivH;
+  float2* B21 = M + kPivH * kPivLd;
+  float2* B22 = M + kPivH * kPivLd + kPivH;
   const int b = blockIdx.x;
   const int t = threadIdx.x;
   const float2* src = A + (size_t)b * np * np;
   for (int e = t; e < kNb * kNb / 2; e += blockDim.x) {
     const int r = e / (kNb / 2), v = e % (kNb / 2);
-    *reinterpret_cast<float4*>(M + r * kNb + 2 * v) =
+    *reinterpret_cast<float4*>(M + r * kPivLd + 2 * v) =
         *reinterpret_cast<const float4*>(src + (size_t)(k0 + r) * np + k0 + 2 * v);
   }
   if (t == 0) sh.bad = 0;
@@ -1021,28 +1042,28 @@ __global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __res
   float2 u[4][2];
   piv_gj64(M, 0, sh);  // B11 <- P1
   __syncthreads();
-  piv_mm(B11, kNb, B12, kNb, s, 32 * half, 32, u);  // P1 A12
+  piv_mm(B11, kPivLd, B12, kPivLd, s, 32 * half, 32, u);  // P1 A12
   if (half) piv_put(T, kPivH, s, u);
   __syncthreads();
   if (!half) {
     piv_acc(T, kPivH, s, 1.f, u);
-    piv_put(B12, kNb, s, u);  // B12 <- P1 A12
+    piv_put(B12, kPivLd, s, u);  // B12 <- P1 A12
   }
   __syncthreads();
-  piv_mm(B21, kNb, half ? B11 : B12, kNb, s, 0, kPivH, u);  // A21 B12 | A21 P1
+  piv_mm(B21, kPivLd, half ? B11 : B12, kPivLd, s, 0, kPivH, u);  // A21 B12 | A21 P1
   __syncthreads();
   if (!half) {
     piv_neg(u);
-    piv_acc(B22, kNb, s, 1.f, u);
-    piv_put(B22, kNb, s, u);  // B22 <- A22 - A21 B12
+    piv_acc(B22, kPivLd, s, 1.f, u);
+    piv_put(B22, kPivLd, s, u);  // B22 <- A22 - A21 B12
   } else {
     piv_neg(u);
-    piv_put(B21, kNb, s, u);  // B21 <- -A21 P1
+    piv_put(B21, kPivLd, s, u);  // B21 <- -A21 P1
   }
   __syncthreads();
   piv_gj64(M, kPivH, sh);  // B22 <- X22
   __syncthreads();
-  piv_mm(B12, kNb, B22, kNb, s, 32 * half, 32, u);  // B12 X22
+  piv_mm(B12, kPivLd, B22, kPivLd, s, 32 * half, 32, u);  // B12 X22
   if (half) piv_put(T, kPivH, s, u);
   __syncthreads();
   if (!half) {
@@ -1051,30 +1072,30 @@ __global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __res
     piv_put(T, kPivH, s, u);  // V = -B12 X22
   }
   __syncthreads();
-  piv_mm(half ? T : B22, half ? kPivH : kNb, B21, kNb, s, 0, kPivH, u);  // X22 B21 | V B21
+  piv_mm(half ? T : B22, half ? kPivH : kPivLd, B21, kPivLd, s, 0, kPivH, u);  // X22 B21 | V B21
   __syncthreads();
   if (!half) {
-    piv_put(B21, kNb, s, u);  // B21 <- X22 B21
+    piv_put(B21, kPivLd, s, u);  // B21 <- X22 B21
     float2 v[4][2] = {};
     piv_acc(T, kPivH, s, 1.f, v);
-    piv_put(B12, kNb, s, v);  // B12 <- V
+    piv_put(B12, kPivLd, s, v);  // B12 <- V
   } else {
-    piv_acc(B11, kNb, s, 1.f, u);
-    piv_put(B11, kNb, s, u);  // B11 <- P1 + V B21
+    piv_acc(B11, kPivLd, s, 1.f, u);
+    piv_put(B11, kPivLd, s, u);  // B11 <- P1 + V B21
   }
   __syncthreads();
   if (sh.bad && t == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
-  // row r, k = 2c .. 2c + 31 for c = 16 g .. 16 g + 15: four 16-byte core-matrix rows per slice
+  // four entries per thread and pass: eight lanes take the eight rows of a 128-byte core
+  // matrix, their quads the core matrices beside it
   __nv_bfloat16* dst = pimg + b * pstride;
-  {
-    const int r = t >> 3, cg = 16 * (t & 7);
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      float2 z[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) z[q] = M[r * kNb + cg + 4 * h + q];
-      piv_store4(dst, pslice, img_offset(r, 2 * (cg + 4 * h), kKt), z);
-    }
+  for (int p = 0; p < 4; ++p) {
+    const int e = t + 1024 * p, r = 8 * (e >> 8) + (e & 7), c4 = 4 * ((e >> 3) & 31);
+    const float4* m = reinterpret_cast<const float4*>(M + r * kPivLd + c4);
+    const float4 z01 = m[0], z23 = m[1];
+    const float2 z[4] = {make_float2(z01.x, z01.y), make_float2(z01.z, z01.w), make_float2(z23.x, z23.y),
+                         make_float2(z23.z, z23.w)};
+    piv_store4(dst, pslice, img_offset(r, 2 * c4, kKt), z);
   }
 }
 
