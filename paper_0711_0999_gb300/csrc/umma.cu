@@ -819,125 +819,175 @@ struct EpiRPack {
 // Gauss-Jordan):
 //   B11 <- P1 = inv(A11);  B12 <- P1 A12;  B22 <- A22 - A21 B12;  B21 <- -A21 P1;
 //   B22 <- X22 = inv(B22); V = -B12 X22;  B21 <- X22 B21;  B11 <- P1 + V B21(old);  B12 <- V,
-// the two 64 x 64 inversions unblocked (one barrier per pivot, 2 x 2 complex
-// entries per thread), the products by two halves of 512 threads (4 x 2
-// outputs each).
+// the two 64 x 64 inversions unblocked by 16 warps, the products by two halves of 512
+// threads (4 x 2 outputs each).
 // Bound by the FP32 pipe in the products (three operations per part and term, the order
-// and roundings of which are fixed: 93 of 230 thousand cycles, 74 at the pipe's rate) and by
-// the chain of pivots in the two inversions (118).  The image was read from rows 1024
+// and roundings of which are fixed: 93 of 207 thousand cycles, 74 at the pipe's rate) and by
+// the chain of pivots in the two inversions (95).  The image was read from rows 1024
 // bytes apart, every lane of a warp on the same bank (23.5 thousand cycles; 8.5 with rows two
 // entries longer and eight lanes on the eight rows of a core matrix): 456 blocks
-// 353 -> 335 us.
+// 353 -> 335 us; 305 with the inversions' present form.
 constexpr int kPivH = kNb / 2;
 constexpr int kPivLd = kNb + 2;  // row stride: eight rows' 16-byte reads hit different banks
 constexpr size_t kPivSmem = (size_t)(kNb * kPivLd + kPivH * kPivH) * sizeof(float2);  // 162 KB
 
 struct alignas(16) PivShared {
-  float4 rowb[2][2][kPivH / 2];  // [buffer][pivot row][column pair]
-  float4 colb[2][kPivH];         // [buffer][row]: the row's two entries in the pivot columns
-  float4 pivb[2][2];             // [buffer][row of P^-1]
-  int bad;
+  float4 rowb[kPivH / 2][2][kPivH / 2];  // [step][pivot row][column pair]
+  float4 pivb[kPivH / 2][2];             // [step][row of P^-1]
+  uint64_t ready[kPivH / 2];             // the step's rows and P^-1 are written
+  int bad, abort;
 };
 
+// a b with the roundings written out (one multiply and one fused multiply-add per part;
+// Y: which of the two products of the imaginary part is the rounded one), whatever the
+// compiler makes of the code around it
+template <int Y = 0>
+__device__ __forceinline__ float2 piv_mul(float2 a, float2 b) {
+  return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)),
+                     Y ? __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)) : __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+// a b + c d
+template <int Y = 0>
+__device__ __forceinline__ float2 piv_mul2(float2 a, float2 b, float2 c, float2 d) {
+  const float2 u = piv_mul<Y>(a, b), v = piv_mul<Y>(c, d);
+  return make_float2(__fadd_rn(u.x, v.x), __fadd_rn(u.y, v.y));
+}
+// 1 / z; false (and a large finite value) below the pivot threshold
+__device__ __forceinline__ bool piv_inv(float2 z, float2& out) {
+  constexpr float tiny = 1e-6f;
+  const float m = __fmaf_rn(z.x, z.x, __fmul_rn(z.y, z.y));
+  if (!(m > tiny * tiny)) {  // also catches NaN
+    out = make_float2(1.f / tiny, 0.f);
+    return false;
+  }
+  const float r = __fdiv_rn(1.f, m);
+  out = make_float2(z.x * r, -z.y * r);
+  return true;
+}
 __device__ __forceinline__ float2 shfl_c(float2 v, int src) {
   return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-// unblocked in-place Gauss-Jordan of the 64 x 64 block of M (row stride kPivLd) at (o, o),
-// two pivots per barrier: thread (warp w, lane l) holds rows 2w, 2w+1 x columns 2l, 2l+1,
-// so step s eliminates with the 2 x 2 pivot block P held by thread (s, s) (P^-1 by
-// two scalar pivots: p11 and the Schur complement p22 - p21 p11^-1 p12).  Warp s
-// broadcasts its rows A_K with the pivot columns replaced by the identity and turns
-// them into P^-1 A_K (P^-1 in the pivot columns); every other row r takes
-// a[r][c] <- [c not a pivot column] a[r][c] - g_r rowb[:, c] with g_r = a[r][K] P^-1
-// (so its pivot columns become -g_r).
-__device__ __forceinline__ void piv_gj64(float2* M, int o, PivShared& sh) {
-  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  const int rr = 2 * w, cc = 2 * lane;
-  float2 a[2][2];
+// unblocked in-place Gauss-Jordan of the 64 x 64 block of M (row stride kPivLd) at (o, o)
+// by 16 warps, two pivots per step: lane group l / 8 of warp w holds row 2w, 2w + 1,
+// 32 + 2w or 33 + 2w, columns 16 j + 2c, 16 j + 2c + 1 (j < 4, c = l % 8).  Warp s % 16 owns
+// step s: it publishes its rows A_K with the pivot columns replaced by the identity and
+// the inverse of its 2 x 2 pivot block P (two scalar pivots: p11 and the Schur complement
+// p22 - p21 p11^-1 p12); the pivot rows become P^-1 A_K (P^-1 in the pivot columns), every
+// other row r takes a[r][c] <- [c not a pivot column] a[r][c] - g_r rowb[:, c] with
+// g_r = a[r][K] P^-1 (so its pivot columns become -g_r).
+// The chain of steps is what bounds it.  A warp waits for nothing but the step's rows
+// (no barrier), and the next step's owner updates its pivot columns first, then forms P^-1
+// (two reciprocals in a row) between the updates of its other columns.  Every step has its own
+// buffers (33 KB), so no write waits for a reader.  95 thousand cycles for a block's two
+// inversions; 118 with 32 warps, 2 x 2 entries a lane and one barrier per step.
+// `parity` counts the calls on `sh`.
+__device__ __forceinline__ void piv_gj64(float2* M, int o, PivShared& sh, uint32_t parity) {
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31, c = lane & 7, h = (lane >> 3) & 1, top = lane >> 4;
+  float2* row = M + (size_t)(o + 32 * top + 2 * w + h) * kPivLd + o + 2 * c;
+  float2 a[4][2];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int j = 0; j < 4; ++j) {
+    const float4 v = *reinterpret_cast<const float4*>(row + 16 * j);
+    a[j][0] = make_float2(v.x, v.y);
+    a[j][1] = make_float2(v.z, v.w);
+  }
+  // first half of P^-1 from the warp's entries n0, n1 in step s's pivot columns
+  float2 p11, p12, p21, p22, i1, t12, t21;
+  bool ok1;
+  auto first_pivot = [&](int s, float2 n0, float2 n1) {
+    const int l = 16 * (s >> 4) + (s & 7);
+    p11 = shfl_c(n0, l);
+    p12 = shfl_c(n1, l);
+    p21 = shfl_c(n0, l + 8);
+    p22 = shfl_c(n1, l + 8);
+    ok1 = piv_inv(p11, i1);
+    t12 = piv_mul<1>(i1, p12);  // p11^-1 p12
+    t21 = piv_mul(p21, i1);     // p21 p11^-1
+  };
+  auto publish = [&](int s) {
+    if (top == s >> 4) {
+      const float2 one = make_float2(h ? 0.f : 1.f, 0.f), two = make_float2(h ? 1.f : 0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) a[i][j] = M[(o + rr + i) * kPivLd + o + cc + j];
-  for (int s = 0; s < kPivH / 2; ++s) {
-    const int buf = s & 1;
-    if (lane == s)  // the rows' entries in the pivot columns, before the step
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-        sh.colb[buf][rr + i] = make_float4(a[i][0].x, a[i][0].y, a[i][1].x, a[i][1].y);
-    if (w == s) {  // warp-uniform: the pivot rows
-      float2 q00 = make_float2(0.f, 0.f), q01 = q00, q10 = q00, q11 = q00;
-      if (lane == s) {
-        float2 i1, is;
-        const bool ok1 = cinv_guard<float>(a[0][0], i1, 1e-6f);
-        const float2 t12 = cmul(i1, a[0][1]);  // p11^-1 p12
-        const float2 t21 = cmul(a[1][0], i1);  // p21 p11^-1
-        const bool ok2 = cinv_guard<float>(csub(a[1][1], cmul(a[1][0], t12)), is, 1e-6f);
-        if (!ok1 || !ok2) sh.bad = 1;
-        const float2 u = cmul(t12, is);
-        q00 = cadd(i1, cmul(u, t21));
-        q01 = make_float2(-u.x, -u.y);
-        const float2 v = cmul(is, t21);
-        q10 = make_float2(-v.x, -v.y);
-        q11 = is;
-        sh.pivb[buf][0] = make_float4(q00.x, q00.y, q01.x, q01.y);
-        sh.pivb[buf][1] = make_float4(q10.x, q10.y, q11.x, q11.y);
-      }
-      q00 = shfl_c(q00, s);
-      q01 = shfl_c(q01, s);
-      q10 = shfl_c(q10, s);
-      q11 = shfl_c(q11, s);
-      float2 r0[2], r1[2];
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        r0[j] = cadd(cmul(q00, a[0][j]), cmul(q01, a[1][j]));
-        r1[j] = cadd(cmul(q10, a[0][j]), cmul(q11, a[1][j]));
-      }
-      if (lane == s) {
-        sh.rowb[buf][0][lane] = make_float4(1.f, 0.f, 0.f, 0.f);
-        sh.rowb[buf][1][lane] = make_float4(0.f, 0.f, 1.f, 0.f);
-        a[0][0] = q00; a[0][1] = q01;
-        a[1][0] = q10; a[1][1] = q11;
-      } else {
-        sh.rowb[buf][0][lane] = make_float4(a[0][0].x, a[0][0].y, a[0][1].x, a[0][1].y);
-        sh.rowb[buf][1][lane] = make_float4(a[1][0].x, a[1][0].y, a[1][1].x, a[1][1].y);
-        a[0][0] = r0[0]; a[0][1] = r0[1];
-        a[1][0] = r1[0]; a[1][1] = r1[1];
+      for (int j = 0; j < 4; ++j) {
+        const bool k = c == (s & 7) && j == s >> 3;
+        const float2 v0 = k ? one : a[j][0], v1 = k ? two : a[j][1];
+        sh.rowb[s][h][8 * j + c] = make_float4(v0.x, v0.y, v1.x, v1.y);
       }
     }
-    __syncthreads();
-    if (w != s) {
-      const float4 p0 = sh.pivb[buf][0], p1 = sh.pivb[buf][1];
-      const float4 b0 = sh.rowb[buf][0][lane], b1 = sh.rowb[buf][1][lane];
-      const float2 rk0[2] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w)};
-      const float2 rk1[2] = {make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
+    float2 is;
+    const bool ok2 = piv_inv(csub(p22, piv_mul(p21, t12)), is);
+    const float2 u = piv_mul(t12, is), v = piv_mul<1>(is, t21), ut = piv_mul(u, t21);
+    if (lane == 0) {
+      sh.pivb[s][0] = make_float4(__fadd_rn(i1.x, ut.x), __fadd_rn(i1.y, ut.y), -u.x, -u.y);
+      sh.pivb[s][1] = make_float4(-v.x, -v.y, is.x, is.y);
+      if (!ok1 || !ok2) sh.bad = 1;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sh.ready[s]);
+  };
+  if (w == 0) {
+    first_pivot(0, a[0][0], a[0][1]);
+    publish(0);
+  }
+  bool ok = true;
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const float4 c4 = sh.colb[buf][rr + i];
-        const float2 x0 = make_float2(c4.x, c4.y), x1 = make_float2(c4.z, c4.w);
-        // g = (x0, x1) P^-1
-        const float2 g0 = cadd(cmul(x0, make_float2(p0.x, p0.y)), cmul(x1, make_float2(p1.x, p1.y)));
-        const float2 g1 = cadd(cmul(x0, make_float2(p0.z, p0.w)), cmul(x1, make_float2(p1.z, p1.w)));
+  for (int jp = 0; jp < 4; ++jp) {  // pivot columns a[jp] of lanes c = sl
+#pragma unroll 1
+    for (int sl = 0; sl < 8 && ok; ++sl) {
+      const int s = 8 * jp + sl;
+      const bool own = c == sl;
+      // the row's entries in the pivot columns
+      const float2 x0 = shfl_c(a[jp][0], (lane & 24) | sl), x1 = shfl_c(a[jp][1], (lane & 24) | sl);
+      ok = __all_sync(0xffffffffu, mbar_wait(&sh.ready[s], parity, &sh.abort));
+      const float4 p0 = sh.pivb[s][0], p1 = sh.pivb[s][1];
+      const float2 q00 = make_float2(p0.x, p0.y), q01 = make_float2(p0.z, p0.w);
+      const float2 q10 = make_float2(p1.x, p1.y), q11 = make_float2(p1.z, p1.w);
+      if (w == (s & 15) && top == jp >> 1) {  // a pivot row
+        const float2 q0 = h ? q10 : q00, q1 = h ? q11 : q01;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          float2 v = lane == s ? make_float2(0.f, 0.f) : a[i][j];
-          v.x -= g0.x * rk0[j].x - g0.y * rk0[j].y + g1.x * rk1[j].x - g1.y * rk1[j].y;
-          v.y -= g0.x * rk0[j].y + g0.y * rk0[j].x + g1.x * rk1[j].y + g1.y * rk1[j].x;
-          a[i][j] = v;
+        for (int j = 0; j < 4; ++j) {
+          const float4 b0 = sh.rowb[s][0][8 * j + c], b1 = sh.rowb[s][1][8 * j + c];
+          const float2 r0 = piv_mul2<1>(q0, make_float2(b0.x, b0.y), q1, make_float2(b1.x, b1.y));
+          const float2 r1 = piv_mul2<1>(q0, make_float2(b0.z, b0.w), q1, make_float2(b1.z, b1.w));
+          a[j][0] = own && j == jp ? q0 : r0;
+          a[j][1] = own && j == jp ? q1 : r1;
         }
+        continue;
+      }
+      // g = (x0, x1) P^-1
+      const float2 g0 = piv_mul2(x0, q00, x1, q10), g1 = piv_mul2(x0, q01, x1, q11);
+      auto update = [&](int j) {
+        const float4 b0 = sh.rowb[s][0][8 * j + c], b1 = sh.rowb[s][1][8 * j + c];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const float2 r0 = q ? make_float2(b0.z, b0.w) : make_float2(b0.x, b0.y);
+          const float2 r1 = q ? make_float2(b1.z, b1.w) : make_float2(b1.x, b1.y);
+          const float2 v = own && j == jp ? make_float2(0.f, 0.f) : a[j][q];
+          const float dx = __fmaf_rn(-g1.y, r1.y, __fmaf_rn(g1.x, r1.x, __fmaf_rn(g0.x, r0.x, -__fmul_rn(g0.y, r0.y))));
+          const float dy = __fmaf_rn(g1.y, r1.x, __fmaf_rn(g1.x, r1.y, __fmaf_rn(g0.x, r0.y, __fmul_rn(g0.y, r0.x))));
+          a[j][q] = make_float2(__fsub_rn(v.x, dx), __fsub_rn(v.y, dy));
+        }
+      };
+      const int jn = jp < 3 ? jp + 1 : jp;  // the group of the next step's pivot columns at a group's end
+      update(jp);
+      if (jn != jp) update(jn);
+      if (w == ((s + 1) & 15) && s + 1 < kPivH / 2) {
+        first_pivot(s + 1, sl == 7 ? a[jn][0] : a[jp][0], sl == 7 ? a[jn][1] : a[jp][1]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j != jp && j != jn) update(j);
+        publish(s + 1);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j != jp && j != jn) update(j);
       }
     }
   }
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) M[(o + rr + i) * kPivLd + o + cc + j] = a[i][j];
-}
-
-// a b with the roundings written out (one multiply and one fused multiply-add per
-// part), whatever the compiler makes of the code around it
-__device__ __forceinline__ float2 piv_mul(float2 a, float2 b) {
-  return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+  for (int j = 0; j < 4; ++j)
+    *reinterpret_cast<float4*>(row + 16 * j) = make_float4(a[j][0].x, a[j][0].y, a[j][1].x, a[j][1].y);
 }
 
 // acc[a][c] = sum_{k0 <= k < k0 + kn} X[i0 + a][k] Y[k][j0 + c] (a < 4, c < 2)
@@ -1034,13 +1084,14 @@ __global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __res
     *reinterpret_cast<float4*>(M + r * kPivLd + 2 * v) =
         *reinterpret_cast<const float4*>(src + (size_t)(k0 + r) * np + k0 + 2 * v);
   }
-  if (t == 0) sh.bad = 0;
+  if (t == 0) sh.bad = sh.abort = 0;
+  if (t < kPivH / 2) mbar_init(&sh.ready[t], 1);
   __syncthreads();
   // two halves of 512 threads: a product alone is split along K (the upper
   // half's partial sums pass through T), two independent products run side by side
   const int half = t >> 9, s = t & 511;
   float2 u[4][2];
-  piv_gj64(M, 0, sh);  // B11 <- P1
+  if (t < 512) piv_gj64(M, 0, sh, 0);  // B11 <- P1
   __syncthreads();
   piv_mm(B11, kPivLd, B12, kPivLd, s, 32 * half, 32, u);  // P1 A12
   if (half) piv_put(T, kPivH, s, u);
@@ -1061,7 +1112,7 @@ __global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __res
     piv_put(B21, kPivLd, s, u);  // B21 <- -A21 P1
   }
   __syncthreads();
-  piv_gj64(M, kPivH, sh);  // B22 <- X22
+  if (t < 512) piv_gj64(M, kPivH, sh, 1);  // B22 <- X22
   __syncthreads();
   piv_mm(B12, kPivLd, B22, kPivLd, s, 32 * half, 32, u);  // B12 X22
   if (half) piv_put(T, kPivH, s, u);
@@ -1084,7 +1135,7 @@ __global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __res
     piv_put(B11, kPivLd, s, u);  // B11 <- P1 + V B21
   }
   __syncthreads();
-  if (sh.bad && t == 0 && status) atomicCAS(status, 0, DS_SINGULAR);
+  if (t == 0 && status && (sh.abort || sh.bad)) atomicCAS(status, 0, sh.abort ? DS_TIMEOUT : DS_SINGULAR);
   // four entries per thread and pass: eight lanes take the eight rows of a 128-byte core
   // matrix, their quads the core matrices beside it
   __nv_bfloat16* dst = pimg + b * pstride;
