@@ -64,7 +64,11 @@ typedef struct {
 
 /* Arithmetic of the per-point Dyson solve of nedmft_lattice_gloc. */
 typedef enum {
-  /* FP64 Gauss-Jordan inversion of each B_q - S (DFMA). */
+  /* FP64-accurate Gauss-Jordan inversion of each B_q - S: up to 20 rows in
+   * shared memory on the FP64 units; above, blocked (32 columns per step) with
+   * every product on the tensor cores (each operand row cut into seven 8-bit
+   * integer digits of a common exponent, digit products exact in FP32, the
+   * sums rounded to FP64 once). */
   NEDMFT_FP64 = 0,
   /* bf16x3 (hi*hi + hi*lo + lo*hi) tcgen05 tensor-core Gauss-Jordan with
    * FP32 accumulation in TMEM; then, for every point outside the
@@ -104,7 +108,8 @@ const char* nedmft_version(void);
  * NEDMFT_ESINGULAR. */
 int nedmft_check_status(void* stream);
 
-/* Failure detection of the tensor-core kernels.  Every wait of those kernels
+/* Failure detection of the tensor-core kernels (both precisions of the
+ * lattice step, the impurity step and the network).  Every wait of those kernels
  * for work (a filled or a free pipeline stage, an accumulator) is bounded: it
  * gives up after the device's wait limit, the kernel stops issuing work,
  * waits (for at most 2 s) for the copies and products it already issued,
@@ -307,7 +312,8 @@ int32_t nedmft_lattice_block_width(const nedmft_contour* c, int32_t nq,
  * buffers, or a plugin running under a framework whose caching allocator owns
  * the device and exposes no raw workspace to it.
  *   Arguments and results are those of nedmft_lattice_gloc with prec =
- *   NEDMFT_FP64 (points are inverted 32 at a time).
+ *   NEDMFT_FP64 (points are inverted 32 at a time, each in shared memory on
+ *   the FP64 units whatever n_c).
  *   Scratch: a fixed device array of about 6.6 MB inside the library, one
  *   per GPU that loads the library, held until the process exits.  The
  *   first call on a device looks up that array's device address
@@ -358,7 +364,7 @@ size_t nedmft_impurity_workspace_size(const nedmft_contour* c);
  * Gauss-Jordan (32 columns per step) whose pivot rows a tournament of
  * partial-pivoting rounds on 256-row chunks chooses, their trailing updates
  * on the tensor cores with FP64 accuracy (each operand row cut into seven
- * 7-bit integer digits, digit products exact in FP32); each step's tournament
+ * 8-bit integer digits, digit products exact in FP32); each step's tournament
  * and pivot block run one step ahead on a second, library-owned stream of
  * the highest priority (one per device and host thread, made by the thread's
  * first call and kept, with its two events, until the process ends), forked
@@ -389,8 +395,9 @@ int nedmft_impurity_update(const nedmft_contour* c, const nedmft_model* m,
  * Network: 17 features -> 4 tanh layers of 256 -> 2 outputs (Re, Im of X).
  * Parameters: one FP32 array of nedmft_mlp_param_count() values, layer by
  * layer, each layer a row-major (in x out) weight block followed by its
- * out biases.  The GEMMs run on the tensor cores: operands rounded to bf16,
- * sums in FP32; the weight gradients add their K slices in a fixed order, so
+ * out biases.  The products run on the tensor cores: operands rounded to bf16,
+ * sums in FP32, a tile of 128 samples through all layers in one block; the
+ * weight gradients add their slices of samples in a fixed order, so
  * nedmft_mlp_grad is deterministic.
  * Features of the pair (t_a, t_b), chosen to carry over from short training
  * contours to longer ones: U/2.5, E/4, tanh(Re(t_a - t_b)/3), then for t_a

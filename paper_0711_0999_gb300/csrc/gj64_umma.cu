@@ -312,8 +312,9 @@ __device__ __forceinline__ void cfmaf(float2& acc, float2 a, float2 b) {
 // residual E = I - A X from the digit products on the tensor cores, exact to
 // 2^-54 of the row and column maxima as in the update, and the small product X E
 // in FP32: E squares from round to round (1e-5, 1e-10 as a rule), and below
-// 2^-30 FP32 is enough for the last correction.  Why: the same block by FP64 elimination is 32768 complex
-// multiply-adds on two FP64 units, 33 us at best and 55 us measured.
+// 2^-30 FP32 is enough for the last correction.  Latency bound.  Why: the same block by
+// FP64 elimination is 32768 complex multiply-adds on two FP64 units, 33 us at best; the
+// kernel with it took 55 us for 64 blocks of matrices of 768 rows, with this 33.
 __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&in)[4], double2 (&out)[4],
                                                 uint32_t tmem, uint32_t& phase) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -676,7 +677,8 @@ struct RSmem {
 // 2r + 1 of seven orders; each thread turns 16 of its column's 64 sums into
 // FP64 and those into the digits of the update's B operand: row 2j =
 // [Re R_j | -Im R_j], row 2j + 1 = [Im R_j | Re R_j], one exponent per column.
-// One CTA per SM, its phases one after the other: latency bound, hence 16 warps.
+// One CTA per SM, its phases one after the other: latency bound, hence 16 warps
+// (47 us for 64 matrices of 768 rows, 32 us for 64 of 256).
 // With `sw` (one matrix, pivoted): row k0 + r of A_K is row sw->win[r]; the rows
 // that leave block K for the winners' places are copied there, each CTA its own
 // columns; and CTAs mtiles .. 2 mtiles - 1 cut C into digits with the rows so
@@ -853,17 +855,21 @@ static_assert(sizeof(UBars) <= USmem::kBars, "barrier block");
 // products (two buffers), two accumulator sets of 7 x 32 TMEM columns let the
 // products of one tile run beside the epilogue of the other.  Warp 0 loads,
 // warp 1 issues 28 MMAs per tile (7 digits x 4 k steps, N = 224 .. 32), warps
-// 2-9 drain: a thread has one row and 8 complex columns, a warp one box of 32
-// rows x 128 bytes, which is added to A at L2 by a TMA FP64 reduction (rows and
-// columns of block K: stored).  Column tiles at or past `jskip` move up by
-// `nskip` (a window that another kernel updates).
-// What bounds it: the L2's FP64 reductions, 2.6 TB/s of payload measured alone;
-// here 604 MB (64 matrices of 768 x 768) in 243 us, 2.5 TB/s.  Products 1792
-// cycles per tile of 4400, epilogue about 1700 issue cycles.  Measured before
-// it: old values loaded by TMA in 64-byte rows two boxes ahead, subtracted and
-// stored, 292 us (the shared memory left for boxes does not cover the latency);
-// half of the boxes each way, 274 us; every other tile of six warps loaded in
-// 128-byte rows one tile ahead, 359 us.
+// 2-9 drain: a thread has one row and 8 complex columns, a warp one 4 KB box of 32
+// rows x 128 bytes (contiguous in A), which is added to A at L2 by a bulk FP64
+// reduction (rows and columns of block K: stored).  Column tiles at or past `jskip`
+// move up by `nskip` (a window that another kernel updates).
+// What bounds it: the sequence of products, drain and additions of a tile, about 3600
+// cycles; 604 MB (64 matrices of 768 x 768) in 238 us, 2.5 TB/s of FP64 additions, of
+// 2.9 measured for contiguous boxes alone.  The products take 2305 cycles (an MMA of
+// 128 rows and K = 16 takes max(72, N / 2)), the epilogue about 1700 issue cycles.  Left
+// out one at a time: the additions 210 us, the epilogue's arithmetic 238, the loads of R
+// 220, the additions and the products' width 208.  Measured before it: old values loaded
+// by TMA in 64-byte rows two boxes ahead, subtracted and stored, 292 us (the shared
+// memory left for boxes does not cover the latency); half of the boxes each way, 274 us;
+// every other tile of six warps loaded in 128-byte rows one tile ahead, 359 us; the
+// additions as 2-D boxes of a row-major A, 243 us (2.6 TB/s alone).  FP64 units: 20.6 ms
+// for all 47 steps of a matrix of 1500 rows; here 0.86 ms, the panels included.
 __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
     gj64_update_kernel(double2* __restrict__ A, int np, int mtiles, int ntn, int total, int k0,
                        int jskip, int nskip, const __nv_bfloat16* __restrict__ cimg, const int* __restrict__ cexp,
