@@ -42,7 +42,8 @@ struct GemmParams {
   const __nv_bfloat16* b;
   size_t b_batch;
   size_t b_slice;
-  int kt;                // K tiles
+  int kt;                // K tiles of the operand images
+  int kn;                // K tiles of the product; what lies beyond is padding
   int* status;
 };
 
@@ -55,7 +56,8 @@ struct TileMapParams {
   CUtensorMap map;
   long long a, a_batch, a_slice;  // tiles
   long long b, b_batch, b_slice;
-  int kt;                          // K tiles (64 k) of the product
+  int kt;                          // K tiles (64 k) of the operand images
+  int kh;                          // half K tiles (32 k) of the product; what lies beyond is padding
   int* status;
 };
 
@@ -141,7 +143,7 @@ __device__ __forceinline__ void umma_gemm_body(const GemmParams& p, const Epi& e
       const __nv_bfloat16* a = p.a + bidx * p.a_batch;
       const __nv_bfloat16* b = p.b + bidx * p.b_batch;
       int issued = 0;
-      for (int kt = 0; kt < p.kt; ++kt) {
+      for (int kt = 0; kt < p.kn; ++kt) {
         const int s = kt % C::kStages;
         const uint32_t ph = (kt / C::kStages) & 1;
         if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) break;
@@ -169,7 +171,7 @@ __device__ __forceinline__ void umma_gemm_body(const GemmParams& p, const Epi& e
   } else if (warp == 1) {
     if (lane == 0) {
       constexpr uint32_t idesc = idesc_bf16(128, C::kBn);
-      for (int kt = 0; kt < p.kt; ++kt) {
+      for (int kt = 0; kt < p.kn; ++kt) {
         const int s = kt % C::kStages;
         const uint32_t ph = (kt / C::kStages) & 1;
         if (!mbar_wait(&full[s], ph, abort_flag)) break;
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(64 + 32 * EPIW, 1)
         const int mt = PAIR * (rem / n_tiles) + rank, nt = rem % n_tiles;
         const long long a0 = p.a + b * p.a_batch + (long long)mt * p.kt;
         const long long b0 = p.b + b * p.b_batch + (long long)nt * C::kBTiles * p.kt;
-        for (int h = 0; h < 2 * p.kt; ++h, ++it) {  // half tiles: kt = h / 2, core columns 4 (h % 2) .. +3
+        for (int h = 0; h < p.kh; ++h, ++it) {  // half tiles: kt = h / 2, core columns 4 (h % 2) .. +3
           const int s = it % C::kStages;
           const uint32_t ph = (it / C::kStages) & 1;
           if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
@@ -398,7 +400,7 @@ __global__ void __launch_bounds__(64 + 32 * EPIW, 1)
           tc_fence_after();
         }
         const uint32_t d = tmem + buf * kAccCols;
-        for (int h = 0; h < 2 * p.kt; ++h, ++it) {
+        for (int h = 0; h < p.kh; ++h, ++it) {
           const int s = it % C::kStages;
           if (!mbar_wait(&full[s], (it / C::kStages) & 1, abort_flag)) { ok = false; break; }
           tc_fence_after();
@@ -1065,7 +1067,7 @@ __device__ __forceinline__ void piv_store4(__nv_bfloat16* dst, size_t slice, siz
   *reinterpret_cast<uint4*>(dst + 3 * slice + o) = make_uint4(l2[0], l2[1], l2[2], l2[3]);
 }
 
-__global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __restrict__ A, int np, int k0,
+__global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __restrict__ A, int np, int k0, int live,
                                                              __nv_bfloat16* __restrict__ pimg, size_t pstride,
                                                              size_t pslice, int* status) {
   extern __shared__ __align__(16) float2 piv_smem[];
@@ -1093,48 +1095,50 @@ __global__ void __launch_bounds__(1024) gj_pivot_pack_kernel(const float2* __res
   float2 u[4][2];
   if (t < 512) piv_gj64(M, 0, sh, 0);  // B11 <- P1
   __syncthreads();
-  piv_mm(B11, kPivLd, B12, kPivLd, s, 32 * half, 32, u);  // P1 A12
-  if (half) piv_put(T, kPivH, s, u);
-  __syncthreads();
-  if (!half) {
-    piv_acc(T, kPivH, s, 1.f, u);
-    piv_put(B12, kPivLd, s, u);  // B12 <- P1 A12
+  if (live > kPivH) {  // else the second half is the identity: columns `live` and on are padding
+    piv_mm(B11, kPivLd, B12, kPivLd, s, 32 * half, 32, u);  // P1 A12
+    if (half) piv_put(T, kPivH, s, u);
+    __syncthreads();
+    if (!half) {
+      piv_acc(T, kPivH, s, 1.f, u);
+      piv_put(B12, kPivLd, s, u);  // B12 <- P1 A12
+    }
+    __syncthreads();
+    piv_mm(B21, kPivLd, half ? B11 : B12, kPivLd, s, 0, kPivH, u);  // A21 B12 | A21 P1
+    __syncthreads();
+    if (!half) {
+      piv_neg(u);
+      piv_acc(B22, kPivLd, s, 1.f, u);
+      piv_put(B22, kPivLd, s, u);  // B22 <- A22 - A21 B12
+    } else {
+      piv_neg(u);
+      piv_put(B21, kPivLd, s, u);  // B21 <- -A21 P1
+    }
+    __syncthreads();
+    if (t < 512) piv_gj64(M, kPivH, sh, 1);  // B22 <- X22
+    __syncthreads();
+    piv_mm(B12, kPivLd, B22, kPivLd, s, 32 * half, 32, u);  // B12 X22
+    if (half) piv_put(T, kPivH, s, u);
+    __syncthreads();
+    if (!half) {
+      piv_acc(T, kPivH, s, 1.f, u);
+      piv_neg(u);
+      piv_put(T, kPivH, s, u);  // V = -B12 X22
+    }
+    __syncthreads();
+    piv_mm(half ? T : B22, half ? kPivH : kPivLd, B21, kPivLd, s, 0, kPivH, u);  // X22 B21 | V B21
+    __syncthreads();
+    if (!half) {
+      piv_put(B21, kPivLd, s, u);  // B21 <- X22 B21
+      float2 v[4][2] = {};
+      piv_acc(T, kPivH, s, 1.f, v);
+      piv_put(B12, kPivLd, s, v);  // B12 <- V
+    } else {
+      piv_acc(B11, kPivLd, s, 1.f, u);
+      piv_put(B11, kPivLd, s, u);  // B11 <- P1 + V B21
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  piv_mm(B21, kPivLd, half ? B11 : B12, kPivLd, s, 0, kPivH, u);  // A21 B12 | A21 P1
-  __syncthreads();
-  if (!half) {
-    piv_neg(u);
-    piv_acc(B22, kPivLd, s, 1.f, u);
-    piv_put(B22, kPivLd, s, u);  // B22 <- A22 - A21 B12
-  } else {
-    piv_neg(u);
-    piv_put(B21, kPivLd, s, u);  // B21 <- -A21 P1
-  }
-  __syncthreads();
-  if (t < 512) piv_gj64(M, kPivH, sh, 1);  // B22 <- X22
-  __syncthreads();
-  piv_mm(B12, kPivLd, B22, kPivLd, s, 32 * half, 32, u);  // B12 X22
-  if (half) piv_put(T, kPivH, s, u);
-  __syncthreads();
-  if (!half) {
-    piv_acc(T, kPivH, s, 1.f, u);
-    piv_neg(u);
-    piv_put(T, kPivH, s, u);  // V = -B12 X22
-  }
-  __syncthreads();
-  piv_mm(half ? T : B22, half ? kPivH : kPivLd, B21, kPivLd, s, 0, kPivH, u);  // X22 B21 | V B21
-  __syncthreads();
-  if (!half) {
-    piv_put(B21, kPivLd, s, u);  // B21 <- X22 B21
-    float2 v[4][2] = {};
-    piv_acc(T, kPivH, s, 1.f, v);
-    piv_put(B12, kPivLd, s, v);  // B12 <- V
-  } else {
-    piv_acc(B11, kPivLd, s, 1.f, u);
-    piv_put(B11, kPivLd, s, u);  // B11 <- P1 + V B21
-  }
-  __syncthreads();
   if (t == 0 && status && (sh.abort || sh.bad)) atomicCAS(status, 0, sh.abort ? DS_TIMEOUT : DS_SINGULAR);
   // four entries per thread and pass: eight lanes take the eight rows of a 128-byte core
   // matrix, their quads the core matrices beside it
@@ -1386,14 +1390,23 @@ int gj_blocked_umma_w(float2* A, int n, int np, int nb, char* scratch, int* stat
   gj_panel_pack_kernel<W>
       <<<dim3(np / 128, nb), 256, 0, st>>>(A, np, 0, cimg, pstride, cslice, timg, pstride, tslice);
   NED_LAUNCH_CHECK("gj_panel_pack_kernel");
-  for (int k0 = 0, step = 0; k0 < np; k0 += W, ++step) {
+  // Rows and columns n .. np - 1 are the identity from first to last.  The products leave out
+  // their share of K in the last step, and column tiles that lie wholly there (a panel
+  // or output column that is not visited keeps what it held and is never read).
+  // N_c = 400 (16 of the last
+  // step's 128 columns), 1024 points 14.9 -> 13.1 ms with the same in the refinement, N_c = 3400
+  // (72 of 256), 256 points 507 -> 469 ms, N_c = 1500 (220 of 256) 356.7 -> 352.3 ms.
+  const int n_tiles = (n + 127) / 128;
+  for (int k0 = 0, step = 0; k0 < n; k0 += W, ++step) {
+    const int live = n - k0 < W ? n - k0 : W;
+    const int kh = (2 * live + 31) / 32;
     __nv_bfloat16* cur_c = cimg + (step & 1) * chalf;
     __nv_bfloat16* cur_t = timg + (step & 1) * thalf;
     __nv_bfloat16* nxt_c = cimg + ((step + 1) & 1) * chalf;
     __nv_bfloat16* nxt_t = timg + ((step + 1) & 1) * thalf;
     if constexpr (W == 128) {
       if (int rc = ensure_dyn_smem(reinterpret_cast<const void*>(gj_pivot_pack_kernel), (int)kPivSmem)) return rc;
-      gj_pivot_pack_kernel<<<nb, 1024, kPivSmem, st>>>(A, np, k0, pimg, pstride, pslice, status);
+      gj_pivot_pack_kernel<<<nb, 1024, kPivSmem, st>>>(A, np, k0, live, pimg, pstride, pslice, status);
       NED_LAUNCH_CHECK("gj_pivot_pack_kernel");
     } else {
       // P = inv(A_KK): the W = 128 Gauss-Jordan on copies of the diagonal blocks
@@ -1402,32 +1415,30 @@ int gj_blocked_umma_w(float2* A, int n, int np, int nb, char* scratch, int* stat
       char* inner_scratch = inner + gj_buffers<128>(W).mat * nb;
       gj_extract_kernel<W><<<dim3(W / kPackRows, nb), 256, 0, st>>>(A, np, k0, Xs);
       NED_LAUNCH_CHECK("gj_extract_kernel");
-      int rc = gj_blocked_umma_w<128>(Xs, W, W, nb, inner_scratch, status, st, false);
+      int rc = gj_blocked_umma_w<128>(Xs, live, W, nb, inner_scratch, status, st, false);
       if (rc) return rc;
       gj_ppack_kernel<W><<<dim3(W / kPackRows, nb), 256, 0, st>>>(Xs, pimg, pstride, pslice);
       NED_LAUNCH_CHECK("gj_ppack_kernel");
     }
     {  // Re R = P' A_K, Im R = P'' A_K: W x np each, K = 2W
       TileMapParams p{tile_map, tile_of(pimg), per_t, (long long)(pslice / kTileElems),
-                      tile_of(cur_t), per_t, (long long)(tslice / kTileElems), kKtW, status};
+                      tile_of(cur_t), per_t, (long long)(tslice / kTileElems), kKtW, kh, status};
       EpiRPack<W> epi{rimg, pstride, rslice};
-      int rc = launch_gemm_persistent<CfgRP, Split3x2, 4>(p, np / EpiRPack<W>::kBn, W / kTileRows, nb, epi, st);
+      int rc = launch_gemm_persistent<CfgRP, Split3x2, 4>(p, n_tiles, W / kTileRows, nb, epi, st);
       if (rc) return rc;
     }
     {  // A <- A - C' R, np x 2np, K = 2W; next step's panels from the epilogue
       TileMapParams p{tile_map, tile_of(cur_c), per_t, (long long)(cslice / kTileElems),
-                      tile_of(rimg), per_t, (long long)(rslice / kTileElems), kKtW, status};
-      const int kn = (k0 + W < np) ? k0 + W : -1;
+                      tile_of(rimg), per_t, (long long)(rslice / kTileElems), kKtW, kh, status};
+      const int kn = (k0 + W < n) ? k0 + W : -1;
       EpiUpdate<W> epi{reinterpret_cast<float*>(A), (size_t)2 * np * np, np, k0, kn, nxt_c, nxt_t, pstride, cslice,
                        tslice};
       epi.red_map = red_map;
       const int slot = instrument ? instr_begin(st) : -1;
-      int rc = launch_gemm_persistent<CfgGJH, Split3, 4>(p, 2 * np / CfgGJ::kBn, np / kTileRows, nb, epi, st);
+      int rc = launch_gemm_persistent<CfgGJH, Split3, 4>(p, n_tiles, np / kTileRows, nb, epi, st);
       if (rc) return rc;
       if (instrument) {
-        const int live = n - k0 < W ? (n - k0 > 0 ? n - k0 : 0) : W;
-        instr_end(slot, st, 8.0 * (double)n * n * live * nb,
-                  live > 0 ? 2.0 * sizeof(float2) * (double)n * n * nb : 0.0);
+        instr_end(slot, st, 8.0 * (double)n * n * live * nb, 2.0 * sizeof(float2) * (double)n * n * nb);
       }
     }
   }
@@ -1735,7 +1746,7 @@ __global__ void __launch_bounds__(256) oz_pack_x_kernel(const float2* __restrict
                                                         int* __restrict__ xexp, __nv_bfloat16* __restrict__ aimg) {
   const int b = blockIdx.y;
   if (!flags[q0 + b]) return;
-  const int j0 = blockIdx.x * 32;
+  const int j0 = blockIdx.x * 32, nr = 32 * gridDim.x;
   const float2* x = X + (size_t)b * np * np;
   const int kt = 2 * np / kTileK;
   const size_t xs = (size_t)2 * np * 2 * np, as = (size_t)np * 2 * np;
@@ -1746,7 +1757,7 @@ __global__ void __launch_bounds__(256) oz_pack_x_kernel(const float2* __restrict
   __shared__ float2 tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   float m = 0.f;
-  for (int k = ty; k < np; k += 8) {
+  for (int k = ty; k < nr; k += 8) {
     const float2 z = x[(size_t)k * np + j0 + tx];
     m = fmaxf(m, fmaxf(fabsf(z.x), fabsf(z.y)));
   }
@@ -1761,7 +1772,7 @@ __global__ void __launch_bounds__(256) oz_pack_x_kernel(const float2* __restrict
     xexp[(size_t)b * np + j0 + threadIdx.x] = e;
   }
   __syncthreads();
-  for (int k0 = 0; k0 < np; k0 += 32) {
+  for (int k0 = 0; k0 < nr; k0 += 32) {
     // coalesced load of rows k0 .. k0+31, columns j0 .. j0+31
     for (int rr = ty; rr < 32; rr += 8) tile[rr][tx] = x[(size_t)(k0 + rr) * np + j0 + tx];
     __syncthreads();
@@ -1839,7 +1850,7 @@ struct OzParams {
   ContourDev c;
   ModelDev m;
   const double* eps;
-  int q0, nb, np, kt;
+  int q0, nb, np, kt, ktn;  // K tiles of the images, K tiles (of 32 columns) up to n
   int* status;
 };
 
@@ -1876,9 +1887,10 @@ __global__ void __launch_bounds__(64 + 32 * kOzEpiW, 1) oz_residual_kernel(const
   __shared__ int refined[kRedMaxBatch];
   __shared__ int n_refined;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_tiles = p.np / kTileRows, n_tiles = 2 * p.np / kOzBn;
+  const int m_tiles = (p.c.n + kTileRows - 1) / kTileRows, n_tiles = p.ktn;
+  static_assert(kOzBn == kTileK, "an output tile of 32 columns per K tile");
   const int per = m_tiles * n_tiles;
-  const int kh = 2 * p.kt;                  // half tiles per unit
+  const int kh = 2 * p.ktn;                 // half tiles per unit
   const int hc = 2 * kOzChunkKt;            // half tiles per chunk
   const int nchunks = (kh + hc - 1) / hc;   // chunks per unit
 
@@ -2368,7 +2380,11 @@ int umma_lattice_batch(const ContourDev& c, const ModelDev& m, const double* eps
   if ((rc = gj_blocked_umma(X, c.n, np, nb, scratch, status, st, width))) return rc;
   oz_coef_kernel<<<dim3((np + 255) / 256, nb), 256, 0, st>>>(c, m, eps, ebar, q0, S, np, coef, sh.flags);
   NED_LAUNCH_CHECK("oz_coef_kernel");
-  oz_pack_x_kernel<<<dim3(np / 32, nb), 256, 0, st>>>(X, np, q0, sh.flags, ximg, xexp, aimg);
+  // Rows and columns from n on are the identity in A' and X' and zero in S_d, so their
+  // products are zero: K ends at n (rounded up to 32), and output columns (a tile of 32
+  // of the residual, 128 of the correction) and rows past n are left out, never read.
+  const int ktn = (c.n + 31) / 32, tiles = (c.n + 127) / 128;
+  oz_pack_x_kernel<<<dim3(ktn, nb), 256, 0, st>>>(X, np, q0, sh.flags, ximg, xexp, aimg);
   NED_LAUNCH_CHECK("oz_pack_x_kernel");
   {
     OzParams p{};
@@ -2382,7 +2398,7 @@ int umma_lattice_batch(const ContourDev& c, const ModelDev& m, const double* eps
     p.b_exp = xexp;
     p.X = X; p.coef = coef; p.flags = sh.flags;
     p.rimg = rimg; p.r_batch = 2 * rs; p.r_slice = rs;
-    p.c = c; p.m = m; p.eps = eps; p.q0 = q0; p.nb = nb; p.np = np; p.kt = 2 * np / kTileK; p.status = status;
+    p.c = c; p.m = m; p.eps = eps; p.q0 = q0; p.nb = nb; p.np = np; p.kt = 2 * np / kTileK; p.ktn = ktn; p.status = status;
     if (nb > kRedMaxBatch) return set_error(NEDMFT_EINVAL, "residual: batch %d > %d", nb, kRedMaxBatch);
     // one CTA per SM, persistent over the refined matrices' units
     int sms = 0;
@@ -2397,23 +2413,23 @@ int umma_lattice_batch(const ContourDev& c, const ModelDev& m, const double* eps
   // product from the bf16 image of X' R' that the first one's epilogue writes
   // (into the X' slice buffer, which the residual no longer needs).
   {
-    GemmParams p{aimg, 2 * as, as, rimg, 2 * rs, rs, 2 * np / kTileK, status};
+    GemmParams p{aimg, 2 * as, as, rimg, 2 * rs, rs, 2 * np / kTileK, ktn, status};
     EpiStore epi{reinterpret_cast<float*>(dx), 2 * mat, np, ximg, kOzS * xs};
     if ((rc = ensure_dyn_smem(reinterpret_cast<const void*>(umma_gemm_flag_kernel<CfgGJ, Split3, EpiStore>),
                               CfgGJ::kSmem)))
       return rc;
     umma_gemm_flag_kernel<CfgGJ, Split3, EpiStore>
-        <<<dim3(2 * np / CfgGJ::kBn, np / kTileRows, nb), 192, CfgGJ::kSmem, st>>>(p, epi, sh.flags, q0);
+        <<<dim3(tiles, tiles, nb), 192, CfgGJ::kSmem, st>>>(p, epi, sh.flags, q0);
     NED_LAUNCH_CHECK("umma_gemm_flag_kernel");
   }
   {
-    GemmParams p{ximg, kOzS * xs, 0, rimg, 2 * rs, rs, 2 * np / kTileK, status};
+    GemmParams p{ximg, kOzS * xs, 0, rimg, 2 * rs, rs, 2 * np / kTileK, ktn, status};
     EpiAdd epi{reinterpret_cast<float*>(dx), 2 * mat, np};
     if ((rc = ensure_dyn_smem(reinterpret_cast<const void*>(umma_gemm_flag_kernel<CfgHi, Split1, EpiAdd>),
                               CfgHi::kSmem)))
       return rc;
     umma_gemm_flag_kernel<CfgHi, Split1, EpiAdd>
-        <<<dim3(2 * np / CfgHi::kBn, np / kTileRows, nb), 192, CfgHi::kSmem, st>>>(p, epi, sh.flags, q0);
+        <<<dim3(tiles, tiles, nb), 192, CfgHi::kSmem, st>>>(p, epi, sh.flags, q0);
     NED_LAUNCH_CHECK("umma_gemm_flag_kernel");
   }
   {

@@ -167,6 +167,20 @@ def test_dos_relative_times(n_t, m_index):
         assert np.abs(rho[row] - O.dos(c, gl, m, omega)).max() <= tol
 
 
+# the last step of the tensor-core Gauss-Jordan with 1, 16, 64, 65 and 128 columns before the padding, both block
+# widths, whole column tiles of padding (513, 641, 897), the 32-column tiles of the residual
+@pytest.mark.parametrize("n", [17, 32, 33, 64, 65, 128, 129, 144, 193, 400, 449, 512, 513, 577, 641, 769, 897, 1025])
+def test_mixed_lattice_padding_edges(n):
+    c, g, mo, mc, sig, (eps, ebar, wq) = setup(n, 3)
+    ref, jref = O.lattice_gloc(c, mo, sig, eps, ebar, wq)
+    for width in (0,) if n <= 512 else (128, 256):
+        api.lattice_set_tuning(g, 3, "mixed_bf16", width=width)
+        gl, j = lattice(g, mc, sig, eps, ebar, wq, "mixed_bf16")
+        assert rel(gl, ref) < 1e-6
+        assert np.abs(j - jref.real).max() < 1e-5
+    api.lattice_set_tuning(g, 3, "mixed_bf16")
+
+
 # weights: zeros and exact ties at the threshold, one heavy point, more points than the sorted choice takes
 @pytest.mark.parametrize("nq,kind", [(1, "one"), (300, "ties"), (300, "zeros"), (300, "heavy"), (8192, "random"),
                                      (8193, "random")])
