@@ -859,19 +859,21 @@ static_assert(sizeof(UBars) <= USmem::kBars, "barrier block");
 // rows x 128 bytes (contiguous in A), which is added to A at L2 by a bulk FP64
 // reduction (rows and columns of block K: stored).  Column tiles at or past `jskip`
 // move up by `nskip` (a window that another kernel updates).
-// What bounds it: the sequence of products, drain and additions of a tile, about 3600
-// cycles; 604 MB (64 matrices of 768 x 768) in 238 us, 2.5 TB/s of FP64 additions, of
-// 2.9 measured for contiguous boxes alone.  The products take 2305 cycles (an MMA of
-// 128 rows and K = 16 takes max(72, N / 2)), the epilogue about 1700 issue cycles.  Left
-// out one at a time: the additions 210 us, the epilogue's arithmetic 238, the loads of R
-// 220, the additions and the products' width 208.  Measured before it: old values loaded
+// What bounds it: HBM.  A passes through L2 once per step, read and written by the
+// additions: 64 matrices of 768 x 768 in 239 us with 1.47 GB of DRAM traffic (counters),
+// 6.1 TB/s, 0.9 of the copy rate.  Close behind: a tile's products take 2305 cycles
+// of 3600 (an MMA of 128 rows and K = 16 takes max(72, N / 2)), the epilogue about 1700
+// issue cycles.  Left out one at a time: the additions 210 us, the epilogue's arithmetic 238,
+// the loads of R 220, the additions and the products' width 208.  Boxes of rows past n
+// are not touched: N_c = 700 7.84 -> 7.66 ms, 1500 42.1 -> 41.5 (around the epilogue's
+// arithmetic too, the same test made it 10 % slower).  Measured before: old values loaded
 // by TMA in 64-byte rows two boxes ahead, subtracted and stored, 292 us (the shared
 // memory left for boxes does not cover the latency); half of the boxes each way, 274 us;
 // every other tile of six warps loaded in 128-byte rows one tile ahead, 359 us; the
-// additions as 2-D boxes of a row-major A, 243 us (2.6 TB/s alone).  FP64 units: 20.6 ms
-// for all 47 steps of a matrix of 1500 rows; here 0.86 ms, the panels included.
+// additions as 2-D boxes of a row-major A, 243 us.  FP64 units: 20.6 ms for all 47 steps of a
+// matrix of 1500 rows; here 0.85 ms, the panels included.
 __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
-    gj64_update_kernel(double2* __restrict__ A, int np, int mtiles, int ntn, int total, int k0,
+    gj64_update_kernel(double2* __restrict__ A, int n, int np, int mtiles, int ntn, int total, int k0,
                        int jskip, int nskip, const __nv_bfloat16* __restrict__ cimg, const int* __restrict__ cexp,
                        const __nv_bfloat16* __restrict__ rimg, const int* __restrict__ rexp, int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -1018,7 +1020,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
       }
       fence_proxy_async();
       __syncwarp();
-      if (lane == 0) {
+      if (lane == 0 && i < n) {  // a box of rows past n stays as it is (zero times anything)
         double2* dst = A + (size_t)b * np * np + box_off(np, i, j & ~7);  // lane 0: row 0 of the box
         if (ik || (j >= k0 && j < k0 + kNB)) bulk_store(dst, box, kBoxBytes);  // block K: nothing to add to
         else bulk_add_f64(dst, box, kBoxBytes);
@@ -1096,7 +1098,7 @@ int gj64_invert(double2* A, int n, int np, int nb, void* scratch, int* status, c
     NED_LAUNCH_CHECK("gj64_rpanel_kernel");
     const int slot = instr_begin(st);
     gj64_update_kernel<<<total < sms ? total : sms, 64 + 32 * kEpiW, USmem::kBytes, st>>>(
-        A, np, mtiles, ntn, total, k0, ntn, 0, cimg, cexp, rimg, rexp, status);
+        A, n, np, mtiles, ntn, total, k0, ntn, 0, cimg, cexp, rimg, rexp, status);
     NED_LAUNCH_CHECK("gj64_update_kernel");
     const int live = n - k0 < kNB ? n - k0 : kNB;
     instr_end(slot, st, 8.0 * (double)n * n * live * nb, 2.0 * sizeof(double2) * (double)n * n * nb);
@@ -1466,7 +1468,7 @@ int pivot_inverse(double2* a, int n, void* ws, cudaStream_t st, int* status) {
     const int total = mtiles * tiles;
     if (total <= 0) return NEDMFT_OK;
     gj64_update_kernel<<<total < ctas ? total : ctas, 64 + 32 * kEpiW, USmem::kBytes, s>>>(
-        ap, np, mtiles, tiles, total, k0, jskip, nskip, cimg, cexp, rimg, rexp, status);
+        ap, n, np, mtiles, tiles, total, k0, jskip, nskip, cimg, cexp, rimg, rexp, status);
     NED_LAUNCH_CHECK("gj64_update_kernel");
     return NEDMFT_OK;
   };

@@ -1393,9 +1393,9 @@ int gj_blocked_umma_w(float2* A, int n, int np, int nb, char* scratch, int* stat
   // Rows and columns n .. np - 1 are the identity from first to last.  The products leave out
   // their share of K in the last step, and column tiles that lie wholly there (a panel
   // or output column that is not visited keeps what it held and is never read).
-  // N_c = 400 (16 of the last
-  // step's 128 columns), 1024 points 14.9 -> 13.1 ms with the same in the refinement, N_c = 3400
-  // (72 of 256), 256 points 507 -> 469 ms, N_c = 1500 (220 of 256) 356.7 -> 352.3 ms.
+  // N_c = 400 (16 of the last step's 128 columns), 1024 points 14.9 -> 13.1 ms with the same
+  // in the refinement; N_c = 3400 (72 of 256), 256 points 507 -> 469 ms; N_c = 1500 (220 of
+  // 256) 356.7 -> 352.3 ms.
   const int n_tiles = (n + 127) / 128;
   for (int k0 = 0, step = 0; k0 < n; k0 += W, ++step) {
     const int live = n - k0 < W ? n - k0 : W;
