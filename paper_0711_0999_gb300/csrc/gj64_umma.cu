@@ -979,12 +979,22 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
       }
     };
     Pos cur{lo % ntn, lo / ntn / mtiles, lo / ntn % mtiles};
+    // exponents of a tile's row and eight columns, fetched a tile ahead (N_c = 700, 64 points
+    // 7.68 -> 7.51 ms, 1500 unchanged)
+    int4 ej[2];
+    int ei = 0;
+    auto exponents = [&](const Pos& p) {
+      const int* r = rexp + (size_t)p.b * np + col_tile(p.jn) * kTn + c0;
+      ej[0] = *reinterpret_cast<const int4*>(r);
+      ej[1] = *reinterpret_cast<const int4*>(r + 4);
+      ei = cexp[(size_t)p.b * np + p.mt * 128 + quarter * 32 + lane] + 1023 - 53;
+    };
+    if (lo < hi) exponents(cur);
     bool ok = true;
     for (int tile = lo, it = 0; tile < hi && ok; ++tile, ++it) {
       const int jt = col_tile(cur.jn), s = it & 1;
       const int b = cur.b, i = cur.mt * 128 + quarter * 32 + lane;
       const bool ik = i >= k0 && i < k0 + kNB;  // the same for the whole warp
-      const int ei = cexp[(size_t)b * np + i] + 1023 - 53;
       ok = __all_sync(0xffffffffu, mbar_wait(&bars.d_full[s], (it >> 1) & 1, abort_flag));
       if (!ok) break;
       tc_fence_after();
@@ -999,18 +1009,22 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
                    acc[hb][o]);
       tmem_wait_ld();
       tc_fence_before();
-      if (lane == 0) bulk_wait_read_n<0>();  // the last tile's box has been read
+      if (lane == 0) {
+        mbar_arrive(&bars.d_empty[s]);
+        bulk_wait_read_n<0>();  // the last tile's box has been read
+      }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars.d_empty[s]);
       const int j = jt * kTn + c0;
+      const int eb8[8] = {ei + ej[0].x, ei + ej[0].y, ei + ej[0].z, ei + ej[0].w,
+                          ei + ej[1].x, ei + ej[1].y, ei + ej[1].z, ei + ej[1].w};
+      step(cur);
+      if (tile + 1 < hi) exponents(cur);
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {
-        const int4 ej = *reinterpret_cast<const int4*>(rexp + (size_t)b * np + j + 4 * hb);
-        const int eq[4] = {ej.x, ej.y, ej.z, ej.w};
         const float(&c)[kS][8] = acc[hb];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const int eb = ei + eq[q];
+          const int eb = eb8[4 * hb + q];
           const double dx = orders_to_double(c[0][2 * q], c[1][2 * q], c[2][2 * q], c[3][2 * q], c[4][2 * q],
                                              c[5][2 * q], c[6][2 * q], eb);
           const double dy = orders_to_double(c[0][2 * q + 1], c[1][2 * q + 1], c[2][2 * q + 1], c[3][2 * q + 1],
@@ -1027,7 +1041,6 @@ __global__ void __launch_bounds__(64 + 32 * kEpiW, 1)
         bulk_commit();
       }
       __syncwarp();
-      step(cur);
     }
     if (lane == 0) bulk_wait_all();
   }
