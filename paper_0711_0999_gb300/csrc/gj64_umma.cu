@@ -860,10 +860,10 @@ static_assert(sizeof(UBars) <= USmem::kBars, "barrier block");
 // reduction (rows and columns of block K: stored).  Column tiles at or past `jskip`
 // move up by `nskip` (a window that another kernel updates).
 // What bounds it: HBM.  A passes through L2 once per step, read and written by the
-// additions: 64 matrices of 768 x 768 in 239 us with 1.47 GB of DRAM traffic (counters),
-// 6.1 TB/s, 0.9 of the copy rate.  Close behind: a tile's products take 2305 cycles
+// additions: 64 matrices of 700 rows (np = 768) in 222 us with 1.38 GB of DRAM traffic
+// (counters), 6.2 TB/s, 0.91 of the copy rate.  Close behind: a tile's products take 2305 cycles
 // of 3600 (an MMA of 128 rows and K = 16 takes max(72, N / 2)), the epilogue about 1700
-// issue cycles.  Left out one at a time: the additions 210 us, the epilogue's arithmetic 238,
+// issue cycles.  Left out one at a time (of 238 us then): the additions 210 us, the epilogue's arithmetic 238,
 // the loads of R 220, the additions and the products' width 208.  Boxes of rows past n
 // are not touched: N_c = 700 7.84 -> 7.66 ms, 1500 42.1 -> 41.5 (around the epilogue's
 // arithmetic too, the same test made it 10 % slower).  Measured before: old values loaded
