@@ -61,8 +61,7 @@ def lattice(g, mc, sig, eps, ebar, wq, prec="fp64"):
     return gl.cpu().numpy(), j.cpu().numpy()
 
 
-# one 32-column step and its neighbours, the 64- and 128-row tiles, the padded sizes 256 and 512, each
-# with an odd and an even number of points (a batch holds an even number)
+# one 32-column step and its neighbours, the 64- and 128-row tiles, the padded sizes 256 and 512
 @pytest.mark.parametrize("n,nq", [(19, 3), (20, 3), (21, 1), (21, 2), (32, 5), (33, 4), (64, 3), (65, 3), (96, 7), (127, 2),
                                   (128, 3), (129, 3), (160, 2), (255, 3), (256, 2), (257, 3), (513, 2)])
 def test_fp64_lattice_tile_edges(n, nq):
@@ -179,6 +178,22 @@ def test_mixed_lattice_padding_edges(n):
         assert rel(gl, ref) < 1e-6
         assert np.abs(j - jref.real).max() < 1e-5
     api.lattice_set_tuning(g, 3, "mixed_bf16")
+
+
+# what the products leave out (panels and columns of padding) keeps the workspace's old bits: NaN there changes nothing
+@pytest.mark.parametrize("n,prec", [(65, "mixed_bf16"), (400, "mixed_bf16"), (513, "mixed_bf16"), (897, "mixed_bf16"),
+                                    (33, "fp64"), (129, "fp64"), (400, "fp64")])
+def test_lattice_does_not_read_stale_workspace(n, prec):
+    c, g, mo, mc, sig, (eps, ebar, wq) = setup(n, 3)
+    s = torch.as_tensor(sig, device="cuda")
+    out = []
+    for fill in (0, 255):
+        ws = torch.full((api.lattice_workspace_size(g, 3, prec),), fill, dtype=torch.uint8, device="cuda")
+        gl, j, _ = api.lattice_gloc(g, mc, s, eps, ebar, wq, precision=prec, ws=ws)
+        torch.cuda.synchronize()
+        api.check_status()
+        out.append((gl.cpu().numpy(), j.cpu().numpy()))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
 # weights: zeros and exact ties at the threshold, one heavy point, more points than the sorted choice takes
