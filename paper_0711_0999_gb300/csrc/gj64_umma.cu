@@ -35,6 +35,7 @@ using namespace umma;
 namespace {
 
 constexpr int kS = 7;    // digits of an operand, orders kept
+constexpr int kO = 8;    // orders of the pivot blocks' residuals
 constexpr int kNB = 32;  // complex columns per step
 constexpr int kK = 64;   // reals per row of C and column of R: [re | im]
 constexpr int kTn = 16;  // complex columns of an update tile
@@ -192,16 +193,23 @@ __device__ __forceinline__ double orders_to_double(float c0, float c1, float c2,
   return __hiloint2double((int)rh, (int)ql);
 }
 
-// the same sum plus `more` (in its units), as a float of about 24 bits, times `scale`
+// The same sum plus `more` (in its units) and with order 7, as a float of about 24 bits, times
+// `scale`.  Orders 6 and 7 and what a unit cannot hold are added to the sum of the others as
+// a float: a sum that cancels down to a few units keeps ten more bits.
 __device__ __forceinline__ float orders_to_float(float c0, float c1, float c2, float c3, float c4, float c5, float c6,
-                                                 unsigned long long more, float scale) {
+                                                 float c7, unsigned long long more, float scale) {
+  constexpr float kM = 12582912.f;
   uint32_t u0, u1, u2;
-  order_words(c0, c1, c2, c3, c4, c5, c6, u0, u1, u2);
+  order_words(c0, c1, c2, c3, c4, c5, 0.f, u0, u1, u2);
+  const float h4 = fmaf(c4, 0.5f, kM) - kM;
+  const float g = fmaf(fmaf(c4, 0.5f, -h4), 512.f, c5);                        // as order_words has it
+  const float frac = fmaf(g, 0.5f, -(fmaf(g, 0.5f, kM) - kM));                 // 0 or +-1/2
+  const float low = frac + fmaf(c7, 7.62939453125e-6f, c6 * 0.001953125f);     // 2^-17, 2^-9
   const long long T = (long long)((unsigned long long)u0 * 0x80000000ull +
                                   ((unsigned long long)u1 * 32768ull + ((unsigned long long)u2 + (kLess + more))));
   const unsigned long long a = (unsigned long long)(T < 0 ? -T : T);
   const float f = __fmaf_rz(__uint2float_rz((uint32_t)(a >> 32)), 4294967296.f, __uint2float_rz((uint32_t)a));
-  return (T < 0 ? -f : f) * scale;
+  return ((T < 0 ? -f : f) + low) * scale;
 }
 
 // ------------------------------------------------------------------ pivot block and C digits
@@ -269,6 +277,7 @@ __device__ __forceinline__ void pack_c_rows(const double2* __restrict__ A, int n
 struct BlockSmem {
   __nv_bfloat16 a[kS * 64 * kK];   // digits of the block: row 2r = [Re | -Im], 2r + 1 = [Im | Re]
   __nv_bfloat16 x[kS * kNB * kK];  // digits of X: row j = [Re X_j | Im X_j], column j over k
+  __nv_bfloat16 zero[kNB * kK];    // a zero digit, which opens the sums of order 7
   float2 xt[kNB][kNB], e[kNB][kNB + 2];  // X by columns, the residual by rows
   float2 mult[2][kNB];
   uint64_t bar;
@@ -279,6 +288,8 @@ struct BlockSmem {
 };
 // The products read 128 rows of a digit; rows past 64 are the next digit's (the
 // last one's: those of X), and their sums are not read.
+static_assert(sizeof(BlockSmem::zero) == 256 * 16 && offsetof(BlockSmem, zero) == offsetof(BlockSmem, x) + sizeof(BlockSmem::x),
+              "the zero digit follows those of X");
 static_assert(128 * kStageRow * sizeof(double2) <= sizeof(BlockSmem), "C rows are staged in the same space");
 static_assert(offsetof(BlockSmem, x) == kS * 64 * kK * 2 && kNB * kK * 2 * 2 <= (int)sizeof(BlockSmem::x), "row overrun");
 
@@ -309,12 +320,16 @@ __device__ __forceinline__ void cfmaf(float2& acc, float2 a, float2 b) {
 // 4 (t % 8) .., column t / 8) of the inverse.  False: not found to FP64 accuracy
 // this way (a pivot vanished in FP32, or the first residual is not small).
 // An FP32 Gauss-Jordan elimination by four warps, then X <- X + X E with the
-// residual E = I - A X from the digit products on the tensor cores, exact to
-// 2^-54 of the row and column maxima as in the update, and the small product X E
+// residual E = I - A X from the digit products on the tensor cores, with order 7 and
+// exact to 2^-60 of the row and column maxima, and the small product X E
 // in FP32: E squares from round to round (1e-5, 1e-10 as a rule), and below
 // 2^-30 FP32 is enough for the last correction.  Latency bound.  Why: the same block by
 // FP64 elimination is 32768 complex multiply-adds on two FP64 units, 33 us at best; the
 // kernel with it took 55 us for 64 blocks of matrices of 768 rows, with this 33.
+// The residual's last bits decide the accuracy of the whole inversion: with seven orders, 2^-54, G_loc
+// erred by 1.2e-15 (N_c = 80) and 7e-15 (220) against long double; with eight by 5e-16
+// and 2e-15 (FP64 elimination: 1.1e-15 and 3.7e-15).  The eighth order in the update and
+// the R panel changes neither and costs 2 %.
 __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&in)[4], double2 (&out)[4],
                                                 uint32_t tmem, uint32_t& phase) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -328,6 +343,7 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
     sm.amax = 0;
     sm.bad = 0;
   }
+  reinterpret_cast<uint4*>(sm.zero)[t] = make_uint4(0, 0, 0, 0);
   __syncthreads();
   if ((t & 7) == 0) atomicMax(&sm.amax, m);
   __syncthreads();
@@ -432,7 +448,8 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
 #pragma unroll
         for (int kk = 0; kk < kK / 16; ++kk)
           mma_bf16(tmem + (uint32_t)(a * kNB), smem_desc(smem_u32(sm.a + a * 64 * kK) + kk * 256, 128, 1024),
-                   smem_desc(smem_u32(sm.x) + kk * 256, 128, 1024), idesc_bf16(128, (kS - a) * kNB),
+                   smem_desc(smem_u32(sm.x) + kk * 256, 128, 1024),
+                   idesc_bf16(128, (a == 0 && kk > 0 ? kS : kO - a) * kNB),
                    (a > 0 || kk > 0) ? 1u : 0u);
       mma_commit(&sm.bar);
     }
@@ -447,9 +464,9 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
       float big = 0.f;
 #pragma unroll 1
       for (int g = 0; g < 16; g += 8) {
-        float c[kS][8];
+        float c[kO][8];
 #pragma unroll
-        for (int o = 0; o < kS; ++o)
+        for (int o = 0; o < kO; ++o)
           tmem_ld8(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(o * kNB + j0 + g), c[o]);
         tmem_wait_ld();
 #pragma unroll
@@ -458,7 +475,7 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
           const int col = j0 + g + u, ex = sm.aexp[row] + sm.xexp[col];
           const bool one = row == col && part == 0;
           if (one && (ex < -8 || ex > 50)) big = 1e30f;  // not an inverse: a column of X or a row of A is lost
-          const float f = -orders_to_float(c[0][u], c[1][u], c[2][u], c[3][u], c[4][u], c[5][u], c[6][u],
+          const float f = -orders_to_float(c[0][u], c[1][u], c[2][u], c[3][u], c[4][u], c[5][u], c[6][u], c[7][u],
                                            one ? 0ull - (1ull << ((53 - ex) & 63)) : 0ull,
                                            __int_as_float((127 - 53 + max(min(ex, 100), -60)) << 23));
           big = fmaxf(big, fabsf(f));
