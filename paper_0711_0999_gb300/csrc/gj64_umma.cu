@@ -14,9 +14,10 @@
 // = sum_s q_s 256^(6-s), |q_s| <= 128, exact in bf16.  A digit product summed
 // over the 64 reals of K is below 2^20 and the up to seven products of one
 // order o = a + b below 7 2^20 < 2^24, so FP32 accumulation in TMEM is exact.
-// The 28 products of order <= 6 are kept (what is left out is 2^-56 of the row
-// and column maxima), their sums are put together in 64-bit integers and
-// rounded once to FP64: the result carries less rounding than 64 FP64 FMAs.
+// The 28 products of order <= 6 are kept (each left out is below 2^-56 of the row
+// and column maxima, all of them together about 2^-53), their sums are put together
+// in 64-bit integers and rounded once to FP64.  The whole inversion errs less than
+// in FP64 FMAs (figures at refined_inverse).
 //
 // One MMA per digit a of the left operand takes all its partners b = 0 .. 6-a
 // at once: the right operand's digits lie back to back in shared memory, and
