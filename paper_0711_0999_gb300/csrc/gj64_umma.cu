@@ -319,7 +319,12 @@ __device__ __forceinline__ void cfmaf(float2& acc, float2 a, float2 b) {
 // The inverse of a 32 x 32 FP64 block by 256 threads.  Thread t brings entries
 // in[0 .. 3] = (row t / 8, columns 4 (t % 8) ..) and gets out[0 .. 3] = (rows
 // 4 (t % 8) .., column t / 8) of the inverse.  False: not found to FP64 accuracy
-// this way (a pivot vanished in FP32, or the first residual is not small).
+// this way (the first residual is not small), or perhaps singular by the measure
+// of `recip`, a pivot of at most 1e-12, which only the FP64 elimination can tell:
+// a small FP32 pivot, or a large inverse.  (The Schur complement of a singular
+// matrix is rounding noise, which has an inverse as good as any.  Over contours of
+// 26 to 1500 rows with U from 0.3 to 2 the smallest pivot is 0.15, so no such
+// block takes the elimination.)
 // An FP32 Gauss-Jordan elimination by four warps, then X <- X + X E with the
 // residual E = I - A X from the digit products on the tensor cores, with order 7 and
 // exact to 2^-60 of the row and column maxima, and the small product X E
@@ -353,6 +358,10 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
   const int ea = (int)(am >> 20) - 1022, e = ea > 20 || ea < -20 ? ea : 0;
   if (am >= 0x7ff00000u || am < (24u << 20) || ea > 900) return false;
   const double sc = __hiloint2double((1023 - e) << 20, 0);
+  // A pivot of at most 2^-10 of the block, or of about 1e-12 before scaling, is left to the FP64 elimination
+  // and its test: FP32 cannot tell it from its own rounding.
+  const int tiny2 = 2 * (max(ea - 10, -39) - e);
+  const float pmin = __int_as_float((127 + max(-126, min(127, tiny2))) << 23);
   const int be = row_biased(m);
   {
     long long y[8];
@@ -391,7 +400,7 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
           p[c] = make_float2(__shfl_sync(0xffffffffu, v[c].x, k), __shfl_sync(0xffffffffu, v[c].y, k));
         if (warp == kw) {
           const float pm = p[kc].x * p[kc].x + p[kc].y * p[kc].y;
-          good = good && pm > 1e-30f;
+          good = good && pm > pmin;
           float rm;
           asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rm) : "f"(pm));
           const float2 pinv = make_float2(p[kc].x * rm, -p[kc].y * rm);
@@ -426,7 +435,7 @@ __device__ __forceinline__ bool refined_inverse(BlockSmem& sm, const double2 (&i
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     const int bx = row_biased(mx);
-    if ((t & 7) == 0) sm.xexp[j] = bx - 1022;
+    if ((t & 7) == 0) sm.xexp[j] = bx - 1022 - e > 39 ? 1000 : bx - 1022;  // about 1e12 and more: as a lost column
     if (t == 0) sm.emax = 0;
     long long y[8];
 #pragma unroll
