@@ -1573,7 +1573,8 @@ __global__ void __launch_bounds__(1024) refine_select_kernel(const double* __res
                                                              int* __restrict__ flags) {
   extern __shared__ double sorted[];  // npow values, a power of two >= nq, if it fits; else npow = 0
   __shared__ double red[1024];
-  __shared__ double sh_lo, sh_cut;
+  __shared__ double sh_lo;
+  __shared__ unsigned long long sh_cut;  // bits of a non-negative double: they order like its values
   const int t = threadIdx.x;
   auto wt = [&](int q) { return fabs(wq[q]) * (1.0 + fabs(eps[q]) + fabs(ebar[q])); };
   auto block_sum = [&](double v) {
@@ -1611,7 +1612,7 @@ __global__ void __launch_bounds__(1024) refine_select_kernel(const double* __res
     double run = 0.0;
     for (int i = i0; i < i1; ++i) run += sorted[i];
     red[t] = run;
-    if (t == 0) sh_cut = isnan(tail) ? -1.0 : INFINITY;  // a NaN among the weights: nothing is skipped
+    if (t == 0) sh_cut = (unsigned long long)__double_as_longlong(INFINITY);
     __syncthreads();
     for (int s = 1; s < 1024; s <<= 1) {  // inclusive scan
       const double add = t >= s ? red[t - s] : 0.0;
@@ -1619,15 +1620,20 @@ __global__ void __launch_bounds__(1024) refine_select_kernel(const double* __res
       red[t] += add;
       __syncthreads();
     }
+    // The first weight past the tail.  A run ends at the very sum from which the next one starts: the
+    // sums then pass from zero to the total without a gap, and one of them passes the tail (a run's own
+    // running sum may end a rounding below the scan's, and a tail in between was passed by neither).
+    // The scan's roundings may let a sum fall back, so more than one weight can pass it: the least counts.
     double sum = t > 0 ? red[t - 1] : 0.0;
-    for (int i = i0; i < i1; ++i) {  // one thread finds the first weight past the tail
-      const double next = sum + sorted[i];
-      if (sum <= tail && !(next <= tail)) sh_cut = sorted[i];
+    for (int i = i0; i < i1; ++i) {
+      const double next = i + 1 < i1 ? sum + sorted[i] : red[t];
+      if (sum <= tail && !(next <= tail)) atomicMin(&sh_cut, (unsigned long long)__double_as_longlong(sorted[i]));
       sum = next;
     }
     __syncthreads();
     if (t == 0) {
-      const double cut = sh_cut, l2 = log2(cut);
+      // a NaN among the weights: nothing is skipped
+      const double cut = isnan(tail) ? -1.0 : __longlong_as_double((long long)sh_cut), l2 = log2(cut);
       for (int it = 0; it < 80; ++it) {
         const double mid = 0.5 * (lo + hi);
         if (mid == lo || mid == hi) break;  // nothing moves any more
