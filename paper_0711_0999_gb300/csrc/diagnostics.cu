@@ -58,6 +58,7 @@ __global__ void moments_kernel(const double2* __restrict__ g, int n, int nt, dou
 // terms where a thread per omega formed one per term (455 us for 5 times x 401
 // frequencies of N_c = 1500 on 20 CTAs, serial in k).  What is left is latency:
 // the staging loads and one sincos after another.
+// CTAs along y take frequencies in strides.
 constexpr int kDosTerms = 1024;
 constexpr int kDosWarps = 8;
 __global__ void __launch_bounds__(32 * kDosWarps)
@@ -65,50 +66,59 @@ __global__ void __launch_bounds__(32 * kDosWarps)
                const double* __restrict__ omega, int n_omega, double* __restrict__ rho) {
   __shared__ double2 term[kDosTerms];
   const int a = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int w = blockIdx.y * kDosWarps + warp;
   const int m = m_list[a];
   const bool inside = m >= 0 && m < nt;
   const int kmax = inside ? min(m, nt - 1 - m) : 0;  // the same for the whole CTA
-  const double h = 2.0 * dt, om = w < n_omega ? omega[w] : 0.0;
-  double im = 0.0;
-  for (int k0 = 0; kmax > 0 && k0 <= kmax; k0 += kDosTerms) {
-    const int cnt = min(kDosTerms, kmax + 1 - k0);
-    const int B = ((cnt + 31) >> 5) | 1;  // odd: the lanes' terms fall on different banks
-    __syncthreads();
+  const double h = 2.0 * dt;
+  auto stage = [&](int k0, int cnt) {
     for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
       const double2 r = retarded_at(g, n, nt, m + k0 + k, m - k0 - k);
       const double wk = (k0 + k == 0 || k0 + k == kmax) ? 0.5 * h : h;
       term[k] = make_double2(wk * r.x, wk * r.y);
     }
-    __syncthreads();
-    double bs, bc, ls, lc;
-    sincos(om * (lane * h), &bs, &bc);
-    double2 p = make_double2(0.0, 0.0);
-    const int l0 = lane * B;
-    for (int b0 = 0; b0 < B; b0 += 32) {  // B is 33 when 1024 terms are staged
-      if (b0 > 0) sincos(om * ((b0 + lane) * h), &bs, &bc);
-      const int nb = min(32, B - b0);
-      for (int b = 0; b < nb; ++b) {
-        const double c = __shfl_sync(0xffffffffu, bc, b), sn = __shfl_sync(0xffffffffu, bs, b);
-        if (l0 + b0 + b < cnt) {
-          const double2 r = term[l0 + b0 + b];
-          p.x = fma(c, r.x, fma(-sn, r.y, p.x));
-          p.y = fma(c, r.y, fma(sn, r.x, p.y));
+  };
+  auto store = [&](long long w, double im) {
+    rho[(size_t)a * n_omega + w] = !inside ? NAN : kmax == 0 ? 0.0 : -im / M_PI;
+  };
+  for (long long w0 = (long long)blockIdx.y * kDosWarps; w0 < n_omega; w0 += (long long)gridDim.y * kDosWarps) {
+    const long long w = w0 + warp;
+    const double om = w < n_omega ? omega[w] : 0.0;
+    double im = 0.0;
+    for (int k0 = 0; kmax > 0 && k0 <= kmax; k0 += kDosTerms) {
+      const int cnt = min(kDosTerms, kmax + 1 - k0);
+      const int B = ((cnt + 31) >> 5) | 1;  // odd: the lanes' terms fall on different banks
+      __syncthreads();
+      stage(k0, cnt);
+      __syncthreads();
+      double bs, bc, ls, lc;
+      sincos(om * (lane * h), &bs, &bc);
+      double2 p = make_double2(0.0, 0.0);
+      const int l0 = lane * B;
+      for (int b0 = 0; b0 < B; b0 += 32) {  // B is 33 when 1024 terms are staged
+        if (b0 > 0) sincos(om * ((b0 + lane) * h), &bs, &bc);
+        const int nb = min(32, B - b0);
+        for (int b = 0; b < nb; ++b) {
+          const double c = __shfl_sync(0xffffffffu, bc, b), sn = __shfl_sync(0xffffffffu, bs, b);
+          if (l0 + b0 + b < cnt) {
+            const double2 r = term[l0 + b0 + b];
+            p.x = fma(c, r.x, fma(-sn, r.y, p.x));
+            p.y = fma(c, r.y, fma(sn, r.x, p.y));
+          }
         }
       }
+      if (l0 < cnt) {
+        // one phase for B terms: the rounding of its angle, which they would share, is put back
+        const double k = (double)(k0 + l0), t = k * h, te = fma(k, h, -t);
+        const double an = om * t, ae = fma(om, t, -an) + om * te;
+        sincos(an, &ls, &lc);
+        const double s1 = fma(lc, ae, ls), c1 = fma(-ls, ae, lc);
+        im += c1 * p.y + s1 * p.x;  // Im(e^{i om s} G^R)
+      }
     }
-    if (l0 < cnt) {
-      // one phase for B terms: the rounding of its angle, which they would share, is put back
-      const double k = (double)(k0 + l0), t = k * h, te = fma(k, h, -t);
-      const double an = om * t, ae = fma(om, t, -an) + om * te;
-      sincos(an, &ls, &lc);
-      const double s1 = fma(lc, ae, ls), c1 = fma(-ls, ae, lc);
-      im += c1 * p.y + s1 * p.x;  // Im(e^{i om s} G^R)
-    }
-  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) im += __shfl_xor_sync(0xffffffffu, im, o);
-  if (lane == 0 && w < n_omega) rho[(size_t)a * n_omega + w] = !inside ? NAN : kmax == 0 ? 0.0 : -im / M_PI;
+    for (int o = 16; o > 0; o >>= 1) im += __shfl_xor_sync(0xffffffffu, im, o);
+    if (lane == 0 && w < n_omega) store(w, im);
+  }
 }
 
 }  // namespace
@@ -137,8 +147,10 @@ extern "C" int nedmft_dos(const nedmft_contour* c, const nedmft_c128* gloc_d, co
   if (n_avg == 0 || n_omega == 0) return NEDMFT_OK;  // nothing to write; the arrays may be NULL
   if (!m_d || !omega_d || !rho_d) return set_error(NEDMFT_EINVAL, "dos: NULL argument");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  dos_kernel<<<dim3(n_avg, ceil_div(n_omega, kDosWarps)), 32 * kDosWarps, 0, st>>>(reinterpret_cast<const double2*>(gloc_d), c->n_c,
-                                                                  c->n_t, c->dt, m_d, omega_d, n_omega, rho_d);
+  // at most 65535 CTAs along y, which take every so many frequencies past that
+  const int blocks = (int)(((long long)n_omega + kDosWarps - 1) / kDosWarps);
+  dos_kernel<<<dim3(n_avg, blocks < 65535 ? blocks : 65535), 32 * kDosWarps, 0, st>>>(
+      reinterpret_cast<const double2*>(gloc_d), c->n_c, c->n_t, c->dt, m_d, omega_d, n_omega, rho_d);
   NED_LAUNCH_CHECK("dos_kernel");
   return NEDMFT_OK;
 }

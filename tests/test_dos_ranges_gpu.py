@@ -1,0 +1,44 @@
+"""The density of states at the ends of its ranges: more frequencies than one
+launch takes along a grid's second dimension."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import nedmft_oracle as O
+from paper_0711_0999_gb300 import api
+from paper_0711_0999_gb300.build import build_library
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    build_library()
+
+
+def setup(n_t, seed=4, dt=0.05):
+    c, g = (f(0.0, dt * n_t, dt, 0.5, 0.25) for f in (O.contour_grid, api.contour_grid))
+    rng = np.random.default_rng(seed)
+    return c, g, rng.standard_normal((c.n_c, c.n_c)) + 1j * rng.standard_normal((c.n_c, c.n_c)), rng
+
+
+def bound(c, gl, m, omega):
+    """Rounding of both sums: one rounding per term and addition, and of the phases, 3 eps |omega| t."""
+    k = min(m, c.n_t - 1 - m) + 1
+    terms = 2 * c.dt * sum(abs(O.retarded(c, gl, m + i, m - i)) for i in range(k))
+    return 2 * np.finfo(np.float64).eps * (k + 4 + 3 * np.abs(omega).max() * 2 * c.dt * k) * terms / np.pi
+
+
+# up to 7 and up to 81 relative times
+@pytest.mark.parametrize("n_t", [12, 161])
+def test_more_frequencies_than_one_launch_takes(n_t):
+    c, g, gl, rng = setup(n_t)
+    omega = rng.uniform(-5.0, 5.0, 8 * 65535 + 1003)
+    m_index = [n_t // 2 - 1, 0, n_t // 2, -1]
+    rho = api.dos(g, torch.as_tensor(gl, device="cuda"), m_index, omega).cpu().numpy()
+    for row, m in enumerate(m_index[:3]):
+        assert np.abs(rho[row] - O.dos(c, gl, m, omega)).max() <= bound(c, gl, m, omega)
+    assert np.isnan(rho[3]).all()
