@@ -109,7 +109,9 @@ __global__ void __launch_bounds__(32 * kDosWarps)
       if (l0 < cnt) {
         // one phase for B terms: the rounding of its angle, which they would share, is put back
         const double k = (double)(k0 + l0), t = k * h, te = fma(k, h, -t);
-        const double an = om * t, ae = fma(om, t, -an) + om * te;
+        const double an = om * t;
+        double ae = fma(om, t, -an) + om * te;
+        if (fabs(ae) > 0x1p-26) ae = 0.0;  // |om t| beyond 2^27: no more than a lone term's angle has
         sincos(an, &ls, &lc);
         const double s1 = fma(lc, ae, ls), c1 = fma(-ls, ae, lc);
         im += c1 * p.y + s1 * p.x;  // Im(e^{i om s} G^R)

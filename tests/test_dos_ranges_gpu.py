@@ -1,5 +1,6 @@
 """The density of states at the ends of its ranges: more frequencies than one
-launch takes along a grid's second dimension."""
+launch takes along a grid's second dimension, and frequencies whose phases carry
+no information any more."""
 
 import numpy as np
 import pytest
@@ -42,3 +43,15 @@ def test_more_frequencies_than_one_launch_takes(n_t):
     for row, m in enumerate(m_index[:3]):
         assert np.abs(rho[row] - O.dos(c, gl, m, omega)).max() <= bound(c, gl, m, omega)
     assert np.isnan(rho[3]).all()
+
+
+# phases far beyond 2^53: any value of a phase is as good as another, but it is a phase
+@pytest.mark.parametrize("n_t", [21, 301, 2301])
+def test_huge_frequencies_stay_within_the_sum_of_the_terms(n_t):
+    c, g, gl, _ = setup(n_t)
+    omega = np.array([1e10, -1e15, 3e18, 1e22, -1e100, 1e300])
+    m = n_t // 2
+    rho = api.dos(g, torch.as_tensor(gl, device="cuda"), [m], omega).cpu().numpy()[0]
+    k = min(m, n_t - 1 - m) + 1
+    top = 2 * c.dt * sum(abs(O.retarded(c, gl, m + i, m - i)) for i in range(k)) / np.pi
+    assert (np.abs(rho) <= top * (1 + 1e-12)).all()
