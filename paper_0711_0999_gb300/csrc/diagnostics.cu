@@ -58,13 +58,20 @@ __global__ void moments_kernel(const double2* __restrict__ g, int n, int nt, dou
 // terms where a thread per omega formed one per term (455 us for 5 times x 401
 // frequencies of N_c = 1500 on 20 CTAs, serial in k).  What is left is latency:
 // the staging loads and one sincos after another.
+// With few relative times those 64 sincos of a frequency are more than its terms:
+// up to `direct` times, a lane per omega, the terms dealt to the CTA's warps.
+// FP64 bound: K sincos per frequency.  The line: 64 terms where 32 frequencies per
+// SM keep all of them busy, else 16, the eight warps' sincos of the other form on
+// one SM (up to 10 relative times, 5 averages x 100000 and 12 x 1000 frequencies:
+// 2455 and 91 us with a warp per omega, 244 and 43 so).
 // CTAs along y take frequencies in strides.
 constexpr int kDosTerms = 1024;
 constexpr int kDosWarps = 8;
 __global__ void __launch_bounds__(32 * kDosWarps)
     dos_kernel(const double2* __restrict__ g, int n, int nt, double dt, const int* __restrict__ m_list,
-               const double* __restrict__ omega, int n_omega, double* __restrict__ rho) {
+               const double* __restrict__ omega, int n_omega, int direct, double* __restrict__ rho) {
   __shared__ double2 term[kDosTerms];
+  __shared__ double part[kDosWarps][32];
   const int a = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m = m_list[a];
   const bool inside = m >= 0 && m < nt;
@@ -80,11 +87,34 @@ __global__ void __launch_bounds__(32 * kDosWarps)
   auto store = [&](long long w, double im) {
     rho[(size_t)a * n_omega + w] = !inside ? NAN : kmax == 0 ? 0.0 : -im / M_PI;
   };
+  if (kmax < direct) {
+    if ((long long)blockIdx.y * 32 >= n_omega) return;
+    if (kmax > 0) stage(0, kmax + 1);
+    __syncthreads();
+    for (long long w0 = (long long)blockIdx.y * 32; w0 < n_omega; w0 += (long long)gridDim.y * 32) {
+      const long long w = w0 + lane;
+      const double om = w < n_omega ? omega[w] : 0.0;
+      double im = 0.0;
+      for (int k = warp; kmax > 0 && k <= kmax; k += kDosWarps) {
+        double sn, cs;
+        sincos(om * (k * h), &sn, &cs);
+        im += cs * term[k].y + sn * term[k].x;  // Im(e^{i om s} G^R)
+      }
+      part[warp][lane] = im;
+      __syncthreads();
+      if (warp == 0 && w < n_omega) {
+        for (int q = 1; q < kDosWarps; ++q) im += part[q][lane];
+        store(w, im);
+      }
+      __syncthreads();
+    }
+    return;
+  }
   for (long long w0 = (long long)blockIdx.y * kDosWarps; w0 < n_omega; w0 += (long long)gridDim.y * kDosWarps) {
     const long long w = w0 + warp;
     const double om = w < n_omega ? omega[w] : 0.0;
     double im = 0.0;
-    for (int k0 = 0; kmax > 0 && k0 <= kmax; k0 += kDosTerms) {
+    for (int k0 = 0; k0 <= kmax; k0 += kDosTerms) {
       const int cnt = min(kDosTerms, kmax + 1 - k0);
       const int B = ((cnt + 31) >> 5) | 1;  // odd: the lanes' terms fall on different banks
       __syncthreads();
@@ -149,10 +179,17 @@ extern "C" int nedmft_dos(const nedmft_contour* c, const nedmft_c128* gloc_d, co
   if (n_avg == 0 || n_omega == 0) return NEDMFT_OK;  // nothing to write; the arrays may be NULL
   if (!m_d || !omega_d || !rho_d) return set_error(NEDMFT_EINVAL, "dos: NULL argument");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // at most 65535 CTAs along y, which take every so many frequencies past that
-  const int blocks = (int)(((long long)n_omega + kDosWarps - 1) / kDosWarps);
+  int sms = 0;
+  if (int rc = device_sm_count(&sms)) return rc;
+  const long long total = (long long)n_avg * n_omega;
+  const int direct = total >= 32ll * sms ? 64 : 16;
+  // 32 frequencies per CTA where that leaves 32 CTAs per SM (fewer idle CTAs with few relative times); at most
+  // 65535 CTAs along y, which take every so many frequencies past that
+  const int per = total >= 1024ll * sms ? 32 : kDosWarps;
+  const int blocks = (int)(((long long)n_omega + per - 1) / per);
   dos_kernel<<<dim3(n_avg, blocks < 65535 ? blocks : 65535), 32 * kDosWarps, 0, st>>>(
-      reinterpret_cast<const double2*>(gloc_d), c->n_c, c->n_t, c->dt, m_d, omega_d, n_omega, rho_d);
+      reinterpret_cast<const double2*>(gloc_d), c->n_c, c->n_t, c->dt, m_d, omega_d, n_omega, direct,
+      rho_d);
   NED_LAUNCH_CHECK("dos_kernel");
   return NEDMFT_OK;
 }

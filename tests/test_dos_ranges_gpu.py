@@ -1,6 +1,7 @@
 """The density of states at the ends of its ranges: more frequencies than one
-launch takes along a grid's second dimension, and frequencies whose phases carry
-no information any more."""
+launch takes along a grid's second dimension, frequencies whose phases carry no
+information any more, and the numbers of relative times at which the kernel
+changes its form."""
 
 import numpy as np
 import pytest
@@ -55,3 +56,15 @@ def test_huge_frequencies_stay_within_the_sum_of_the_terms(n_t):
     k = min(m, n_t - 1 - m) + 1
     top = 2 * c.dt * sum(abs(O.retarded(c, gl, m + i, m - i)) for i in range(k)) / np.pi
     assert (np.abs(rho) <= top * (1 + 1e-12)).all()
+
+
+# 1 to 65 relative times, with few frequencies and with enough for every SM
+@pytest.mark.parametrize("n_omega", [1, 33, 700])
+def test_numbers_of_relative_times(n_omega):
+    c, g, gl, rng = setup(160)
+    m_index = [0, 1, 2, 7, 8, 14, 15, 16, 17, 62, 63, 64, 65, 79, 80, 96, 159, 160]
+    omega = rng.uniform(-5.0, 5.0, n_omega)
+    rho = api.dos(g, torch.as_tensor(gl, device="cuda"), m_index, omega).cpu().numpy()
+    for row, m in enumerate(m_index[:-1]):
+        assert np.abs(rho[row] - O.dos(c, gl, m, omega)).max() <= bound(c, gl, m, omega), m
+    assert np.isnan(rho[-1]).all()
