@@ -62,7 +62,7 @@ int default_batch(const nedmft_contour& c, int nq, Path path, int width) {
       // every step of 32 columns is three launches for the whole batch, two of
       // them latency bound: larger batches while a step is short (1024 points of
       // 80 rows 4286 / 3100 / 2420 / 2315 us in batches of 76 / 152 / 304 / 1024;
-      // of 220 rows 11.9 / 10.6 / 8.9 / 8.0 ms)
+      // of 220 rows 11.9 / 10.6 / 8.9 / 8.0 ms))
       per = sizeof(double2) * np * np + gj64_scratch_bytes((int)np, 1);
       cap = np <= 256 ? 1024 : np <= 512 ? 608 : 304;
       break;
@@ -93,6 +93,7 @@ LatticeLayout lattice_layout(const nedmft_contour& c, int nq, nedmft_precision p
   L.np = padded_for(L.path, c.n_c, width);
   if (batch <= 0) batch = t.batch;
   L.mb = batch > 0 ? (batch < nq ? batch : nq) : default_batch(c, nq, L.path, width);
+  if (L.path == Path::Blocked64 && L.mb > 65535) L.mb = 65535;  // the points of a batch lie along a grid's y
   const size_t n = c.n_c, np = L.np, mb = L.mb;
   L.S = align256(sizeof(double2) * n * n);
   L.gscratch = align256(sizeof(double2) * n * n);
