@@ -62,9 +62,11 @@ int default_batch(const nedmft_contour& c, int nq, Path path, int width) {
       // every step of 32 columns is three launches for the whole batch, two of
       // them latency bound: larger batches while a step is short (1024 points of
       // 80 rows 4286 / 3100 / 2420 / 2315 us in batches of 76 / 152 / 304 / 1024;
-      // of 220 rows 11.9 / 10.6 / 8.9 / 8.0 ms))
+      // of 220 rows 11.9 / 10.6 / 8.9 / 8.0 ms); above 1024 rows the workspace (13 and
+      // 61 GB for 304 points of 1500 and 3400 rows) is not worth what is left to gain
+      // (608 points of 1500 rows 521 / 516 ms in batches of 152 / 304)
       per = sizeof(double2) * np * np + gj64_scratch_bytes((int)np, 1);
-      cap = np <= 256 ? 1024 : np <= 512 ? 608 : 304;
+      cap = np <= 256 ? 1024 : np <= 512 ? 608 : np <= 1024 ? 304 : 152;
       break;
     case Path::MixedUmma: per = umma_batch_bytes_per_matrix((int)np, width); cap = umma_default_batch((int)np); break;
   }

@@ -24,3 +24,9 @@ def test_fp64_batches_fit_one_launch():
         assert api.lattice_batch(g, nq, "fp64") == 65535
     finally:
         api.lattice_set_tuning(g, nq, "fp64")
+
+
+# 16 bytes an entry, 152 matrices of up to the next multiple of 128 rows, and a tenth for the operands
+@pytest.mark.parametrize("n_t,rows", [(700, 1536), (1650, 3456)])
+def test_fp64_workspace_of_long_contours(n_t, rows):
+    assert api.lattice_workspace_size(contour(n_t, 100), 2809, "fp64") <= 1.1 * 16 * rows**2 * 152
