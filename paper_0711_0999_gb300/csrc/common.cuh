@@ -194,5 +194,6 @@ __device__ __forceinline__ int unshift_col(int j, int n, bool sh) { return sh ? 
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+inline char* align256(void* p) { return reinterpret_cast<char*>(align256(reinterpret_cast<size_t>(p))); }
 
 }  // namespace nedmft

@@ -93,7 +93,7 @@ using namespace nedmft;
 extern "C" size_t nedmft_impurity_workspace_size(const nedmft_contour* c) {
   if (!c || c->n_c < 1) return 0;
   size_t n = (size_t)c->n_c;
-  return 3 * align256(sizeof(double2) * n * n) + pivot_inverse_workspace((int)n);
+  return 3 * align256(sizeof(double2) * n * n) + pivot_inverse_workspace((int)n) + 256;  // aligned to 256 bytes inside
 }
 
 extern "C" int nedmft_impurity_update(const nedmft_contour* c, const nedmft_model* m, const nedmft_c128* gloc_d,
@@ -113,7 +113,7 @@ extern "C" int nedmft_impurity_update(const nedmft_contour* c, const nedmft_mode
   ModelDev md{m->U, m->E, m->w1, isnan(m->mu) ? m->U / 2 : m->mu};
   const int n = cd.n;
   const size_t mat = align256(sizeof(double2) * (size_t)n * n);
-  char* p = static_cast<char*>(ws_d);
+  char* p = align256(ws_d);  // the digit images are written 32 bytes at a time
   double2* a0 = reinterpret_cast<double2*>(p); p += mat;
   double2* ah = reinterpret_cast<double2*>(p); p += mat;
   double2* g = reinterpret_cast<double2*>(p); p += mat;

@@ -147,8 +147,6 @@ __global__ void target_kernel(ContourDev c, ModelDev m, const double2* __restric
   }
 }
 
-char* aligned(void* ws) { return reinterpret_cast<char*>(align256(reinterpret_cast<uintptr_t>(ws))); }
-
 int grid_for(size_t n) {
   size_t b = (n + 255) / 256;
   return (int)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b));
@@ -172,7 +170,7 @@ extern "C" int nedmft_mlp_forward(const float* params_d, const float* x_d, int32
   if (ws_bytes < nedmft_mlp_workspace_size(n)) return set_error(NEDMFT_ENOMEM, "mlp_forward: workspace too small");
   MlpInput in;
   in.x = x_d;
-  return mlp_forward(params_d, in, n, y_d, false, true, 1.f, true, aligned(ws_d),
+  return mlp_forward(params_d, in, n, y_d, false, true, 1.f, true, align256(ws_d),
                      static_cast<cudaStream_t>(stream));
 }
 
@@ -181,7 +179,7 @@ extern "C" int nedmft_mlp_grad(const float* params_d, const float* x_d, const fl
   if (!params_d || !x_d || !target_d || !grad_d || !loss_d || !ws_d || n < 1)
     return set_error(NEDMFT_EINVAL, "mlp_grad: bad argument");
   if (ws_bytes < nedmft_mlp_workspace_size(n)) return set_error(NEDMFT_ENOMEM, "mlp_grad: workspace too small");
-  return mlp_gradient(params_d, x_d, target_d, n, grad_d, loss_d, aligned(ws_d),
+  return mlp_gradient(params_d, x_d, target_d, n, grad_d, loss_d, align256(ws_d),
                       static_cast<cudaStream_t>(stream));
 }
 
@@ -238,7 +236,7 @@ extern "C" int nedmft_sigma_warm_start(const nedmft_contour* c, const nedmft_mod
     return set_error(NEDMFT_ENOMEM, "sigma_warm_start: workspace too small");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t n = c->n_c, n2 = n * n;
-  char* p = aligned(ws_d);
+  char* p = align256(ws_d);
   char* scratch = p; p += mlp_forward_scratch();
   float* row = reinterpret_cast<float*>(p); p += align256(sizeof(float) * n * 6);
   float* rel = reinterpret_cast<float*>(p); p += align256(sizeof(float) * n2);
