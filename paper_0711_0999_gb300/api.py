@@ -183,6 +183,12 @@ def current(grid: Grid, model: N.Model, sigma, eps, ebar, wq, precision="fp64", 
     return j, ji
 
 
+def autotune_candidates(grid: Grid, nq: int, precision="mixed_bf16") -> list[int]:
+    """Batch sizes that lattice_autotune times unless told otherwise: the one in use (so tuning never
+    makes a step slower) and others up to 304 points."""
+    return sorted({76, 114, 152, 228, 304, lattice_batch(grid, nq, precision)})
+
+
 def lattice_autotune(grid: Grid, model: N.Model, sigma, eps, ebar, wq, precision="mixed_bf16", candidates=None,
                      stream=None):
     """Times one lattice step per candidate batch size and makes the fastest the
@@ -193,7 +199,7 @@ def lattice_autotune(grid: Grid, model: N.Model, sigma, eps, ebar, wq, precision
     nq = eps_t.numel()
     p = _prec(precision)
     if candidates is None:
-        candidates = [76, 114, 152, 228, 304]
+        candidates = autotune_candidates(grid, nq, precision)
     cand = (N.c_int32 * len(candidates))(*candidates)
     need = max(N.lib().nedmft_lattice_workspace_size(ctypes.byref(grid.contour), nq, p, int(b)) for b in candidates)
     if need == 0:
