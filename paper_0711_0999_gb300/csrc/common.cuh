@@ -52,14 +52,6 @@ int max_active_clusters(const void* kern, int block, int smem_bytes, int* out);
 
 // ------------------------------------------------------------------ complex
 
-template <class T> struct cplx;
-template <> struct cplx<double> { using type = double2; };
-template <> struct cplx<float> { using type = float2; };
-template <class T> using cplx_t = typename cplx<T>::type;
-
-template <class T> __host__ __device__ __forceinline__ cplx_t<T> mk(T re, T im) {
-  cplx_t<T> z; z.x = re; z.y = im; return z;
-}
 __host__ __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
@@ -70,32 +62,17 @@ __host__ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-// acc += a * b
-__device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
-  acc.x = fma(a.x, b.x, acc.x); acc.x = fma(-a.y, b.y, acc.x);
-  acc.y = fma(a.x, b.y, acc.y); acc.y = fma(a.y, b.x, acc.y);
-}
-__device__ __forceinline__ void cfma(float2& acc, float2 a, float2 b) {
-  acc.x = fmaf(a.x, b.x, acc.x); acc.x = fmaf(-a.y, b.y, acc.x);
-  acc.y = fmaf(a.x, b.y, acc.y); acc.y = fmaf(a.y, b.x, acc.y);
-}
-__device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
-__device__ __forceinline__ float cabs2(float2 a) { return a.x * a.x + a.y * a.y; }
 // 1/z with a guard: returns false (and a large finite value) if |z| is below `tiny`.
-template <class T> __device__ __forceinline__ bool cinv_guard(cplx_t<T> z, cplx_t<T>& out, T tiny) {
-  T m = z.x * z.x + z.y * z.y;
+__device__ __forceinline__ bool cinv_guard(double2 z, double2& out, double tiny) {
+  const double m = z.x * z.x + z.y * z.y;
   if (!(m > tiny * tiny)) {  // also catches NaN
-    out = mk<T>(T(1) / tiny, T(0));
+    out = make_double2(1.0 / tiny, 0.0);
     return false;
   }
-  T r = T(1) / m;
-  out = mk<T>(z.x * r, -z.y * r);
+  const double r = 1.0 / m;
+  out = make_double2(z.x * r, -z.y * r);
   return true;
 }
-template <class T> __device__ __forceinline__ cplx_t<T> cvt(double2 z);
-template <> __device__ __forceinline__ double2 cvt<double>(double2 z) { return z; }
-template <> __device__ __forceinline__ float2 cvt<float>(double2 z) { return make_float2((float)z.x, (float)z.y); }
-__device__ __forceinline__ double2 to_d(double2 z) { return z; }
 __device__ __forceinline__ double2 to_d(float2 z) { return make_double2((double)z.x, (double)z.y); }
 
 // ------------------------------------------------------------------ contour

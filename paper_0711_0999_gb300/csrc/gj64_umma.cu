@@ -46,11 +46,6 @@ constexpr int kBDig = 2 * kTn * kK;          // bf16 elements of one digit of a 
 constexpr int kBTile = kS * kBDig;
 constexpr int kPTile = kS * 64 * kK;         // ... of the 64 real rows of P
 
-__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = global_ns();
-  while (!mbar_test(bar, parity) && global_ns() - t0 < kDrainNs) {
-  }
-}
 // shared -> global bulk copy and FP64 reduction (add at L2), tracked by bulk groups
 __device__ __forceinline__ void bulk_store(double2* dst, const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
@@ -1155,10 +1150,6 @@ constexpr int kPanCand = 256;  // candidate rows of a CTA
 constexpr int kPanCtas = 8;    // most CTAs of a cluster
 constexpr int kPanRows = kPanCand * kPanCtas;
 
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 constexpr int kStagePitch = kNB + 1;  // staged candidate rows: conflict-free with a lane per row
 struct PanSmem {
   float4 prow[2][kNB / 2];  // the pivot row, from the step's column on (by step parity)
@@ -1289,11 +1280,11 @@ __global__ void __launch_bounds__(kPanThreads, 1)
   __syncthreads();
   choose_rows(sm, stage, A, np, n, k0);
   if (nq > 1) {
-    cluster_barrier();  // the first CTA has read its own candidates
+    cluster_sync();  // the first CTA has read its own candidates
     if (t < kNB)
       asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(cluster_addr(&sm.cand[q * kNB + t], 0)), "r"(sm.win[t])
                    : "memory");
-    cluster_barrier();
+    cluster_sync();
     if (q > 0) return;
     if (t >= (int)nq * kNB) sm.cand[t] = -1;
     __syncthreads();

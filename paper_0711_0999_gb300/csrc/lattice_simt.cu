@@ -1,7 +1,7 @@
-// CUDA-core kernels of the lattice step: S = W Sigma W, the fused B_q - S
-// generator, the dense G0 builder, Gauss-Jordan inversion (single-CTA for
-// small N_c, blocked and batched for large N_c), the refinement residual and
-// the FP64 quadrature / current reductions.
+// CUDA-core kernels of the lattice step: S = W Sigma W, the dense G0 builder,
+// the FP64 path's B_q - S generator, Gauss-Jordan inversion of small matrices
+// in shared memory (a CTA per point) and the FP64 quadrature / current
+// reductions.
 #include "lattice.cuh"
 
 namespace nedmft {
@@ -132,27 +132,25 @@ __device__ __forceinline__ void record_status(int* status, int code) {
 // In-place inverse of the n x n matrix `a` (row stride ld) held in shared
 // memory, no pivoting (the static row order makes the pivots safe), all
 // threads of the block participating.  `col` is n scratch entries.
-template <class T>
-__device__ void smem_gauss_jordan(cplx_t<T>* a, int n, int ld, cplx_t<T>* col, T tiny, int* status) {
-  using C = cplx_t<T>;
+__device__ void smem_gauss_jordan(double2* a, int n, int ld, double2* col, double tiny, int* status) {
   for (int k = 0; k < n; ++k) {
     for (int t = threadIdx.x; t < n; t += blockDim.x) col[t] = a[t * ld + k];
     __syncthreads();
-    C pinv;
-    bool ok = cinv_guard<T>(col[k], pinv, tiny);
+    double2 pinv;
+    bool ok = cinv_guard(col[k], pinv, tiny);
     if (!ok && threadIdx.x == 0) record_status(status, DS_SINGULAR);
     for (int t = threadIdx.x; t < n; t += blockDim.x) a[k * ld + t] = (t == k) ? pinv : cmul(a[k * ld + t], pinv);
     __syncthreads();
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
       int i = e / n, j = e % n;
       if (i == k) continue;
-      C f = col[i];
+      double2 f = col[i];
       if (j == k) {
-        C v = cmul(f, pinv);
-        a[i * ld + k] = mk<T>(-v.x, -v.y);
+        double2 v = cmul(f, pinv);
+        a[i * ld + k] = make_double2(-v.x, -v.y);
       } else {
-        C v = a[i * ld + j];
-        C r = a[k * ld + j];
+        double2 v = a[i * ld + j];
+        double2 r = a[k * ld + j];
         v.x -= f.x * r.x - f.y * r.y;
         v.y -= f.x * r.y + f.y * r.x;
         a[i * ld + j] = v;
@@ -180,7 +178,7 @@ __global__ void __launch_bounds__(512) gj_small_fp64_kernel(ContourDev c, ModelD
     a[e] = a_entry(c, m, eps, ebar, S, i, j);
   }
   __syncthreads();
-  smem_gauss_jordan<double>(a, n, n, col, 1e-12, status);
+  smem_gauss_jordan(a, n, n, col, 1e-12, status);
   double2* o = out + (size_t)b * n * n;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     int i = e / n, j = e % n;
