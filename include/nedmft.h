@@ -68,7 +68,10 @@ typedef enum {
    * shared memory on the FP64 units; above, blocked (32 columns per step) with
    * every product on the tensor cores (each operand row cut into seven 8-bit
    * integer digits of a common exponent, digit products exact in FP32, the
-   * sums rounded to FP64 once). */
+   * sums rounded to FP64 once).  Digits of a common exponent keep an entry to
+   * 2^-55 of its row's (column's) largest: results are accurate relative to
+   * the largest entries of a point's matrices, and an entry f times the
+   * largest to about 2^-53 / f of itself. */
   NEDMFT_FP64 = 0,
   /* bf16x3 (hi*hi + hi*lo + lo*hi) tcgen05 tensor-core Gauss-Jordan with
    * FP32 accumulation in TMEM; then, for every point outside the
@@ -222,7 +225,10 @@ int nedmft_g0_build(const nedmft_contour* c, const nedmft_model* m,
 
 /* Workspace bytes nedmft_lattice_gloc / nedmft_current need for this contour,
  * point count and precision.  `batch` = points solved concurrently
- * (0 = library default for n_c).  Returns 0 on a bad argument. */
+ * (0 = the tuned size, else the library default for n_c, which is chosen for
+ * speed and may take tens of GB for long contours; where memory is short,
+ * nedmft_lattice_set_tuning pins a smaller one).  FP64 batches are clamped to
+ * 65535 points.  Returns 0 on a bad argument. */
 size_t nedmft_lattice_workspace_size(const nedmft_contour* c, int32_t nq,
                                      nedmft_precision prec, int32_t batch);
 
