@@ -84,16 +84,16 @@ __global__ void __launch_bounds__(32 * kDosWarps)
       term[k] = make_double2(wk * r.x, wk * r.y);
     }
   };
-  auto store = [&](long long w, double im) {
+  auto store = [&](unsigned w, double im) {
     rho[(size_t)a * n_omega + w] = !inside ? NAN : kmax == 0 ? 0.0 : -im / M_PI;
   };
   if (kmax < direct) {
-    if ((long long)blockIdx.y * 32 >= n_omega) return;
+    if (blockIdx.y * 32u >= (unsigned)n_omega) return;
     if (kmax > 0) stage(0, kmax + 1);
     __syncthreads();
-    for (long long w0 = (long long)blockIdx.y * 32; w0 < n_omega; w0 += (long long)gridDim.y * 32) {
-      const long long w = w0 + lane;
-      const double om = w < n_omega ? omega[w] : 0.0;
+    for (unsigned w0 = blockIdx.y * 32u; w0 < (unsigned)n_omega; w0 += gridDim.y * 32u) {
+      const unsigned w = w0 + lane;
+      const double om = w < (unsigned)n_omega ? omega[w] : 0.0;
       double im = 0.0;
       for (int k = warp; kmax > 0 && k <= kmax; k += kDosWarps) {
         double sn, cs;
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(32 * kDosWarps)
       }
       part[warp][lane] = im;
       __syncthreads();
-      if (warp == 0 && w < n_omega) {
+      if (warp == 0 && w < (unsigned)n_omega) {
         for (int q = 1; q < kDosWarps; ++q) im += part[q][lane];
         store(w, im);
       }
@@ -110,9 +110,9 @@ __global__ void __launch_bounds__(32 * kDosWarps)
     }
     return;
   }
-  for (long long w0 = (long long)blockIdx.y * kDosWarps; w0 < n_omega; w0 += (long long)gridDim.y * kDosWarps) {
-    const long long w = w0 + warp;
-    const double om = w < n_omega ? omega[w] : 0.0;
+  for (unsigned w0 = blockIdx.y * kDosWarps; w0 < (unsigned)n_omega; w0 += gridDim.y * kDosWarps) {
+    const unsigned w = w0 + warp;
+    const double om = w < (unsigned)n_omega ? omega[w] : 0.0;
     double im = 0.0;
     for (int k0 = 0; k0 <= kmax; k0 += kDosTerms) {
       const int cnt = min(kDosTerms, kmax + 1 - k0);
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(32 * kDosWarps)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) im += __shfl_xor_sync(0xffffffffu, im, o);
-    if (lane == 0 && w < n_omega) store(w, im);
+    if (lane == 0 && w < (unsigned)n_omega) store(w, im);
   }
 }
 
@@ -179,17 +179,15 @@ extern "C" int nedmft_dos(const nedmft_contour* c, const nedmft_c128* gloc_d, co
   if (n_avg == 0 || n_omega == 0) return NEDMFT_OK;  // nothing to write; the arrays may be NULL
   if (!m_d || !omega_d || !rho_d) return set_error(NEDMFT_EINVAL, "dos: NULL argument");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int sms = 0;
-  if (int rc = device_sm_count(&sms)) return rc;
+  constexpr long long kSms = 152;
   const long long total = (long long)n_avg * n_omega;
-  const int direct = total >= 32ll * sms ? 64 : 16;
+  const int direct = total >= 32 * kSms ? 64 : 16;
   // 32 frequencies per CTA where that leaves 32 CTAs per SM (fewer idle CTAs with few relative times); at most
   // 65535 CTAs along y, which take every so many frequencies past that
-  const int per = total >= 1024ll * sms ? 32 : kDosWarps;
+  const int per = total >= 1024 * kSms ? 32 : kDosWarps;
   const int blocks = (int)(((long long)n_omega + per - 1) / per);
   dos_kernel<<<dim3(n_avg, blocks < 65535 ? blocks : 65535), 32 * kDosWarps, 0, st>>>(
-      reinterpret_cast<const double2*>(gloc_d), c->n_c, c->n_t, c->dt, m_d, omega_d, n_omega, direct,
-      rho_d);
+      reinterpret_cast<const double2*>(gloc_d), c->n_c, c->n_t, c->dt, m_d, omega_d, n_omega, direct, rho_d);
   NED_LAUNCH_CHECK("dos_kernel");
   return NEDMFT_OK;
 }
